@@ -17,7 +17,7 @@ from paper_2607_24593_b200 import inputs
 
 H, D = 64, 128
 MODES = {"refine": pv.REFINE, "reuse": pv.REUSE}
-MASK_MAX = 1 << 26          # rows x keys up to which the mask is of booleans
+MASK_MAX = 1 << 30          # rows x keys up to which the mask is of booleans
 
 
 def _prefill(name, L, dtype, g, c, k, mode, row0=0, W=0):
@@ -289,9 +289,9 @@ def work(case):
 def tolerance(case):
     """Share of mask entries (words) of another correct implementation that differ: scores within the
     rounding of the sums around a cut-off trade places.  fp8, this library's default (ReLU values rounded
-    to bf16) against its fp32 head sums on the same inputs: one of the k keys in a third of the rows, 2.8e-4
-    of a boolean mask, 0.8e-3 .. 6.9e-3 of the words.  bf16 against the CUDA-core kernels: 0 .. 6e-8, and
-    1.7e-6 of the words."""
+    to bf16) against its fp32 head sums on the same inputs: a key or two of the k in a third of the rows, at
+    most 2.8e-4 of a boolean mask, 0.8e-3 .. 2.2e-3 of the words.  bf16 against the CUDA-core kernels: 0 ..
+    6e-8, and 1.7e-6 of the words."""
     n_keys = max(_lens(case)) if case["kind"] == "varlen" else case.get("L", case.get("hi"))
     if case["dtype"] == "bf16":
         return {"differ": 1e-5}
