@@ -178,8 +178,9 @@ int pivot_index_prefill_ex(const pivot_tensor* q, const float* w, const pivot_te
  *                cu_seqlens[n_req]).  With FP8 every request must start on a multiple of 4 rows
  *                (the key-scale rows are read in 16-byte units); empty requests are allowed.
  *   out_idx      [total rows, k]; positions are relative to the start of the row's own request.
- * Each request is indexed by the prefill path above, one after the other on `stream`, sharing
- * one workspace sized for the longest request (opts->workspace, else the registered one).
+ * Each request is indexed by the prefill path above on `stream`.  The workspace (opts->workspace, else
+ * the registered one) has to hold the longest request; requests that fit it together -- row and
+ * group counts added up, four rows more per request -- share one set of launches.
  * opts may be NULL; row_begin / row_end and the debug buffers are not available here.
  */
 int pivot_index_prefill_varlen(const pivot_tensor* q, const float* w, const pivot_tensor* kcache,

@@ -193,8 +193,13 @@ def pivot_index_prefill_varlen(q, w, kcache, cu_seqlens, H_I, d, g, c, k, mode, 
     tq, tk = _tensor(q, q_scale), _tensor(kcache, k_scale)
     assert w.dtype == torch.float32 and out_idx.dtype == torch.int32 and out_idx.numel() >= cu[-1] * k
     if workspace is None:
-        Lmax = max((b - a for a, b in zip(cu[:-1], cu[1:])), default=1)
-        ensure_workspace(max(Lmax, 1), (max(Lmax, 1) + g - 1) // g, c, k, q.device)
+        # room for the longest request, and for the batch up to 16384 groups: what fits shares its launches
+        Lmax = max(max((b - a for a, b in zip(cu[:-1], cu[1:])), default=1), 1)
+        rows, groups = Lmax + 4, (Lmax + g - 1) // g
+        both = [(b - a + 4, (b - a + g - 1) // g) for a, b in zip(cu[:-1], cu[1:]) if b > a]
+        rows = max(rows, min(sum(r for r, _ in both), 16384 * g + 4 * n_req))
+        groups = max(groups, min(sum(n for _, n in both), 16384 + n_req))
+        ensure_workspace(rows, groups, c, k, q.device)
     o = _opts(guard_len, pool, None, None, None, workspace, impl, None, W)
     arr = (C.c_int32 * (n_req + 1))(*cu)
     _check(lib.pivot_index_prefill_varlen(C.byref(tq), w.data_ptr(), C.byref(tk), arr, n_req, H_I, d, g, c, k, mode,

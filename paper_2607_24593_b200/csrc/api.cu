@@ -208,79 +208,94 @@ int resolve_ws(const pivot_opts* o, size_t need, void** ws) {
   return PIVOT_OK;
 }
 
-int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kc, int L, int g, int c,
-                int k, int mode, bool dense_only, int32_t* out_idx, cudaStream_t st,
-                const pivot_opts* o) {
-  const int nG = (L + g - 1) / g;
-  const size_t need = pivot_workspace_bytes(L, nG, c, k);
-  void* wsp = nullptr;
-  int rc = resolve_ws(o, need, &wsp);
-  if (rc) return rc;
-  Workspace ws = carve_workspace(wsp, L, nG, c, k);
+// Requests cu[0] .. cu[n] of a packed batch (host array; one request: {0, L}), each indexed on its own.
+// All of them go through one prepare, one scan and one re-score launch.
+int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kcache, const int32_t* cu, int n, int g,
+                int c, int k, int mode, bool dense_only, int32_t* out_idx, cudaStream_t st, const pivot_opts* o, void* wsp,
+                int ws_rows, int ws_groups) {
+  Workspace ws = carve_workspace(wsp, ws_rows, ws_groups, c, k);
   g_dev[cur_device()].last_status = ws.status;
-
-  int guard = (o && o->guard_len >= 0) ? o->guard_len : c;
-  int first_group = guard <= 1 ? 0 : (guard - 1 + g - 1) / g;
-  if (first_group > nG) first_group = nG;
-  if (dense_only) first_group = nG;
-  long long nd = (long long)first_group * g;      // rows below nd are scored densely
-  if (nd > L) nd = L;
-  // optional row range (chunked prefill): groups never straddle a chunk boundary
-  int r0 = 0, r1 = L;
-  if (o && (o->row_begin || o->row_end)) {
-    r0 = o->row_begin; r1 = o->row_end;
-    if (r0 < 0 || r1 <= r0 || r1 > L || r0 % g || (r1 % g && r1 != L)) return PIVOT_ERR_INVALID_ARG;
-  }
+  const int guard = (o && o->guard_len >= 0) ? o->guard_len : c;
   // local window (Appendix B): needs room in the candidate set and a scan of at least one key
   const int W = (o && !dense_only) ? o->W : 0;
   if (W < 0) return PIVOT_ERR_INVALID_ARG;
   if (W > 0 && (W + g - 1 >= c || guard < W + g || (o && o->impl == 1))) return PIVOT_ERR_INVALID_ARG;
-  const int g_begin = r0 / g, g_end = (r1 + g - 1) / g;
-  const int dense0 = r0 < nd ? r0 : (int)nd;
-  const int dense1 = r1 < nd ? r1 : (int)nd;
-  const int pg0 = g_begin > first_group ? g_begin : first_group;   // first proxy group of this call
+
+  const int tokens = cu[n];
   PrefillPlan p;
   p.q = q->data; p.w = w; p.qscale = q->scale;
-  p.kc = kc->data; p.kscale = kc->scale;
-  p.k_stride = key_stride(kc);
+  p.kc = kcache->data; p.kscale = kcache->scale;
+  p.k_stride = key_stride(kcache);
   if (p.k_stride && o && o->impl == 1) return PIVOT_ERR_UNSUPPORTED;
   p.proxy_q = ws.proxy_q; p.proxy_w = ws.proxy_w;
-  p.cand = (o && o->dbg_cand) ? o->dbg_cand + (size_t)pg0 * c : ws.cand;
+  p.g = g; p.c = c; p.k = k; p.mode = mode; p.dtype = q->dtype;
+  p.W = W;
+  p.pool = o ? o->pool : 0;
+  p.skip_trivial = !(o && o->impl == 1);      // (the cross-check kernels score every row)
+  p.status = ws.status;
+  int pg0 = 0, live = 0;
+  for (int i = 0; i < n; ++i) live += cu[i + 1] > cu[i];
+  for (int i = 0; i < n; ++i) {
+    const int L = cu[i + 1] - cu[i];
+    if (L == 0) continue;
+    const int nG = (L + g - 1) / g;
+    int first_group = guard <= 1 ? 0 : (guard - 1 + g - 1) / g;
+    if (first_group > nG || dense_only) first_group = nG;
+    long long nd = (long long)first_group * g;      // rows below nd are scored densely
+    if (nd > L) nd = L;
+    // optional row range (chunked prefill, one request): groups never straddle a chunk boundary
+    int r0 = 0, r1 = L;
+    if (o && (o->row_begin || o->row_end)) {
+      r0 = o->row_begin; r1 = o->row_end;
+      if (r0 < 0 || r1 <= r0 || r1 > L || r0 % g || (r1 % g && r1 != L)) return PIVOT_ERR_INVALID_ARG;
+    }
+    const int g_begin = r0 / g, g_end = (r1 + g - 1) / g;
+    const int dense0 = r0 < nd ? r0 : (int)nd;
+    const int dense1 = r1 < nd ? r1 : (int)nd;
+    pg0 = g_begin > first_group ? g_begin : first_group;   // first proxy group of this call
+    const int n_proxy = g_end > pg0 ? g_end - pg0 : 0;
+    const int rows = dense1 - dense0 + n_proxy;
+    p.req[p.n_req++] = PrefillReq{cu[i], L, dense0, dense1 - dense0, pg0, n_proxy, p.n_slots, p.n_proxy};
+    p.n_slots += live > 1 ? (rows + 3) / 4 * 4 : rows;
+    p.n_proxy += n_proxy;
+  }
+  p.cand = (o && o->dbg_cand) ? o->dbg_cand + (size_t)pg0 * c : ws.cand;          // (debug buffers: one request)
   p.cand_score = (o && o->dbg_cand_scores) ? o->dbg_cand_scores + (size_t)pg0 * c : nullptr;
   p.out = out_idx; p.out_score = o ? o->dbg_scores : nullptr;
-  p.L = L; p.g = g; p.c = c; p.k = k; p.mode = mode; p.dtype = q->dtype;
-  p.W = W;
-  p.dense_begin = dense0;
-  p.n_dense = dense1 - dense0;
-  p.first_group = pg0;
-  p.n_proxy = g_end > pg0 ? g_end - pg0 : 0;
 
-  if ((rc = check_cuda(cudaMemsetAsync(ws.status, 0, 2 * sizeof(int), st)))) return rc;
+  int rc;
   mark(0, st);
-  launch_proxy_build(q->data, q->scale, w, ws.proxy_q, ws.proxy_w, L, g, pg0, p.n_proxy,
-                     q->dtype, o ? o->pool : 0, st);
+  if ((rc = check_cuda(launch_prepare_prefill(p, ws.rows, ws.groups, st)))) return rc;
   mark(1, st);
-  launch_plan_prefill(p, ws.rows, ws.groups, st);
   mark(2, st);
   if (o && o->impl == 1) {
-    launch_scan_simt(ws.rows, p.n_dense + p.n_proxy, q->dtype, ws.scan, st);
+    launch_scan_simt(ws.rows, p.n_slots, q->dtype, ws.scan, st);
   } else {
-    ScanOperands op{kc->data, L, kc->scale, q->data, L, ws.proxy_q, p.n_proxy, q->dtype};
+    ScanOperands op{kcache->data, tokens, kcache->scale, q->data, tokens, ws.proxy_q, p.n_proxy, q->dtype};
     op.k_stride = p.k_stride;
-    if ((rc = check_cuda(launch_scan_tc(op, ws.rows, p.n_dense + p.n_proxy, 4, tc_scratch(ws), sm_count(), st,
-                                        o && o->impl == 2))))
+    if ((rc = check_cuda(launch_scan_tc(op, ws.rows, p.n_slots, 4, tc_scratch(ws), sm_count(), st, o && o->impl == 2, true))))
       return rc;
   }
   mark(3, st);
   if (mode == PIVOT_REFINE) {
     const int nd = p.n_proxy * group_chunks(g);
     if (o && o->impl == 1) launch_refine_simt(ws.groups, nd, q->dtype, ws.scan, st);
-    else if ((rc = check_cuda(launch_refine_tc(q->data, L, q->dtype, ws.groups, nd, tc_scratch(ws), sm_count(), st,
-                                               o && o->impl == 2, false, c))))
+    else if ((rc = check_cuda(launch_refine_tc(q->data, tokens, q->dtype, ws.groups, nd, tc_scratch(ws), sm_count(), st,
+                                               o && o->impl == 2, false, c, true))))
       return rc;
   }
   mark(4, st);
   return check_cuda(cudaGetLastError());
+}
+
+int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kc, int L, int g, int c,
+                int k, int mode, bool dense_only, int32_t* out_idx, cudaStream_t st,
+                const pivot_opts* o) {
+  const int nG = (L + g - 1) / g;
+  void* wsp = nullptr;
+  if (int rc = resolve_ws(o, pivot_workspace_bytes(L, nG, c, k), &wsp)) return rc;
+  const int32_t cu[2] = {0, L};
+  return run_prefill(q, w, kc, cu, 1, g, c, k, mode, dense_only, out_idx, st, o, wsp, L, nG);
 }
 
 }  // namespace
@@ -335,15 +350,38 @@ int pivot_index_prefill_varlen(const pivot_tensor* q, const float* w, const pivo
     if (cu_seqlens[i + 1] < cu_seqlens[i]) return PIVOT_ERR_INVALID_ARG;
     if (fp8 && (cu_seqlens[i] & 3)) return PIVOT_ERR_INVALID_ARG;
   }
+  if (opts && (opts->pool < 0 || opts->pool > 2 || opts->impl < 0 || opts->impl > 2)) return PIVOT_ERR_INVALID_ARG;
+  // As many consecutive requests per set of launches as the workspace and the planner take: short requests
+  // leave most of the GPU idle and pay every kernel's ramp and tail each (12 requests of 128 .. 5212 tokens
+  // one after the other: 930 us, together 530).  A workspace for the longest request is always enough.
   const size_t esz = fp8 ? 1 : 2;
-  for (int i = 0; i < n_req; ++i) {
-    const size_t r0 = (size_t)cu_seqlens[i];
-    const int L = cu_seqlens[i + 1] - cu_seqlens[i];
-    if (L == 0) continue;
-    const size_t krow = kcache->stride_row ? kcache->stride_row : (size_t)d * esz;
-    pivot_tensor tq{(const char*)q->data + r0 * H_I * d * esz, q->scale ? q->scale + r0 * H_I : nullptr, q->dtype, 0};
-    pivot_tensor tk{(const char*)kcache->data + r0 * krow, kcache->scale ? kcache->scale + r0 : nullptr, q->dtype, kcache->stride_row};
-    rc = pivot_index_prefill_ex(&tq, w + r0 * H_I, &tk, L, H_I, d, g, c, k, mode, out_idx + r0 * k, stream, opts);
+  const size_t krow = kcache->stride_row ? kcache->stride_row : (size_t)d * esz;
+  const size_t ws_have = opts && opts->workspace ? opts->workspace_bytes : g_dev[cur_device()].ws_bytes;
+  int32_t cu[kMaxPlanReqs + 1];
+  for (int i = 0; i < n_req;) {
+    const int r0 = cu_seqlens[i];
+    int n = 0, rows = 0, groups = 0;
+    cu[0] = 0;
+    while (i < n_req && n < kMaxPlanReqs) {
+      const int L = cu_seqlens[i + 1] - cu_seqlens[i];
+      const int more_rows = L > 0 ? L + 4 : 0, more_groups = (L + g - 1) / g;
+      if (groups > 0 && (pivot_workspace_bytes(rows + more_rows, groups + more_groups, c, k) > ws_have ||
+                         (opts && opts->impl == 1)))
+        break;
+      rows += more_rows;
+      groups += more_groups;
+      cu[++n] = cu_seqlens[++i] - r0;
+    }
+    if (groups == 0) continue;
+    int live = 0;
+    for (int j = 0; j < n; ++j) live += cu[j + 1] > cu[j];
+    if (live == 1) rows -= 4;                    // no padding then: what a call for that request alone needs
+    void* wsp = nullptr;
+    if ((rc = resolve_ws(opts, pivot_workspace_bytes(rows, groups, c, k), &wsp))) return rc;
+    pivot_tensor tq{(const char*)q->data + (size_t)r0 * H_I * d * esz, q->scale ? q->scale + (size_t)r0 * H_I : nullptr, q->dtype, 0};
+    pivot_tensor tk{(const char*)kcache->data + (size_t)r0 * krow, kcache->scale ? kcache->scale + r0 : nullptr, q->dtype, kcache->stride_row};
+    rc = run_prefill(&tq, w + (size_t)r0 * H_I, &tk, cu, n, g, c, k, mode, false, out_idx + (size_t)r0 * k, (cudaStream_t)stream,
+                     opts, wsp, rows, groups);
     if (rc) return rc;
   }
   return PIVOT_OK;

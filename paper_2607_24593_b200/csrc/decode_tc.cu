@@ -539,12 +539,10 @@ decode_prepare_kernel(DecodePlan p, RowDesc* rows, GroupDesc* plan_groups, uint3
     // ---- the sequence's proxy: one warp per unit of four (e4m3) or two (bf16) heads
     if (p.dtype == DT_FP8) {
       for (int u = wid; u < proxy_units_per_group<DT_FP8>(); u += 32)
-        proxy_build_unit<DT_FP8>(p.q, p.qscale, p.w, p.proxy_q, p.proxy_w, B * g, g, 0, B, pool,
-                                 (long long)b * proxy_units_per_group<DT_FP8>() + u, lane);
+        proxy_build_unit<DT_FP8>(p.q, p.qscale, p.w, p.proxy_q, p.proxy_w, b * g, g, b, u, pool, lane);
     } else {
       for (int u = wid; u < proxy_units_per_group<DT_BF16>(); u += 32)
-        proxy_build_unit<DT_BF16>(p.q, p.qscale, p.w, p.proxy_q, p.proxy_w, B * g, g, 0, B, pool,
-                                  (long long)b * proxy_units_per_group<DT_BF16>() + u, lane);
+        proxy_build_unit<DT_BF16>(p.q, p.qscale, p.w, p.proxy_q, p.proxy_w, b * g, g, b, u, pool, lane);
     }
   }
   if (mode != 1) return;

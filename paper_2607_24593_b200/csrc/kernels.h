@@ -58,20 +58,36 @@ struct EntryList {
   float* out_score;
 };
 
-// Geometry of a prefill-shaped call, shared by the planner kernels.
+// One request of a prefill-shaped call: where it lies in the packed tensors and which of its rows are indexed.
+struct PrefillReq {
+  int tok0;         // first token (query row = key row) of the request in the packed tensors
+  int L;            // its tokens
+  int dense_begin;  // first densely scored row of this call (positions are relative to the request)
+  int n_dense;      // rows dense_begin .. dense_begin+n_dense-1 are scored densely (guarded groups or dense control)
+  int first_group;  // first group taking the proxy path
+  int n_proxy;      // groups on the proxy path
+  int slot0;        // scan-row slots of the requests before it
+  int proxy0;       // proxies of the requests before it
+};
+constexpr int kMaxPlanReqs = 64;
+
+// Geometry of a prefill-shaped call (by value to the planner kernel).
 struct PrefillPlan {
   const void* q; const float* w; const float* qscale;   // raw per-query operands
   const void* kc; const float* kscale;                  // key cache
   int k_stride = 0;                                     // bytes between key rows (0: dense)
   void* proxy_q; float* proxy_w;                        // [nP, H, d], [nP, H]
   int32_t* cand; float* cand_score;                     // [nP, c] (Refine)
-  int32_t* out; float* out_score;                       // [L, k]
-  int L, g, c, k, mode, dtype;
-  int W;            // local window (Appendix B); 0 = off
-  int dense_begin;  // first densely scored row of this call
-  int n_dense;      // rows dense_begin .. dense_begin+n_dense-1 are scored densely (guarded groups or dense control)
-  int first_group;  // first group taking the proxy path
-  int n_proxy;      // groups on the proxy path
+  int32_t* out; float* out_score;                       // [tokens, k]
+  int g, c, k, mode, dtype;
+  int pool = 0;
+  int W = 0;            // local window (Appendix B); 0 = off
+  bool skip_trivial = true;   // rows that select all they see are written by the planner instead of scanned
+  int* status = nullptr;      // status word and row counter: cleared by the planner
+  int n_slots = 0;      // scan-row slots: the rows of all requests, each request padded to whole blocks of four if there are several
+  int n_proxy = 0;      // proxies of all requests
+  int n_req = 0;
+  PrefillReq req[kMaxPlanReqs];
 };
 
 struct DecodePlan {
@@ -111,7 +127,8 @@ struct ScanScratch {
 void launch_proxy_build(const void* q, const float* qscale, const float* w, void* proxy_q,
                         float* proxy_w, int rows, int g, int first_group, int n_proxy, int dtype,
                         int pool, cudaStream_t st);
-void launch_plan_prefill(const PrefillPlan& p, RowDesc* rows, GroupDesc* groups, cudaStream_t st);
+// One kernel prepares a prefill call: proxies (Eq. 4), row and group descriptors, rows without a choice.
+cudaError_t launch_prepare_prefill(const PrefillPlan& p, RowDesc* rows, GroupDesc* groups, cudaStream_t st);
 void launch_plan_decode(const DecodePlan& p, RowDesc* rows, GroupDesc* groups, cudaStream_t st);
 // Decode proxies need the guard test on device (pos0 lives there): rows of guarded sequences
 // get K = 0 and are skipped.
@@ -130,10 +147,9 @@ struct ScanOperands {
 // rows_per_block consecutive scan rows share one key stream (4 in prefill, 1 in decode).
 // fp32_head_sum: keep the gate-weighted head sum in fp32 FMAs even where the tensor-core form
 // (FP8, four rows per block) is available.
-// fp32_head_sum: keep the gate-weighted head sum in fp32 FMAs even where the tensor-core form
-// (FP8, four rows per block) is available.
 cudaError_t launch_scan_tc(const ScanOperands& op, const RowDesc* rows, int n_rows, int rows_per_block,
-                           const ScanScratch& s, int sms, cudaStream_t st, bool fp32_head_sum = false);
+                           const ScanScratch& s, int sms, cudaStream_t st, bool fp32_head_sum = false,
+                           bool overlap_prev = false);
 
 cudaError_t launch_refine_tc(const void* q, int q_rows, int dtype, const GroupDesc* groups, int n_groups,
                              const ScanScratch& s, int sms, cudaStream_t st, bool fp32_head_sum = false,

@@ -1,4 +1,5 @@
-// Kernel 1: proxy-query build (Eq. 4) and the row / group planners.
+// Kernel 1 on its own: proxy-query build (Eq. 4) for the CUDA-core decode path (the other paths form their
+// proxies inside their prepare kernels).
 //
 // A warp forms the proxy vectors of four (e4m3) or two (bf16) heads of a group: members are de-quantised, summed in member
 // order in fp32, scaled by fl32(1/m) and rounded once to the storage type.  For FP8 the proxy
@@ -21,7 +22,11 @@ proxy_build_kernel(const void* __restrict__ q, const float* __restrict__ qscale,
                    const float* __restrict__ w, void* __restrict__ proxy_q,
                    float* __restrict__ proxy_w, int rows, int g, int first_group, int n_proxy, int pool) {
   const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  proxy_build_unit<DT>(q, qscale, w, proxy_q, proxy_w, rows, g, first_group, n_proxy, pool, wid, threadIdx.x & 31);
+  constexpr int WPG = proxy_units_per_group<DT>();
+  const int r = (int)(wid / WPG);
+  if (r >= n_proxy) return;
+  const int t0 = (first_group + r) * g;
+  proxy_build_unit<DT>(q, qscale, w, proxy_q, proxy_w, t0, min(g, rows - t0), r, (int)(wid % WPG), pool, threadIdx.x & 31);
 }
 
 void launch_proxy_build(const void* q, const float* qscale, const float* w, void* proxy_q,

@@ -15,23 +15,17 @@ constexpr int proxy_units_per_group() { return kHeads / (32 / (kDim / (DT == DT_
 // (bf16: 16 lanes x 8 values), and the members' loads go out four at a time -- with 4-byte
 // loads issued one member after the other the kernel had too few bytes in flight to get near
 // the HBM rate (it reads every query once: 1.07 GB at the 128K FP8 configuration).
-// `wid` numbers the warp-sized units of work: unit wid forms heads (wid % WPG) * HPW .. of proxy wid / WPG.
+// Unit `u` of a group forms heads u * HPW .. of proxy r from the members at query rows t0 .. t0 + m - 1.
 template <int DT>
 __device__ __forceinline__ void proxy_build_unit(const void* __restrict__ q, const float* __restrict__ qscale,
                                                  const float* __restrict__ w, void* __restrict__ proxy_q,
-                                                 float* __restrict__ proxy_w, int rows, int g, int first_group, int n_proxy,
-                                                 int pool, long long wid, int lane) {
+                                                 float* __restrict__ proxy_w, int t0, int m, int r, int u, int pool, int lane) {
   constexpr bool FP8 = DT == DT_FP8;
   constexpr int E = FP8 ? 16 : 8;            // elements per lane
   constexpr int LPH = kDim / E;              // lanes per head: 8 or 16
   constexpr int HPW = 32 / LPH;              // heads per warp: 4 or 2
-  constexpr int WPG = kHeads / HPW;          // warps per group
-  if (wid >= (long long)n_proxy * WPG) return;
-  const int r = (int)(wid / WPG);
-  const int h = (int)(wid % WPG) * HPW + lane / LPH;
+  const int h = u * HPW + lane / LPH;
   const int sub = lane % LPH;                // which 16 bytes of the head's row
-  const int t0 = (first_group + r) * g;
-  const int m = min(g, rows - t0);
   int lo = 0, hi = m;                        // members pooled
   if (pool == 1) hi = 1;
   if (pool == 2) lo = m - 1;
@@ -42,39 +36,39 @@ __device__ __forceinline__ void proxy_build_unit(const void* __restrict__ q, con
     uint4 pk[4];
     float sc[4], wv[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {            // up to four members in flight
-      if (i0 + u < hi) {
-        const size_t row = (size_t)(t0 + i0 + u) * kHeads + h;
-        pk[u] = __ldg(q4 + row * LPH + sub);
-        sc[u] = FP8 ? __ldg(qscale + row) : 1.f;
-        wv[u] = __ldg(w + row);
+    for (int j = 0; j < 4; ++j) {            // up to four members in flight
+      if (i0 + j < hi) {
+        const size_t row = (size_t)(t0 + i0 + j) * kHeads + h;
+        pk[j] = __ldg(q4 + row * LPH + sub);
+        sc[j] = FP8 ? __ldg(qscale + row) : 1.f;
+        wv[j] = __ldg(w + row);
       }
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (i0 + u < hi) {
-        const uint32_t wd[4] = {pk[u].x, pk[u].y, pk[u].z, pk[u].w};
+    for (int j = 0; j < 4; ++j) {
+      if (i0 + j < hi) {
+        const uint32_t wd[4] = {pk[j].x, pk[j].y, pk[j].z, pk[j].w};
         float x[E];
         if (FP8) {                           // two codes per conversion (e4m3 -> half is exact, and so is half -> float)
 #pragma unroll
           for (int e = 0; e < E; e += 2) {
             const __half2_raw h2 = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)((wd[e >> 2] >> (8 * (e & 3))) & 0xffff), __NV_E4M3);
             const float2 f2 = __half22float2(__half2(h2));
-            x[e] = __fmul_rn(f2.x, sc[u]);
-            x[e + 1] = __fmul_rn(f2.y, sc[u]);
+            x[e] = __fmul_rn(f2.x, sc[j]);
+            x[e + 1] = __fmul_rn(f2.y, sc[j]);
           }
         } else {
 #pragma unroll
           for (int e = 0; e < E; ++e) x[e] = bf16_bits_to_float((wd[e >> 1] >> (16 * (e & 1))) & 0xffff);
         }
-        if (i0 + u == lo) {
+        if (i0 + j == lo) {
 #pragma unroll
           for (int e = 0; e < E; ++e) acc[e] = x[e];
-          wacc = wv[u];
+          wacc = wv[j];
         } else {
 #pragma unroll
           for (int e = 0; e < E; ++e) acc[e] = __fadd_rn(acc[e], x[e]);
-          wacc = __fadd_rn(wacc, wv[u]);
+          wacc = __fadd_rn(wacc, wv[j]);
         }
       }
     }

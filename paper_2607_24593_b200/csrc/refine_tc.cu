@@ -709,12 +709,12 @@ cudaError_t launch_refine_tc(const void* q, int q_rows, int dtype, const GroupDe
   // the select warps need the caller's score-row buffers, long enough for every group
   const bool rows_ok = s.rkeys && max_cand > 0 && max_cand <= s.rslots;
   if (dtype != DT_FP8)
-    return rows_ok && !chunked ? launch_one<DT_BF16, 3>(mq, groups, n_groups, q_rows, s, sms, st)
-                               : launch_one<DT_BF16>(mq, groups, n_groups, q_rows, s, sms, st);
-  if (fp32_head_sum) return launch_one<DT_FP8, 0>(mq, groups, n_groups, q_rows, s, sms, st);
+    return rows_ok && !chunked ? launch_one<DT_BF16, 3>(mq, groups, n_groups, q_rows, s, sms, st, overlap_prev)
+                               : launch_one<DT_BF16>(mq, groups, n_groups, q_rows, s, sms, st, overlap_prev);
+  if (fp32_head_sum) return launch_one<DT_FP8, 0>(mq, groups, n_groups, q_rows, s, sms, st, overlap_prev);
   if (chunked) return launch_one<DT_FP8, 2>(mq, groups, n_groups, q_rows, s, sms, st, overlap_prev);
   if (!rows_ok) return cudaErrorInvalidValue;
-  return launch_one<DT_FP8, 3>(mq, groups, n_groups, q_rows, s, sms, st);
+  return launch_one<DT_FP8, 3>(mq, groups, n_groups, q_rows, s, sms, st, overlap_prev);
 }
 
 }  // namespace pivot

@@ -130,9 +130,13 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
   const int lane = threadIdx.x & 31;
   const int n_blocks = (n_rows + NROWS - 1) / NROWS;
 
+  // (a prefill launches this kernel so that its set-up overlaps the prepare kernel, and the re-score so
+  // that its own overlaps this one's last blocks)
+  ptx::grid_launch_dependents();
   // A small launch whose rows are all dead (decode: no guarded sequence in the batch) leaves
   // before any barrier or TMEM is set up.
   if (n_rows <= (int)blockDim.x) {
+    ptx::grid_dependency_wait();
     const bool live = (int)threadIdx.x < n_rows && rows[threadIdx.x].K > 0 && rows[threadIdx.x].n_vis > 0;
     if (!__syncthreads_or(live)) return;
   }
@@ -171,6 +175,7 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = ct.tmem_base;
+  ptx::grid_dependency_wait();            // the row descriptors and the proxies
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -543,7 +548,7 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
 
 template <int DT, int NROWS, int EPI = 1>
 cudaError_t launch_one(const CUtensorMap& mk, const CUtensorMap& mq0, const CUtensorMap& mq1, const CUtensorMap& mks,
-                       const RowDesc* rows, int n_rows, const ScanScratch& s, int sms, cudaStream_t st) {
+                       const RowDesc* rows, int n_rows, const ScanScratch& s, int sms, cudaStream_t st, bool overlap_prev = false) {
   using C = Cfg<DT, NROWS, EPI>;
   auto kern = scan_select_tc_kernel<DT, NROWS, EPI>;
   static bool attr_set[kMaxDevices] = {};
@@ -551,9 +556,8 @@ cudaError_t launch_one(const CUtensorMap& mk, const CUtensorMap& mq0, const CUte
   if (cudaError_t e = opt_in_dynamic_smem(kern, smem, attr_set); e != cudaSuccess) return e;
   const int n_blocks = (n_rows + NROWS - 1) / NROWS;
   const int grid = n_blocks < sms ? n_blocks : sms;
-  kern<<<grid, C::THREADS, smem, st>>>(mk, mq0, mq1, mks, rows, n_rows, s);
   ++launch_counter();
-  return cudaGetLastError();
+  return launch_kernel(kern, dim3(grid), dim3(C::THREADS), smem, st, overlap_prev, mk, mq0, mq1, mks, rows, n_rows, s);
 }
 
 }  // namespace
@@ -605,7 +609,7 @@ bool make_scale_map(CUtensorMap* m, const float* base, long long n, int box) {
 
 
 cudaError_t launch_scan_tc(const ScanOperands& op, const RowDesc* rows, int n_rows, int rows_per_block,
-                           const ScanScratch& s, int sms, cudaStream_t st, bool fp32_head_sum) {
+                           const ScanScratch& s, int sms, cudaStream_t st, bool fp32_head_sum, bool overlap_prev) {
   if (n_rows <= 0) return cudaSuccess;
   CUtensorMap mk, mq0, mq1, mks;
   memset(&mks, 0, sizeof(mks));
@@ -616,10 +620,10 @@ cudaError_t launch_scan_tc(const ScanOperands& op, const RowDesc* rows, int n_ro
     return cudaErrorInvalidValue;
   if (op.dtype == DT_FP8) {
     if (rows_per_block != 4) return launch_one<DT_FP8, 1>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st);
-    return fp32_head_sum ? launch_one<DT_FP8, 4, 0>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st)
-                         : launch_one<DT_FP8, 4, 1>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st);
+    return fp32_head_sum ? launch_one<DT_FP8, 4, 0>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev)
+                         : launch_one<DT_FP8, 4, 1>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev);
   }
-  return rows_per_block == 4 ? launch_one<DT_BF16, 4>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st)
+  return rows_per_block == 4 ? launch_one<DT_BF16, 4>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev)
                              : launch_one<DT_BF16, 1>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st);
 }
 

@@ -59,18 +59,18 @@ extern "C" int dense_index_static(const pivot_tensor* q, const float* w, const p
   off += (size_t)kStaticCtas * 4 * 2 * kStaticCap * sizeof(unsigned long long);   // two segments per row
   if (off > kStaticBytes) return PIVOT_ERR_WORKSPACE;
 
-  // The array keeps whatever the previous call left: the status word must start at zero; row
+  // The array keeps whatever the previous call left: the planner clears the status word, row
   // descriptors are rewritten for rows 0..L-1 and candidate cursors start at zero in registers.
-  if (int rc = record_cuda(cudaMemsetAsync(status, 0, 2 * sizeof(int), st))) return rc;
-
   PrefillPlan p;
   p.q = q->data; p.w = w; p.qscale = q->scale;
   p.kc = kcache->data; p.kscale = kcache->scale;
   p.proxy_q = nullptr; p.proxy_w = nullptr; p.cand = nullptr; p.cand_score = nullptr;
   p.out = out_idx; p.out_score = nullptr;
-  p.L = L; p.g = 1; p.c = k; p.k = k; p.mode = 0; p.dtype = q->dtype;
-  p.W = 0; p.dense_begin = 0; p.n_dense = L; p.first_group = L; p.n_proxy = 0;
-  launch_plan_prefill(p, rows, nullptr, st);
+  p.g = 1; p.c = k; p.k = k; p.mode = 0; p.dtype = q->dtype;
+  p.status = status;
+  p.n_slots = L; p.n_req = 1;
+  p.req[0] = PrefillReq{0, L, 0, L, L, 0, 0, 0};
+  if (int rc = record_cuda(launch_prepare_prefill(p, rows, nullptr, st))) return rc;
 
   ScanScratch sc;
   sc.cand_key = nullptr; sc.cand_idx = nullptr;

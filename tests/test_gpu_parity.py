@@ -890,3 +890,37 @@ def test_prefill_varlen_equals_per_request_calls(pv, gu, dtype):
             pv.pivot_index_prefill_varlen(q, w, kk, [0, 702, int(cu[-1])], 64, 128, g, c, k, mode, packed, **sc)
     with pytest.raises(pv.PivotError, match="invalid"):
         pv.pivot_index_prefill_varlen(q, w, kk, [0, 800, 400], 64, 128, g, c, k, mode, packed, **sc)
+
+
+@pytest.mark.parametrize("g,mode,W,guard", [(1, 1, 0, None), (4, 1, 4, None), (8, 0, 0, 0), (16, 1, 0, 40)])
+def test_prefill_varlen_batches(pv, gu, g, mode, W, guard):
+    """A batch beyond the planner's 64 requests, requests from one token up (blocks of one live row, whole
+    requests without a choice), against separate calls; once more with a workspace that only holds the
+    longest request."""
+    lens = ([1, 2, 3, 5, 700, 63, 64, 65, 129, 257, 0, 31] * 6)[:70]
+    lens = [(n + 3) // 4 * 4 if i + 1 < len(lens) else n for i, n in enumerate(lens)]      # FP8: starts at multiples of 4
+    lens[5] = 0
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(int)
+    c, k = 128, 96
+    x = inputs.make_prefill(int(cu[-1]), dtype="fp8", seed=55)
+    q, w, kk, qs, ks = x.q.cuda(), x.w.cuda(), x.k.cuda(), x.qscale.cuda(), x.kscale.cuda()
+    kw = dict(W=W, guard_len=guard)
+    n = max(lens)
+    ws = torch.empty(pv.pivot_workspace_bytes(n, (n + g - 1) // g, c, k), dtype=torch.uint8, device="cuda")
+    packed = []
+    for workspace in (None, ws):
+        out = torch.full((int(cu[-1]), k), -7, dtype=torch.int32, device="cuda")
+        pv.pivot_index_prefill_varlen(q, w, kk, cu, 64, 128, g, c, k, mode, out, q_scale=qs, k_scale=ks, workspace=workspace, **kw)
+        torch.cuda.synchronize()
+        assert pv.pivot_device_status() == 0
+        packed.append(_sorted_rows(out.cpu().numpy()))
+    one = torch.full((int(cu[-1]), k), -7, dtype=torch.int32, device="cuda")
+    for a, b in zip(cu[:-1], cu[1:]):
+        if b > a:
+            pv.pivot_index_prefill(q[a:b], w[a:b], kk[a:b], int(b - a), 64, 128, g, c, k, mode, one[a:b], q_scale=qs[a:b],
+                                   k_scale=ks[a:b], **kw)
+    one = _sorted_rows(one.cpu().numpy())
+    assert np.array_equal(packed[0], one) and np.array_equal(packed[1], one)
+    if guard is None:                     # rows below the guardrail that see no more keys than they select
+        for t in range(k):
+            assert np.array_equal(one[cu[4] + t][k - t - 1:], np.arange(t + 1))
