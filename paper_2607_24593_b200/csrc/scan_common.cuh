@@ -16,11 +16,7 @@ constexpr int KS_SLOTS = 8;       // key-scale ring: deeper than (key stages + a
 #ifndef PIVOT_CHK
 #define PIVOT_CHK 32
 #endif
-constexpr int kThresholdRefreshTiles = PIVOT_CHK;
-#ifndef PIVOT_COMPACT_EVERY
-#define PIVOT_COMPACT_EVERY 0
-#endif
-constexpr int kCompactEveryTiles = PIVOT_COMPACT_EVERY;   // a multiple of the refresh interval, or 0 = never   // the append warp re-reads its row's threshold off the histogram this often
+constexpr int kThresholdRefreshTiles = PIVOT_CHK;   // the append warp re-reads its row's threshold off the histogram this often
 
 // Block sequence of one CTA: blocks sorted longest-first are dealt in snake order.
 struct BlockIter {
@@ -106,6 +102,13 @@ __device__ __forceinline__ int select_bin(uint32_t key, int base) {
   return b < 0 ? 0 : (b > kSelBins - 1 ? kSelBins - 1 : b);
 }
 
+// Smallest key of a bin: the end bins take everything beyond them (key 0 stands for "no entry").
+// (bins the boundary asks for lie above 0 and at most at kSelBins, so the top bin's end is the largest key)
+__device__ __forceinline__ uint32_t select_bin_lo(int bin, int base) {
+  if (bin <= 0) return 1u;
+  return bin >= kSelBins || bin + base > 0x1ffff ? 0xffffffffu : (uint32_t)(bin + base) << 15;
+}
+
 // The append warp of row r (one warp, all blocks of this CTA): counts the survivors of every tile
 // in the row histogram, moves them to the row's segment in the L2-resident scratch and keeps the
 // row's threshold fresh -- alone, without barriers.  At the end of a block it reads the boundary
@@ -149,65 +152,83 @@ __device__ __noinline__ void append_role(SelectCtrl<NROWS, QD>& s, int r, int la
     entry_t* const seg = row_segment<NROWS>(sc, r, seq);
     bool sel_mine = seq == 0;                    // the finisher of the previous block may still use `sel`
     __syncwarp();
+    int due = CHK;                               // tiles until the next refresh
     for (int t = 0; t < ntiles; ++t, ++it) {
-      if (K > 0 && t > 0 && (t % CHK) == 0) {
-        const uint32_t th = hist_threshold(K, base);
-        thr = th > thr ? th : thr;
-        // Housekeeping while this warp has slack: every kCompactEveryTiles tiles the entries that fell
-        // below the threshold leave the segment, so that the final selection at the end of the block
-        // (which stalls the whole pipeline) reads a segment of about K entries instead of
-        // K (1 + ln(n / K)).  They lie below every bin the final boundary can be in, so the histogram
-        // stays exact for what the selection looks at.
-        const bool tidy = kCompactEveryTiles > 0 && (t % kCompactEveryTiles) == 0 && cnt > K + K / 2;
-        if (cnt + headroom > CAP || tidy) {
-          // (nearly full: the same filter; if that is not enough -- ties, adversarial order -- compact
-          // exactly to the K best)
-          const uint32_t tcur = thr;
-          cnt = seg_filter_inplace(seg, cnt, lane, [tcur](entry_t x) { return entry_key(x) > tcur; });
-          if (cnt + headroom > CAP && cnt > K) {
-            if (!sel_mine) {                     // (rare path: waiting here costs nothing that matters)
-              (void)ptx::mbar_wait(&s.fin_done[r][fb ^ 1], ((seq - 1) >> 1) & 1, abort_flag, 64);
-              sel_mine = true;
+      if (due-- == 0) {
+        due = CHK - 1;
+        if (K > 0) {
+          const uint32_t th = hist_threshold(K, base);
+          thr = th > thr ? th : thr;
+          if (cnt + headroom > CAP) {
+            // Nearly full: drop what fell below the threshold; if that is not enough (ties, adversarial
+            // order) compact exactly to the K best.  What goes lies below every bin the final boundary can
+            // be in, so the histogram stays exact for what the selection looks at.
+            const uint32_t tcur = thr;
+            cnt = seg_filter_inplace(seg, cnt, lane, [tcur](entry_t x) { return entry_key(x) > tcur; });
+            if (cnt + headroom > CAP && cnt > K) {
+              if (!sel_mine) {                     // (rare path: waiting here costs nothing that matters)
+                (void)ptx::mbar_wait(&s.fin_done[r][fb ^ 1], ((seq - 1) >> 1) & 1, abort_flag, 64);
+                sel_mine = true;
+              }
+              entry_t cut;
+              cnt = seg_compact<false>(tm, sel, Seg{seg, cnt}, K, &cut);
+              thr = entry_key(cut) > thr ? entry_key(cut) : thr;
             }
-            entry_t cut;
-            cnt = seg_compact<false>(tm, sel, Seg{seg, cnt}, K, &cut);
-            thr = entry_key(cut) > thr ? entry_key(cut) : thr;
           }
+          if (lane == 0) s.thr[r] = ((unsigned long long)seq << 32) | thr;
         }
-        if (lane == 0) s.thr[r] = ((unsigned long long)seq << 32) | thr;
       }
       const int sb = it % QD;
       (void)ptx::mbar_wait(&s.sc_full[sb], (it / QD) & 1, abort_flag);
       const uint4 n4 = *reinterpret_cast<const uint4*>(&s.qn[sb][r][0]);
-      const uint32_t nq[4] = {n4.x, n4.y, n4.z, n4.w};
-      entry_t e[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) e[j] = (uint32_t)lane < nq[j] ? s.q[sb][r][j][lane] : kPadEntry;
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(&s.sc_empty[sb]);
-      if (K <= 0) continue;                    // a dead row still takes part in the handshake
-      if (t == 0) {          // anchor the histogram range on the first tile's maximum
-        uint32_t mx = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) mx = entry_key(e[j]) > mx ? entry_key(e[j]) : mx;
-        mx = __reduce_max_sync(0xffffffffu, mx);
-        const int top = (int)(mx >> 15) + 512 - (kSelBins - 1);
-        base = top > 0 ? top : 0;
-      }
+      const uint32_t total = n4.x + n4.y + n4.z + n4.w;
       // Every entry that reaches the segment is counted: the ones the score warps dropped were
       // at or below a valid threshold and can never reach a bin edge the threshold could still
       // move to, so the counts that matter stay exact.
-      int p = cnt + lane;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if ((uint32_t)lane < nq[j]) {
-          atomicAdd(&rhist[select_bin(entry_key(e[j]), base)], 1u);
-          if (p < CAP) seg[p] = e[j];
+      auto take = [&](entry_t x, bool on, int p) {
+        hist_add_if(rhist, (uint32_t)select_bin(entry_key(x), base), on);
+        if (on) {
+          if (p < CAP) seg[p] = x;
           else s.abort_code = DEV_CAND_OVERFLOW;
         }
-        p += (int)nq[j];
+      };
+      if (t > 0 && total <= 32) {
+        // All of the tile's survivors in one step, a lane each: once the threshold has settled a tile
+        // leaves some twenty, and the step's cost is its instruction count, not the entries.
+        const uint32_t c1 = n4.x, c2 = c1 + n4.y, c3 = c2 + n4.z;
+        const uint32_t l = (uint32_t)lane;
+        const uint32_t j = (l >= c1 ? 1u : 0u) + (l >= c2 ? 1u : 0u) + (l >= c3 ? 1u : 0u);
+        const uint32_t first = l >= c3 ? c3 : l >= c2 ? c2 : l >= c1 ? c1 : 0u;
+        const bool on = l < total;
+        const entry_t x = on ? s.q[sb][r][j][l - first] : kPadEntry;
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&s.sc_empty[sb]);
+        if (K <= 0) continue;                    // a dead row still takes part in the handshake
+        take(x, on, cnt + lane);
+      } else {
+        const uint32_t nq[4] = {n4.x, n4.y, n4.z, n4.w};
+        entry_t e[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) e[j] = (uint32_t)lane < nq[j] ? s.q[sb][r][j][lane] : kPadEntry;
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&s.sc_empty[sb]);
+        if (K <= 0) continue;
+        if (t == 0) {          // anchor the histogram range on the first tile's maximum
+          uint32_t mx = 0;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) mx = entry_key(e[j]) > mx ? entry_key(e[j]) : mx;
+          mx = __reduce_max_sync(0xffffffffu, mx);
+          const int top = (int)(mx >> 15) + 512 - (kSelBins - 1);
+          base = top > 0 ? top : 0;
+        }
+        int p = cnt + lane;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          take(e[j], (uint32_t)lane < nq[j], p);
+          p += (int)nq[j];
+        }
       }
-      cnt = min(cnt + (int)(nq[0] + nq[1] + nq[2] + nq[3]), CAP);
+      cnt = min(cnt + (int)total, CAP);
     }
     // ---- end of the block: the histogram is exact for everything the segment still holds; read
     //      the boundary bin off it and hand the row to its finisher
@@ -247,19 +268,31 @@ __device__ __noinline__ void finisher_role(SelectCtrl<NROWS, QD>& s, int r0, int
         const RowDesc rd = rows[ri];
         const typename SelectCtrl<NROWS, QD>::FinRow f = s.fin[r][fb];
         const int rbase = f.base;
-        auto key_bin = [rbase](uint32_t key) { return select_bin(key, rbase); };
-        const int n_valid = warp_seg_topk_binned(s.sel[r], row_segment<NROWS>(sc, r, seq), f.cnt, key_bin, f.bsel,
+        auto bin_lo = [rbase](int bin) { return select_bin_lo(bin, rbase); };
+        const int n_valid = warp_seg_topk_binned(s.sel[r], row_segment<NROWS>(sc, r, seq), f.cnt, bin_lo, f.bsel,
                                                  f.need_b, f.pop, rd.out, rd.out_score, K, lane);
         for (int i = n_valid + lane; i < K; i += 32) {
           rd.out[i] = -1;
           if (rd.out_score) rd.out_score[i] = -INFINITY;
         }
         __syncwarp();
-        for (int rr = 1; rr < rd.out_rows; ++rr)
-          for (int i = lane; i < K; i += 32) {
-            rd.out[(size_t)rr * rd.out_stride + i] = rd.out[i];
-            if (rd.out_score) rd.out_score[(size_t)rr * rd.out_stride + i] = rd.out_score[i];
+        if (rd.out_rows > 1) {
+          constexpr int U = 16;               // one load for all copies, sixteen in flight
+          for (int i0 = 0; i0 < K; i0 += 32 * U) {
+            int32_t v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) v[u] = i0 + u * 32 + lane < K ? rd.out[i0 + u * 32 + lane] : 0;
+            for (int rr = 1; rr < rd.out_rows; ++rr) {
+              int32_t* const o = rd.out + (size_t)rr * rd.out_stride + i0 + lane;
+#pragma unroll
+              for (int u = 0; u < U; ++u)
+                if (i0 + u * 32 + lane < K) o[u * 32] = v[u];
+            }
           }
+          if (rd.out_score)
+            for (int rr = 1; rr < rd.out_rows; ++rr)
+              for (int i = lane; i < K; i += 32) rd.out_score[(size_t)rr * rd.out_stride + i] = rd.out_score[i];
+        }
       }
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&s.fin_done[r][fb]);

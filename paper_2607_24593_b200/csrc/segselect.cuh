@@ -389,6 +389,18 @@ struct KeyRowSrc {
   int nslots;
   const int32_t* __restrict__ cand;
   int n_cand;
+  __device__ __forceinline__ int slots() const { return nslots; }
+  // U slots per lane from slot i0 on (key 0: empty)
+  template <int U>
+  __device__ __forceinline__ void load(int i0, int lane, uint32_t (&k)[U], int32_t (&ps)[U]) const {
+    const uint32_t* kp = keys + i0 + lane;
+    const int32_t* cp = cand + i0 + lane;
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      k[j] = i0 + j * 32 < nslots ? __ldcg(kp + j * 32) : 0u;
+      ps[j] = i0 + j * 32 + lane < n_cand ? __ldg(cp + j * 32) : -1;
+    }
+  }
   template <int U, typename F>
   __device__ __forceinline__ void sweep_keys(int lane, F f) const {
     for (int s0 = 0; s0 < nslots; s0 += 32 * U) {
@@ -424,6 +436,17 @@ struct SegSrc {
   static constexpr bool kKeysApart = false;
   const entry_t* e;
   int cnt;
+  __device__ __forceinline__ int slots() const { return cnt; }
+  template <int U>
+  __device__ __forceinline__ void load(int i0, int lane, uint32_t (&k)[U], int32_t (&ps)[U]) const {
+    const entry_t* p = e + i0 + lane;
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const entry_t x = i0 + j * 32 + lane < cnt ? __ldcg(p + j * 32) : kPadEntry;
+      ps[j] = entry_pos(x);
+      k[j] = ps[j] >= 0 ? entry_key(x) : 0u;
+    }
+  }
   template <int U, bool NEED_POS, typename F>
   __device__ __forceinline__ void sweep(int lane, F f) const {
     for (int i0 = 0; i0 < cnt; i0 += 32 * U) {
@@ -439,11 +462,95 @@ struct SegSrc {
   }
 };
 
+// hist[bin] += 1 where `on`, as one predicated reduction (a branch around it would end the basic block).
+__device__ __forceinline__ void hist_add_if(uint32_t* hist, uint32_t bin, bool on) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(hist) + bin * 4u;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p red.shared.add.u32 [%0], 1;\n\t}" ::"r"(a), "r"((uint32_t)on) : "memory");
+}
+
+// The sweep that writes a selection whose boundary is a range of keys: entries with key > khi go out, those
+// among the n_keys keys up to khi are listed (at most kSelSmall) and counted in *n_list.  Returns how many went out.
+//
+// What a sweep by one warp costs is its instruction count -- beside the other warps of the CTA each takes
+// about ten clocks: one vote and two population counts per 32 entries, 32-bit compares, and the few entries
+// of the boundary marked in a bit mask on the side (about 14 instructions against 30 with 64-bit compares,
+// two votes and four population counts).  Entries leave in the order they lie in, which is
+// nearly that of their positions: the caller's next step, a gather or scatter over the row, runs over
+// neighbouring addresses (lane-wise runs saved another two instructions here and cost that step a quarter).
+template <int U, typename Src>
+__device__ __forceinline__ int warp_emit_keys(SegSelSmem& sm, const Src& src, uint32_t khi, uint32_t n_keys, uint32_t* n_list,
+                                              int32_t* __restrict__ out, int K, int lane) {
+  const uint32_t lt = (1u << lane) - 1u;
+  const uint32_t klo = khi - n_keys + 1u;
+  uint32_t base = 0, ln = 0;
+  const int n = src.slots();
+  for (int i0 = 0; i0 < n; i0 += 32 * U) {
+    uint32_t k[U];
+    int32_t ps[U];
+    src.template load<U>(i0, lane, k, ps);
+    uint32_t edge = 0;                                   // a handful per row
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const bool em = k[j] > khi;
+      const uint32_t m = __ballot_sync(0xffffffffu, em);
+      const uint32_t p = base + __popc(m & lt);
+      if (em && p < (uint32_t)K) out[p] = ps[j];
+      base += __popc(m);
+      edge |= k[j] - klo < n_keys ? 1u << j : 0u;
+    }
+    if (__any_sync(0xffffffffu, edge != 0)) {
+      const uint32_t ec = (uint32_t)__popc(edge);
+      uint32_t ei = ec;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, ei, o);
+        if (lane >= o) ei += v;
+      }
+      uint32_t q = ln + ei - ec;
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        const bool e = (edge >> j) & 1u;
+        if (e && q < (uint32_t)kSelSmall) sm.list[q] = make_entry(k[j], ps[j]);
+        q += e ? 1u : 0u;
+      }
+      ln += __shfl_sync(0xffffffffu, ei, 31);
+    }
+  }
+  *n_list = ln < (uint32_t)kSelSmall ? ln : (uint32_t)kSelSmall;
+  return (int)(base < (uint32_t)K ? base : (uint32_t)K);
+}
+
+// The need_b best of the ln listed entries follow the `base` entries already written (entries are distinct: a
+// rank is a slot).  Returns the row's length.
+__device__ __forceinline__ int warp_emit_list(const SegSelSmem& sm, uint32_t ln, uint32_t need_b, uint32_t base, int32_t* out,
+                                              float* out_score, int K, int lane) {
+  __syncwarp();
+  for (uint32_t t = lane; t < ln; t += 32) {
+    const entry_t xt = sm.list[t];
+    uint32_t rank = 0;
+    for (uint32_t u = 0; u < ln; ++u) rank += sm.list[u] > xt ? 1u : 0u;
+    if (rank < need_b && base + rank < (uint32_t)K) {
+      out[base + rank] = entry_pos(xt);
+      if (out_score) out_score[base + rank] = key_to_score(entry_key(xt));
+    }
+  }
+  __syncwarp();
+  const uint32_t n_out = base + (ln < need_b ? ln : need_b);
+  return (int)(n_out < (uint32_t)K ? n_out : (uint32_t)K);
+}
+
 // Last sweep: entries above bhi go out, those in [elo, bhi] are listed and the need_b best of
 // the list follow.  elo > bhi: nothing is listed.
 template <typename Src>
 __device__ __forceinline__ int warp_emit_above(SegSelSmem& sm, const Src& src, entry_t elo, entry_t bhi, uint32_t need_b,
                                                int32_t* out, float* out_score, int K, int lane) {
+  // boundary = a range of keys (always, unless ties narrowed it further): the lean sweep
+  if (!out_score && ((uint32_t)bhi == 0xffffffffu || bhi == 0ull) && ((uint32_t)elo == 0u || elo > bhi)) {
+    uint32_t ln = 0;
+    const uint32_t khi = (uint32_t)(bhi >> 32);
+    const int base = warp_emit_keys<16>(sm, src, khi, elo > bhi ? 0u : khi - (uint32_t)(elo >> 32) + 1u, &ln, out, K, lane);
+    return warp_emit_list(sm, ln, need_b, (uint32_t)base, out, out_score, K, lane);
+  }
   const uint32_t lt = (1u << lane) - 1u;
   uint32_t base = 0, ln = 0;
   src.template sweep<16, true>(lane, [&](entry_t e) {
@@ -468,20 +575,8 @@ __device__ __forceinline__ int warp_emit_above(SegSelSmem& sm, const Src& src, e
       b2 += __popc(m);
     });
   }
-  __syncwarp();
   ln = ln < (uint32_t)kSelSmall ? ln : (uint32_t)kSelSmall;
-  for (uint32_t t = lane; t < ln; t += 32) {                      // entries are distinct: ranks are slots
-    const entry_t xt = sm.list[t];
-    uint32_t rank = 0;
-    for (uint32_t u = 0; u < ln; ++u) rank += sm.list[u] > xt ? 1u : 0u;
-    if (rank < need_b && base + rank < (uint32_t)K) {
-      out[base + rank] = entry_pos(xt);
-      if (out_score) out_score[base + rank] = key_to_score(entry_key(xt));
-    }
-  }
-  __syncwarp();
-  const uint32_t n_out = base + (ln < need_b ? ln : need_b);
-  return (int)(n_out < (uint32_t)K ? n_out : (uint32_t)K);
+  return warp_emit_list(sm, ln, need_b, base, out, out_score, K, lane);
 }
 
 // [lo, hi] holds every entry of the source, n_filled of them.
@@ -506,8 +601,8 @@ __device__ __noinline__ int warp_topk_entries(SegSelSmem& sm, const Src src, ent
         if (shift >= 32) {                   // bins are key ranges (lo has a zero low word then)
           const uint32_t klo = (uint32_t)(lo >> 32), khi = (uint32_t)(hi >> 32);
           const int ksh = shift - 32;
-          src.template sweep_keys<32>(lane, [&](uint32_t k) {
-            if (k >= klo && k <= khi && k) atomicAdd(&sm.hist[(k - klo) >> ksh], 1u);
+          src.template sweep_keys<32>(lane, [&](uint32_t k) {      // (klo > 0: an empty slot wraps around out of range)
+            hist_add_if(sm.hist, (k - klo) >> ksh, k - klo <= khi - klo);
           });
           counted = true;
         }
@@ -536,11 +631,11 @@ __device__ __forceinline__ int warp_row_topk(SegSelSmem& sm, const uint32_t* key
                            ((entry_t)kmax << 32) | 0xffffffffull, n_filled, out, out_score, K, lane);
 }
 
-// A scan row's segment whose entries were all counted in a histogram with bins bin_of(key):
-// bsel = the boundary bin (need_b of its pop entries are wanted), -1 = everything is wanted.
+// A scan row's segment whose entries were all counted in a histogram whose bin b holds the keys
+// bin_lo(b) .. bin_lo(b + 1) - 1: bsel = the boundary bin (need_b of its pop entries are wanted), -1 = everything is wanted.
 // One sweep, unless the boundary bin is too crowded to rank (ties): then the general way.
 template <typename BinFn>
-__device__ __noinline__ int warp_seg_topk_binned(SegSelSmem& sm, const entry_t* seg, int cnt, BinFn bin_of, int bsel,
+__device__ __noinline__ int warp_seg_topk_binned(SegSelSmem& sm, const entry_t* seg, int cnt, BinFn bin_lo, int bsel,
                                                  uint32_t need_b, uint32_t pop, int32_t* out, float* out_score, int K,
                                                  int lane) {
   const SegSrc src{seg, cnt};
@@ -561,48 +656,18 @@ __device__ __noinline__ int warp_seg_topk_binned(SegSelSmem& sm, const entry_t* 
     nv = __reduce_add_sync(0xffffffffu, nv);
     return warp_topk_entries(sm, src, mn, mx, nv, out, out_score, K, lane);
   }
-  // the boundary bin as a set of entries: {e : bin_of(key(e)) == bsel}; above it: bin > bsel
-  const uint32_t lt = (1u << lane) - 1u;
+  // the boundary bin is the range of keys [lo_key(bsel), lo_key(bsel + 1)); a bin wanted whole counts as "above"
   const bool whole = bsel >= 0 && pop == need_b;
-  const int bcut = whole ? bsel - 1 : bsel;  // a bin wanted whole counts as "above"
-  uint32_t base = 0, ln = 0;
-  src.template sweep<16, true>(lane, [&](entry_t e) {
-    const int bn = e ? (int)bin_of(entry_key(e)) : -2;
-    const bool em = bn > bcut;
-    const bool edge = bn == bcut && bsel >= 0 && !whole;
-    const uint32_t m = __ballot_sync(0xffffffffu, em);
-    const uint32_t me = __ballot_sync(0xffffffffu, edge);
-    const uint32_t p = base + __popc(m & lt);
-    const uint32_t q = ln + __popc(me & lt);
-    if (em && p < (uint32_t)K) out[p] = entry_pos(e);
-    if (edge && q < (uint32_t)kSelSmall) sm.list[q] = e;
-    base += __popc(m);
-    ln += __popc(me);
-  });
-  if (out_score) {
-    uint32_t b2 = 0;
-    src.template sweep<16, true>(lane, [&](entry_t e) {
-      const bool em = (e ? (int)bin_of(entry_key(e)) : -2) > bcut;
-      const uint32_t m = __ballot_sync(0xffffffffu, em);
-      const uint32_t p = b2 + __popc(m & lt);
-      if (em && p < (uint32_t)K) out_score[p] = key_to_score(entry_key(e));
-      b2 += __popc(m);
-    });
+  const uint32_t above = bsel < 0 ? 1u : bin_lo(whole ? bsel : bsel + 1);      // smallest key above the boundary (0 = empty slot)
+  const uint32_t khi = above - 1u;
+  const uint32_t n_keys = bsel < 0 || whole ? 0u : above - bin_lo(bsel);      // keys of the boundary bin
+  if (!out_score) {
+    uint32_t ln = 0;
+    const int base = warp_emit_keys<16>(sm, src, khi, n_keys, &ln, out, K, lane);
+    return warp_emit_list(sm, ln, need_b, (uint32_t)base, out, out_score, K, lane);
   }
-  __syncwarp();
-  ln = ln < (uint32_t)kSelSmall ? ln : (uint32_t)kSelSmall;
-  for (uint32_t t = lane; t < ln; t += 32) {
-    const entry_t xt = sm.list[t];
-    uint32_t rank = 0;
-    for (uint32_t u = 0; u < ln; ++u) rank += sm.list[u] > xt ? 1u : 0u;
-    if (rank < need_b && base + rank < (uint32_t)K) {
-      out[base + rank] = entry_pos(xt);
-      if (out_score) out_score[base + rank] = key_to_score(entry_key(xt));
-    }
-  }
-  __syncwarp();
-  const uint32_t n_out = base + (ln < need_b ? ln : need_b);
-  return (int)(n_out < (uint32_t)K ? n_out : (uint32_t)K);
+  const entry_t ebhi = ((entry_t)khi << 32) | 0xffffffffull;
+  return warp_emit_above(sm, src, n_keys == 0u ? ~0ull : (entry_t)(above - n_keys) << 32, ebhi, need_b, out, out_score, K, lane);
 }
 
 }  // namespace pivot
