@@ -13,7 +13,8 @@ struct BlkSelSmem {
   entry_t small[kSelSmall];
   entry_t vmin, vmax, cut;
   uint32_t wsum[32];
-  uint32_t bin, need, pop, small_n, out_count, list_n;
+  uint32_t bin, need, pop, small_n, out_count, list_n, edge_n;
+  uint32_t kmin, kmax;
 };
 
 // Largest bin b (walking from the top) such that bins >= b hold at least `need` entries.
@@ -144,6 +145,111 @@ __device__ __forceinline__ entry_t blk_find_cut(BlkSelSmem& sm, const entry_t* l
     __syncthreads();
   }
   return lo;
+}
+
+// The same for a list that is read once into registers: U entries per thread cover it (n <= U * 1024, n > K).
+// Every later pass is then arithmetic; the range is taken over the 32-bit keys by warp reductions.
+template <int U>
+__device__ __forceinline__ entry_t blk_find_cut_regs(BlkSelSmem& sm, const entry_t (&x)[U], int K) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  uint32_t kmn = 0xffffffffu, kmx = 0u;
+#pragma unroll
+  for (int j = 0; j < U; ++j) {
+    const uint32_t k = entry_key(x[j]);                  // (0: a padding entry)
+    kmn = k && k < kmn ? k : kmn;
+    kmx = k > kmx ? k : kmx;
+  }
+  kmn = __reduce_min_sync(0xffffffffu, kmn);
+  kmx = __reduce_max_sync(0xffffffffu, kmx);
+  if (tid == 0) { sm.kmin = 0xffffffffu; sm.kmax = 0u; }
+  for (int i = tid; i < kSelBins; i += kBlk) sm.hist[i] = 0;
+  __syncthreads();
+  if (lane == 0) { atomicMin(&sm.kmin, kmn); atomicMax(&sm.kmax, kmx); }
+  __syncthreads();
+  entry_t lo = (entry_t)sm.kmin << 32, hi = ((entry_t)sm.kmax << 32) | 0xffffffffull;
+  uint32_t need = (uint32_t)K;
+  for (int iter = 0; iter < 8; ++iter) {
+    const int bitsw = 64 - __clzll((long long)((hi - lo) | 1ull));
+    const int shift = bitsw > 11 ? bitsw - 11 : 0;
+#pragma unroll
+    for (int j = 0; j < U; ++j)
+      if (x[j] >= lo && x[j] <= hi && x[j] != kPadEntry) atomicAdd(&sm.hist[(uint32_t)((x[j] - lo) >> shift)], 1u);
+    if (tid == 0) sm.small_n = 0;
+    blk_boundary(sm, sm.hist, kSelBins, need);
+    const uint32_t b = sm.bin, pop = sm.pop;
+    need = sm.need;
+    const entry_t lo2 = lo + ((entry_t)b << shift);
+    const entry_t width1 = shift ? (((entry_t)1 << shift) - 1ull) : 0ull;
+    const entry_t hi2 = (hi - lo2) < width1 ? hi : lo2 + width1;
+    if (pop == need) return lo2;
+    if (pop <= (uint32_t)kSelSmall) {
+#pragma unroll
+      for (int j = 0; j < U; ++j)
+        if (x[j] >= lo2 && x[j] <= hi2) {
+          const uint32_t p = atomicAdd(&sm.small_n, 1u);
+          if (p < (uint32_t)kSelSmall) sm.small[p] = x[j];
+        }
+      __syncthreads();
+      const int P = min((int)sm.small_n, kSelSmall);
+      if (tid < P) {
+        const entry_t xt = sm.small[tid];
+        uint32_t rank = 0;
+        for (int u = 0; u < P; ++u) rank += sm.small[u] > xt ? 1u : 0u;
+        if (rank == need - 1) sm.cut = xt;
+      }
+      __syncthreads();
+      return sm.cut;
+    }
+    lo = lo2;
+    hi = hi2;
+    __syncthreads();
+    for (int i = tid; i < kSelBins; i += kBlk) sm.hist[i] = 0;
+    __syncthreads();
+  }
+  return lo;
+}
+
+// blk_emit_topk for a list of at most U * 1024 entries, in list order, warp by warp.
+template <int U>
+__device__ __forceinline__ void blk_emit_topk_regs(BlkSelSmem& sm, const entry_t* list, int n, int K, int32_t* out,
+                                                   float* out_score, int copies, int stride) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  entry_t x[U];
+  // warp w holds entries [w * 32 U, (w + 1) * 32 U): its kept entries are one run of the output
+#pragma unroll
+  for (int j = 0; j < U; ++j) {
+    const int i = wid * (32 * U) + j * 32 + lane;
+    const entry_t e = i < n ? list[i] : kPadEntry;
+    x[j] = entry_pos(e) >= 0 ? e : kPadEntry;
+  }
+  const entry_t cut = n > K ? blk_find_cut_regs<U>(sm, x, K) : 1ull;
+  uint32_t m[U], cnt = 0;
+#pragma unroll
+  for (int j = 0; j < U; ++j) {
+    m[j] = __ballot_sync(0xffffffffu, x[j] >= cut && x[j] != kPadEntry);
+    cnt += (uint32_t)__popc(m[j]);
+  }
+  __syncthreads();
+  if (lane == 0) sm.wsum[wid] = cnt;
+  __syncthreads();
+  const uint32_t v = sm.wsum[lane];
+  uint32_t before = __reduce_add_sync(0xffffffffu, lane < wid ? v : 0u);
+  const uint32_t got = __reduce_add_sync(0xffffffffu, v);
+#pragma unroll
+  for (int j = 0; j < U; ++j) {
+    const uint32_t p = before + __popc(m[j] & ((1u << lane) - 1u));
+    if (((m[j] >> lane) & 1u) && p < (uint32_t)K)
+      for (int r = 0; r < copies; ++r) {
+        out[(size_t)r * stride + p] = entry_pos(x[j]);
+        if (out_score) out_score[(size_t)r * stride + p] = key_to_score(entry_key(x[j]));
+      }
+    before += (uint32_t)__popc(m[j]);
+  }
+  for (int i = (int)got + tid; i < K; i += kBlk)
+    for (int r = 0; r < copies; ++r) {
+      out[(size_t)r * stride + i] = -1;
+      if (out_score) out_score[(size_t)r * stride + i] = -INFINITY;
+    }
 }
 
 // Writes the K best entries of list[0..n) (positions, optional scores; unordered; padding

@@ -135,6 +135,8 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
       TileWalk tw(tile_prefix, B);
       int cur_b = -1;
       uint32_t it = 0, blk = 0;
+      // keys are read once a step: they give way in L2 before the scores, which the select reads next
+      const uint64_t once = ptx::l2_evict_first();
       PIVOT_PROF_DO(long long pwait = 0;)
       for (int g = g_lo; g < g_hi; ++g, ++it) {
         const int b = tw.seq_of(g);
@@ -160,7 +162,7 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
         PIVOT_PROF_DO(pwait += clock64() - pw0;)
         ptx::mbar_arrive_expect_tx(&ct.full[s], C::STAGE_BYTES);
         for (int h = 0; h < C::KHALVES; ++h)
-          ptx::tma_load_2d(kring + s * C::STAGE_BYTES + h * C::HALF_TILE_BYTES, &tm_k, h * 64, krow, &ct.full[s]);
+          ptx::tma_load_2d_hint(kring + s * C::STAGE_BYTES + h * C::HALF_TILE_BYTES, &tm_k, h * 64, krow, &ct.full[s], once);
         if (C::FP8) {
           const int ksl = it % DKS_SLOTS;       // free by construction (see the prefill scan)
           ptx::mbar_arrive_expect_tx(&ct.ks_full[ksl], TILE_KEYS * 4);
@@ -311,7 +313,11 @@ struct SelSmem {
   entry_t list[SEL_CAP];
 };
 
-// The SEL_SPLIT CTAs of a sequence are one thread-block cluster (blockIdx.x = rank in it).
+// The SEL_SPLIT CTAs of a sequence are one thread-block cluster (blockIdx.x = rank in it).  The histogram the
+// scan left names the bin that holds the K-th best score: whatever lies above it is selected, each CTA writes
+// what its share of the scores holds of that, and only the bin's own entries go to CTA 0 to be ranked (with
+// all survivors collected there and ranked together that CTA's part alone took 13 of 36 K clocks, the
+// hand-over 6 K: 24.6 us a step of 32 sequences of 64K .. 128K keys against 20.5).
 __global__ void __cluster_dims__(SEL_SPLIT, 1, 1) __launch_bounds__(kBlk, 1)
 decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __restrict__ scores,
                      const uint32_t* __restrict__ ghist, int* status) {
@@ -323,22 +329,30 @@ decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __re
   PIVOT_PROF_DO(long long pt[5]; pt[0] = clock64();)
   const RowDesc rd = prox[b];
   const int K = rd.K, n0 = rd.n_vis;
-  if (K <= 0) return;
+  if (K <= 0) return;                     // (the whole cluster)
   const float* sc = scores + (size_t)b * Ls;
-  // ---- narrow the candidates: entries whose top `pbits` bits are >= prefix
+  // ---- the boundary: keys >= above are selected, of the keys in [edge, above) `need` are
+  uint32_t need = 0, above = 1u, edge = 1u;           // n0 <= K: everything (a score key is never 0)
   unsigned long long prefix = 0;
   int pbits = 0;
   bool solo = false;              // this CTA handles the whole sequence by itself
-  if (n0 > SEL_CAP) {
+  if (n0 > K) {
     blk_boundary(sm.blk, ghist + (size_t)b * DHIST, DHIST, (uint32_t)K);
-    uint32_t need = sm.blk.need, pop = sm.blk.pop;
-    prefix = sm.blk.bin;
-    pbits = DHIST_BITS;
+    const uint32_t bin = sm.blk.bin;
+    uint32_t pop = sm.blk.pop;
+    need = sm.blk.need;
+    edge = bin << (32 - DHIST_BITS);
+    above = bin + 1 < (uint32_t)DHIST ? (bin + 1) << (32 - DHIST_BITS) : 0xffffffffu;
+    if (pop == need) { above = edge; need = 0; }      // the bin is wanted whole
     // too crowded a boundary bin (every CTA of the sequence sees the same histogram): the
     // refinement passes need the whole score array, CTA 0 takes the sequence alone
-    solo = (uint32_t)K - need + pop > (uint32_t)SEL_CAP;
+    solo = need > 0 && (uint32_t)K - need + pop > (uint32_t)SEL_CAP;
     if (solo && split != 0) return;          // (the whole cluster takes this branch or none: no cluster barrier follows)
-    while ((uint32_t)K - need + pop > (uint32_t)SEL_CAP && pbits < 64) {
+    if (solo) {
+      prefix = bin;
+      pbits = DHIST_BITS;
+    }
+    while (solo && (uint32_t)K - need + pop > (uint32_t)SEL_CAP && pbits < 64) {
       const int wbits = 64 - pbits < 12 ? 64 - pbits : 12;
       __syncthreads();
       for (int i = tid; i < 4096; i += kBlk) sm.blk.hist[i] = 0;
@@ -372,10 +386,11 @@ decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __re
     }
   }
   PIVOT_PROF_DO(pt[1] = clock64();)
-  // ---- collect them in shared memory: this CTA's share of the scores (multiples of four)
+  // ---- collect them in shared memory: this CTA's share of the scores (multiples of four); what is selected
+  //      grows from the start of the list, what has to be ranked from its end
   const int lo = solo ? 0 : (int)(((long long)n0 * split / SEL_SPLIT) & ~3ll);
   const int hi = (solo || split == SEL_SPLIT - 1) ? n0 : (int)(((long long)n0 * (split + 1) / SEL_SPLIT) & ~3ll);
-  if (tid == 0) sm.blk.list_n = 0;
+  if (tid == 0) { sm.blk.list_n = 0; sm.blk.edge_n = 0; }
   __syncthreads();
   for (int i0 = lo; i0 < hi; i0 += 32 * kBlk) {        // eight 16-byte loads in flight per thread
     float4 v4[8];
@@ -384,76 +399,108 @@ decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __re
       const int i = i0 + (u * kBlk + tid) * 4;
       v4[u] = i < hi ? __ldcg(reinterpret_cast<const float4*>(sc + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    // One list-cursor bump per warp and pass: each thread counts its keepers among its 32
+    // One cursor bump per warp, pass and list: each thread counts its keepers among its 32
     // scores, a warp scan turns the counts into offsets (a bump per keeper group would queue
-    // hundreds of same-address atomics per pass).  The test runs on the 32-bit score key while
-    // the prefix is no longer than that (always, unless a crowded bin was refined further):
-    // the pass is bound by its instruction count, not by the loads.
+    // hundreds of same-address atomics per pass).  The tests run on the 32-bit score key (but for the
+    // refined prefix of a crowded bin): the pass is bound by its instruction count, not by the loads.
     auto score_of = [&](int u) -> float {
       const float4 q4 = v4[u >> 2];
       return (u & 3) == 0 ? q4.x : (u & 3) == 1 ? q4.y : (u & 3) == 2 ? q4.z : q4.w;
     };
     auto pos_of = [&](int u) -> int { return i0 + ((u >> 2) * kBlk + tid) * 4 + (u & 3); };
-    uint32_t keepmask = 0;
-    if (pbits <= 32) {
-      const uint32_t kthr = pbits ? (uint32_t)prefix << (32 - pbits) : 0u;
+    uint32_t sel = 0, rank = 0;
+    if (!solo) {
 #pragma unroll
-      for (int u = 0; u < 32; ++u)
-        keepmask |= (pos_of(u) < hi && score_to_key(score_of(u)) >= kthr) ? 1u << u : 0u;
+      for (int u = 0; u < 32; ++u) {
+        const uint32_t key = score_to_key(score_of(u));
+        const bool in = pos_of(u) < hi;
+        sel |= in && key >= above ? 1u << u : 0u;
+        rank |= in && key >= edge && key < above ? 1u << u : 0u;
+      }
     } else {
 #pragma unroll
       for (int u = 0; u < 32; ++u) {
         const entry_t e = make_entry(score_to_key(score_of(u)), pos_of(u));
-        keepmask |= (pos_of(u) < hi && (e >> (64 - pbits)) >= prefix) ? 1u << u : 0u;
+        rank |= (pos_of(u) < hi && (e >> (64 - pbits)) >= prefix) ? 1u << u : 0u;
       }
     }
-    const uint32_t cnt = (uint32_t)__popc(keepmask);
-    uint32_t incl = cnt;
+    auto collect = [&](uint32_t mask, uint32_t* cursor, bool down) {
+      const uint32_t cnt = (uint32_t)__popc(mask);
+      uint32_t incl = cnt;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
-    if (tot) {                                           // warp-uniform
-      uint32_t base = 0;
-      if (lane == 31) base = atomicAdd(&sm.blk.list_n, tot);
-      base = __shfl_sync(0xffffffffu, base, 31);
-      uint32_t p = base + incl - cnt;
-      while (keepmask) {                                 // a few per cent of the scores are kept
-        const int u = __ffs(keepmask) - 1;
-        keepmask &= keepmask - 1u;
-        float vu = 0.f;
-#pragma unroll
-        for (int q = 0; q < 32; ++q) vu = q == u ? score_of(q) : vu;
-        if (p < (uint32_t)SEL_CAP) sm.list[p] = make_entry(score_to_key(vu), pos_of(u));
-        ++p;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
       }
-    }
+      const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
+      if (tot) {                                           // warp-uniform
+        uint32_t base = 0;
+        if (lane == 31) base = atomicAdd(cursor, tot);
+        base = __shfl_sync(0xffffffffu, base, 31);
+        uint32_t p = base + incl - cnt;
+        while (mask) {                                     // a few per cent of the scores are kept
+          const int u = __ffs(mask) - 1;
+          mask &= mask - 1u;
+          float vu = 0.f;
+#pragma unroll
+          for (int q = 0; q < 32; ++q) vu = q == u ? score_of(q) : vu;
+          if (p < (uint32_t)SEL_CAP) sm.list[down ? SEL_CAP - 1 - p : p] = make_entry(score_to_key(vu), pos_of(u));
+          ++p;
+        }
+      }
+    };
+    collect(sel, &sm.blk.list_n, false);
+    collect(rank, &sm.blk.edge_n, true);
   }
   __syncthreads();
   PIVOT_PROF_DO(pt[2] = clock64();)
-  int n = min((int)sm.blk.list_n, SEL_CAP);
-  if (!solo) {
-    // ---- hand the shares over: the four CTAs of a sequence form a cluster, and CTA 0 reads the
-    //      others' lists out of their shared memory
-    cg::cluster_group cluster = cg::this_cluster();
-    cluster.sync();                                      // every list is complete
-    if (split == 0) {
-      for (int r = 1; r < SEL_SPLIT; ++r) {
-        const SelSmem* rs = cluster.map_shared_rank(&sm, r);
-        const int nr = min((int)rs->blk.list_n, SEL_CAP);
-        for (int i = tid; i < nr; i += kBlk)
-          if (n + i < SEL_CAP) sm.list[n + i] = rs->list[i];
-        n = min(n + nr, SEL_CAP);
-      }
+  const int n_sel = min((int)sm.blk.list_n, SEL_CAP);
+  int n_edge = min((int)sm.blk.edge_n, SEL_CAP - n_sel);
+  if (solo) {
+    blk_emit_topk(sm.blk, sm.list + SEL_CAP - n_edge, n_edge, n_edge, K, rd.out, rd.out_score, rd.out_rows, rd.out_stride);
+    return;
+  }
+  // ---- hand the shares over: the four CTAs of a sequence form a cluster.  Everybody writes its selected
+  //      entries behind those of the CTAs before it; CTA 0 reads the others' boundary entries out of their
+  //      shared memory and ranks them all.
+  cg::cluster_group cluster = cg::this_cluster();
+  cluster.sync();                                      // every list is complete
+  int before = 0, all_sel = 0;
+  for (int r = 0; r < SEL_SPLIT; ++r) {
+    const int nr = r == split ? n_sel : min((int)cluster.map_shared_rank(&sm, r)->blk.list_n, SEL_CAP);
+    before += r < split ? nr : 0;
+    all_sel += nr;
+  }
+  if (split == 0 && need > 0) {
+    for (int r = 1; r < SEL_SPLIT; ++r) {
+      const SelSmem* rs = cluster.map_shared_rank(&sm, r);
+      const int nr = min((int)rs->blk.edge_n, SEL_CAP);
+      for (int i = tid; i < nr; i += kBlk)
+        if (n_sel + n_edge + i < SEL_CAP) sm.list[SEL_CAP - 1 - n_edge - i] = rs->list[SEL_CAP - 1 - i];
+      n_edge = min(n_edge + nr, SEL_CAP - n_sel);
     }
-    cluster.sync();                                      // nobody leaves while its list is being read
-    if (split != 0) return;
-    __syncthreads();
   }
   PIVOT_PROF_DO(pt[3] = clock64();)
-  blk_emit_topk(sm.blk, sm.list, n, n, K, rd.out, rd.out_score, rd.out_rows, rd.out_stride);
+  for (int i = tid; i < n_sel; i += kBlk) {
+    const entry_t e = sm.list[i];
+    if (before + i < K)
+      for (int r = 0; r < rd.out_rows; ++r) {
+        rd.out[(size_t)r * rd.out_stride + before + i] = entry_pos(e);
+        if (rd.out_score) rd.out_score[(size_t)r * rd.out_stride + before + i] = key_to_score(entry_key(e));
+      }
+  }
+  cluster.sync();                                      // nobody leaves while its list is being read
+  if (split != 0) return;
+  // the boundary's best, and -1 behind them where the sequence has fewer than K keys
+  const int rest = K - min(all_sel, K);
+  if (rest > 0) {
+    int32_t* const out = rd.out + (K - rest);
+    float* const outs = rd.out_score ? rd.out_score + (K - rest) : nullptr;
+    const entry_t* const list = sm.list + SEL_CAP - n_edge;
+    const int n = need > 0 ? n_edge : 0;
+    if (n <= 2 * kBlk) blk_emit_topk_regs<2>(sm.blk, list, n, rest, out, outs, rd.out_rows, rd.out_stride);
+    else blk_emit_topk(sm.blk, list, n, n, rest, out, outs, rd.out_rows, rd.out_stride);
+  }
   PIVOT_PROF_DO(__syncthreads(); if (tid == 0) {
     pt[4] = clock64();
     for (int i = 0; i < 4; ++i) prof_add(status, PROF_DSEL_BOUNDARY + i, pt[i + 1] - pt[i]);
@@ -470,8 +517,13 @@ __global__ void __launch_bounds__(kBlk, 1) entries_topk_kernel(const EntryList* 
   ptx::grid_dependency_wait();            // the re-score's entries
   const EntryList el = lists[blockIdx.x];
   if (el.K <= 0) return;
-  blk_emit_topk(sm, (const entry_t*)el.list, el.n, el.n, el.K, el.out, el.out_score, 1, el.K);
+  // by the entries a thread holds: the list is read once
+  const entry_t* list = (const entry_t*)el.list;
+  if (el.n <= 2 * kBlk) blk_emit_topk_regs<2>(sm, list, el.n, el.K, el.out, el.out_score, 1, el.K);
+  else if (el.n <= 5 * kBlk) blk_emit_topk_regs<5>(sm, list, el.n, el.K, el.out, el.out_score, 1, el.K);
+  else blk_emit_topk_regs<9>(sm, list, el.n, el.K, el.out, el.out_score, 1, el.K);
 }
+static_assert(8192 + kDecodeWinMax <= 9 * kBlk, "largest candidate budget plus window slots");
 
 // Union of candidate lists -> packed entries -> exact top-K, one block.
 __global__ void __launch_bounds__(kBlk, 1)
@@ -498,12 +550,15 @@ merge_topk_kernel(const float* __restrict__ scores, const int32_t* __restrict__ 
 // its place in the tile order of the key-split scan (the tile counts of the sequences before it,
 // recomputed from their pos0 -- a few loads instead of a hand-over between blocks), and writes its
 // candidate chunks for the re-score and its entry lists for the final top-k.  1024 threads per block.
+__device__ __forceinline__ bool decode_bad_pos(const DecodePlan& p, int p_in) {
+  const int step = p.g > p.kv_share ? p.g : p.kv_share;
+  return p_in < 0 || p_in > p.Lmax - step;
+}
 __device__ __forceinline__ int decode_live_tiles(const DecodePlan& p, int b) {
   // tiles of sequence b's proxy scan, as plan_decode_sequence decides them: 0 for a guarded
   // sequence and for a pos0 outside the cache
   const int p_in = p.pos0[b / p.kv_share];
-  const int step = p.g > p.kv_share ? p.g : p.kv_share;
-  if (p_in < 0 || p_in > p.Lmax - step) return 0;
+  if (decode_bad_pos(p, p_in)) return 0;
   const int n0 = p_in + b % p.kv_share + 1;
   return n0 < p.guard_len ? 0 : (n0 + TILE_KEYS - 1) / TILE_KEYS;
 }
@@ -511,7 +566,7 @@ __device__ __forceinline__ int decode_live_tiles(const DecodePlan& p, int b) {
 __global__ void __launch_bounds__(1024)
 decode_prepare_kernel(DecodePlan p, RowDesc* rows, GroupDesc* plan_groups, uint32_t* ghist, int W, int pool, int chunk,
                       int* tile_prefix, GroupDesc* chunks, EntryList* lists, unsigned long long* entries,
-                      const int32_t* wcand) {
+                      const int32_t* wcand, int* status) {
   const int b = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int B = p.B, g = p.g, c = p.c, k = p.k, mode = p.mode;
@@ -520,6 +575,12 @@ decode_prepare_kernel(DecodePlan p, RowDesc* rows, GroupDesc* plan_groups, uint3
   __shared__ int seq_ok;
   __shared__ int wsum[32];
   if (tid == 0) seq_ok = plan_decode_sequence(p, b, rows, plan_groups) ? 1 : 0;
+  if (b == 0) {                    // the step's status word and row counter start here (p.status is not set)
+    bool bad = false;
+    for (int bb = tid; bb < B; bb += blockDim.x) bad |= decode_bad_pos(p, p.pos0[bb / p.kv_share]);
+    const int any = __syncthreads_or(bad);
+    if (tid < 2) status[tid] = tid == 0 && any ? DEV_BAD_POS : 0;
+  }
   // ---- tiles of the sequences before this one
   int part = 0;
   for (int bb = tid; bb < b; bb += blockDim.x) part += decode_live_tiles(p, bb);
@@ -680,7 +741,7 @@ cudaError_t launch_decode_fast(const DecodeFast& d, cudaStream_t st) {
   unsigned long long* entries = (unsigned long long*)p;
 
   decode_prepare_kernel<<<d.B, 1024, 0, st>>>(d.plan, d.prox, d.groups, ghist, W, d.pool, chunk, tile_prefix, chunks, lists,
-                                              entries, wcand);
+                                              entries, wcand, d.status);
   ++launch_counter();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;

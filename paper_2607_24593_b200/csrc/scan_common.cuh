@@ -186,8 +186,8 @@ __device__ __noinline__ void append_role(SelectCtrl<NROWS, QD>& s, int r, int la
       // at or below a valid threshold and can never reach a bin edge the threshold could still
       // move to, so the counts that matter stay exact.
       auto take = [&](entry_t x, bool on, int p) {
-        hist_add_if(rhist, (uint32_t)select_bin(entry_key(x), base), on);
         if (on) {
+          atomicAdd(&rhist[select_bin(entry_key(x), base)], 1u);
           if (p < CAP) seg[p] = x;
           else s.abort_code = DEV_CAND_OVERFLOW;
         }
