@@ -487,7 +487,7 @@ static int run_decode(const pivot_tensor* q, const float* w, const pivot_tensor*
     if (!paged) {
       ScanOperands op{kcache->data, k_rows, kcache->scale, q->data, B * g, ws.proxy_q, B, q->dtype};
       op.k_stride = p.k_stride;
-      if ((rc = check_cuda(launch_scan_tc(op, ws.rows + B, B * g, 1, tc_scratch(ws), sm_count(), st)))) return rc;
+      if ((rc = check_cuda(launch_scan_tc(op, ws.rows + B, B * g, 1, tc_scratch(ws), sm_count(), st, false, true)))) return rc;
     }
   }
   mark(3, st);

@@ -10,7 +10,7 @@
 //                        epilogue (ReLU, gate-weighted head sum, key scale) -> one fp32 score per
 //                        key to an L2-resident score array (3 % of the bytes read), plus a
 //                        8192-bin histogram of the scores' top 13 key bits per sequence.
-//   decode_select_kernel a cluster of four 1024-thread CTAs per sequence: the histogram gives the
+//   decode_select_kernel a cluster of up to four 1024-thread CTAs per sequence: the histogram gives the
 //                        bin holding the K-th best score; each CTA collects the survivors of its
 //                        quarter of the score array in its shared memory; after a cluster barrier
 //                        CTA 0 reads the other three lists through distributed shared memory and
@@ -45,7 +45,6 @@ constexpr int DHIST = 1 << DHIST_BITS;
 constexpr int D_N = kHeads;             // MMA N: one proxy
 constexpr int D_THREADS = 64 + 256;     // TMA warp, MMA warp, two sets of four epilogue warps
 constexpr int SEL_CAP = 16384;          // candidates collected in shared memory per sequence
-constexpr int SEL_SPLIT = 4;            // CTAs sharing the collection pass of one sequence
 
 template <int DT>
 struct DCfg {
@@ -55,7 +54,7 @@ struct DCfg {
   static constexpr int STAGE_BYTES = KHALVES * HALF_TILE_BYTES;
   static constexpr int QHALF_BYTES = kHeads * 128;
   static constexpr int QBUF_BYTES = KHALVES * QHALF_BYTES;
-  static constexpr int STAGES = FP8 ? 8 : 3;
+    static constexpr int STAGES = FP8 ? 8 : 3;
   static constexpr uint32_t IDESC = ptx::make_idesc(FP8 ? 0u : 1u, TILE_KEYS, D_N);
 };
 
@@ -313,12 +312,13 @@ struct SelSmem {
   entry_t list[SEL_CAP];
 };
 
-// The SEL_SPLIT CTAs of a sequence are one thread-block cluster (blockIdx.x = rank in it).  The histogram the
+// The SPLIT CTAs of a sequence are one thread-block cluster (blockIdx.x = rank in it).  The histogram the
 // scan left names the bin that holds the K-th best score: whatever lies above it is selected, each CTA writes
 // what its share of the scores holds of that, and only the bin's own entries go to CTA 0 to be ranked (with
 // all survivors collected there and ranked together that CTA's part alone took 13 of 36 K clocks, the
 // hand-over 6 K: 24.6 us a step of 32 sequences of 64K .. 128K keys against 20.5).
-__global__ void __cluster_dims__(SEL_SPLIT, 1, 1) __launch_bounds__(kBlk, 1)
+template <int SEL_SPLIT>
+__global__ void __launch_bounds__(kBlk, 1)
 decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __restrict__ scores,
                      const uint32_t* __restrict__ ghist, int* status) {
   extern __shared__ uint8_t sel_raw[];
@@ -438,14 +438,11 @@ decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __re
         if (lane == 31) base = atomicAdd(cursor, tot);
         base = __shfl_sync(0xffffffffu, base, 31);
         uint32_t p = base + incl - cnt;
-        while (mask) {                                     // a few per cent of the scores are kept
-          const int u = __ffs(mask) - 1;
-          mask &= mask - 1u;
-          float vu = 0.f;
 #pragma unroll
-          for (int q = 0; q < 32; ++q) vu = q == u ? score_of(q) : vu;
-          if (p < (uint32_t)SEL_CAP) sm.list[down ? SEL_CAP - 1 - p : p] = make_entry(score_to_key(vu), pos_of(u));
-          ++p;
+        for (int u = 0; u < 32; ++u) {                     // (a loop over the set bits picks each score by 32 selects)
+          const bool on = (mask >> u) & 1u;
+          if (on && p < (uint32_t)SEL_CAP) sm.list[down ? SEL_CAP - 1 - p : p] = make_entry(score_to_key(score_of(u)), pos_of(u));
+          p += on ? 1u : 0u;
         }
       }
     };
@@ -511,7 +508,10 @@ decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __re
 
 // ------------------------------------------------------------------------------ top-k of entry lists
 
-__global__ void __launch_bounds__(kBlk, 1) entries_topk_kernel(const EntryList* __restrict__ lists) {
+// PER_SM: blocks that share an SM (two where one wave would not hold the queries otherwise: 192 queries took
+// two waves, 9 us; one block per SM has the registers to hold its list without spills, 5 us against 7.6).
+template <int PER_SM>
+__global__ void __launch_bounds__(kBlk, PER_SM) entries_topk_kernel(const EntryList* __restrict__ lists) {
   __shared__ BlkSelSmem sm;
   ptx::grid_launch_dependents();
   ptx::grid_dependency_wait();            // the re-score's entries
@@ -616,8 +616,8 @@ decode_prepare_kernel(DecodePlan p, RowDesc* rows, GroupDesc* plan_groups, uint3
   const int w_g = W > 0 ? W + g - 1 : 0;
   const int stride = c + kDecodeWinMax;            // entries per query
   for (int j = tid; j < mc * nch; j += blockDim.x) {
-    const int i = b * mc * nch + j;
-    const int gi = i / nch, cc = i % nch;
+    const int gi = b * mc + j / nch, cc = j % nch;
+    const int i = cc * (B * mc) + gi;              // (all full chunks before the window's: the last wave is the light one)
     GroupDesc gd = groups[gi];
     gd.ent_out = entries + (size_t)gd.q_row * stride;
     gd.ent_stride = stride;
@@ -694,6 +694,17 @@ cudaError_t launch_scan(const CUtensorMap& mk, const CUtensorMap& mq, const CUte
                        ghist, status);
 }
 
+template <int SPLIT>
+cudaError_t launch_select(const DecodeFast& d, int Ls, const float* scores, const uint32_t* ghist, cudaStream_t st) {
+  auto kern = decode_select_kernel<SPLIT>;
+  static bool attr_set[kMaxDevices] = {};
+  const size_t smem = sizeof(SelSmem) + 16;
+  if (cudaError_t e = opt_in_dynamic_smem(kern, smem, attr_set); e != cudaSuccess) return e;
+  ++launch_counter();
+  return launch_clusters(SPLIT, kern, dim3(SPLIT, d.B), dim3(kBlk), smem, st, true, (const RowDesc*)d.prox, Ls, scores, ghist,
+                         d.status);
+}
+
 }  // namespace
 
 bool make_operand_map(CUtensorMap* m, const void* base, long long rows, int dtype, int box_rows, int row_stride);
@@ -760,13 +771,12 @@ cudaError_t launch_decode_fast(const DecodeFast& d, cudaStream_t st) {
           : launch_scan<DT_BF16>(mk, mq, mks, d.prox, tile_prefix, d.B, Ls, scores, ghist, d.status, d.sms, st);
   if (e != cudaSuccess) return e;
   if (d.ev_scan_end) cudaEventRecord(d.ev_scan_end, st);
-  static bool sel_attr[kMaxDevices] = {};
-  const size_t sel_smem = sizeof(SelSmem) + 16;
-  if ((e = opt_in_dynamic_smem(decode_select_kernel, sel_smem, sel_attr)) != cudaSuccess) return e;
-  if ((e = launch_kernel(decode_select_kernel, dim3(SEL_SPLIT, d.B), dim3(kBlk), sel_smem, st, true, (const RowDesc*)d.prox,
-                         Ls, (const float*)scores, (const uint32_t*)ghist, d.status)) != cudaSuccess)
+  // CTAs per sequence: as many as still make one wave (the kernel takes an SM to itself; 48 sequences in
+  // clusters of four took two waves, 32 us)
+  if ((e = d.B * 4 <= d.sms   ? launch_select<4>(d, Ls, scores, ghist, st)
+           : d.B * 2 <= d.sms ? launch_select<2>(d, Ls, scores, ghist, st)
+                              : launch_select<1>(d, Ls, scores, ghist, st)) != cudaSuccess)
     return e;
-  ++launch_counter();
   if (d.ev_scan_end && d.ev_select_end) cudaEventRecord(d.ev_select_end, st);
   }
   if (d.mode == 1) {
@@ -779,8 +789,8 @@ cudaError_t launch_decode_fast(const DecodeFast& d, cudaStream_t st) {
     ScanScratch sc = d.scratch_tc;
     e = launch_refine_tc(d.q, d.B * d.g, d.dtype, chunks, d.B * mc * nch, sc, d.sms, st, false, true, 0, true);
     if (e != cudaSuccess) return e;
-    if ((e = launch_kernel(entries_topk_kernel, dim3(d.B * d.g), dim3(kBlk), 0, st, true, (const EntryList*)lists)) !=
-        cudaSuccess)
+    if ((e = launch_kernel(d.B * d.g <= d.sms ? entries_topk_kernel<1> : entries_topk_kernel<2>, dim3(d.B * d.g), dim3(kBlk), 0,
+                           st, true, (const EntryList*)lists)) != cudaSuccess)
       return e;
     ++launch_counter();
   }

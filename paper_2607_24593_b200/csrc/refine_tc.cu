@@ -72,7 +72,7 @@ static_assert(META_SLOTS >= 6 + 2, "meta ring");
 // What the epilogue needs to know about a gathered key: its position and scale.
 struct KeyMeta {
   int idx;       // key position, -1 for a padding slot
-  float ks;      // key scale (1 for bf16)
+  float ks;      // key scale (FP8)
 };
 
 // MMA2: the group's gate matrix, bf16, K-major with 128-byte swizzle, in the compact form the
@@ -110,6 +110,9 @@ static_assert(rsmem_bytes<DT_FP8, 0>() <= 232448 && rsmem_bytes<DT_FP8, 2>() <= 
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int NPEND>
@@ -327,9 +330,10 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* __re
       const int ntiles = group_tiles(gd);
       if (ntiles == 0) continue;
       const int krow_bytes = gd.k_stride > 0 ? gd.k_stride : C::ROW_BYTES;   // padded cache rows (32-bit: one wide multiply per address)
-      // Candidate positions are fetched three tiles ahead, their rows in the key tensor (a
-      // block-table lookup when the cache is paged) two tiles ahead and key scales one tile
-      // ahead, so no round trip sits on this thread's issue path.
+      // Candidate positions are fetched three tiles ahead and their rows in the key tensor (a
+      // block-table lookup when the cache is paged) two tiles ahead, so no round trip sits on this
+      // thread's issue path.  Key scales go straight to shared memory with the keys (as loads into
+      // registers a tile ahead they stalled every tile of a decode step, whose scales lie in HBM).
       const int pos_limit = gd.pos_max;
       auto load_idx = [&](int tile, int half) -> int {
         const int sl = tile * TILE_KEYS + wrow0 + half * 32 + lane;
@@ -347,27 +351,25 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* __re
         (void)PIVOT_BOUNDS(pg < (uint32_t)gd.n_pages, sc.status);     // checked build: a hole in the block table is reported
         return pg < (uint32_t)gd.n_pages ? (int)(pg * 128u + (uint32_t)(ix & 127)) : -1;
       };
-      auto load_ks = [&](int row) -> float { return (gd.kscale && row >= 0) ? __ldg(gd.kscale + row) : 1.f; };
       int idx0[2] = {load_idx(0, 0), load_idx(0, 1)}, idx1[2] = {load_idx(1, 0), load_idx(1, 1)};
       int idx2[2] = {load_idx(2, 0), load_idx(2, 1)};
       int row0[2] = {key_row(idx0[0]), key_row(idx0[1])}, row1[2] = {key_row(idx1[0]), key_row(idx1[1])};
-      float ks0[2] = {load_ks(row0[0]), load_ks(row0[1])};
       for (int t = 0; t < ntiles; ++t, ++it) {
         const int s = it % C::STAGES;
         const uint32_t ph = (it / C::STAGES) & 1;
         const int idx3[2] = {load_idx(t + 3, 0), load_idx(t + 3, 1)};
         const int row2[2] = {key_row(idx2[0]), key_row(idx2[1])};
-        const float ks1[2] = {load_ks(row1[0]), load_ks(row1[1])};
         if (ok) ok = ptx::mbar_wait(&ct.empty[s], ph ^ 1, abort_flag, 64);   // whole warps wait here: sleep, do not spin
         int krow[2];
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
           const int row = wrow0 + half * 32 + lane;
-          ct.meta[it % META_SLOTS][row] = KeyMeta{row0[half] < 0 ? -1 : idx0[half], ks0[half]};
+          KeyMeta& km = ct.meta[it % META_SLOTS][row];
+          km.idx = row0[half] < 0 ? -1 : idx0[half];
           krow[half] = row0[half] < 0 ? 0 : row0[half];
+          if (gd.kscale) cp_async4(ptx::smem_u32(&km.ks), gd.kscale + krow[half]);   // (only read where there are scales)
           idx0[half] = idx1[half]; idx1[half] = idx2[half]; idx2[half] = idx3[half];
           row0[half] = row1[half]; row1[half] = row2[half];
-          ks0[half] = ks1[half];
         }
         const uint32_t dst0 = ptx::smem_u32(kring + s * C::STAGE_BYTES);
 #pragma unroll

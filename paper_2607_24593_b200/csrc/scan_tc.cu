@@ -619,12 +619,12 @@ cudaError_t launch_scan_tc(const ScanOperands& op, const RowDesc* rows, int n_ro
       !make_operand_map(&mq1, op.proxy_q, (long long)(op.proxy_rows > 0 ? op.proxy_rows : 1) * kHeads, op.dtype, kHeads, 0))
     return cudaErrorInvalidValue;
   if (op.dtype == DT_FP8) {
-    if (rows_per_block != 4) return launch_one<DT_FP8, 1>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st);
+    if (rows_per_block != 4) return launch_one<DT_FP8, 1>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev);
     return fp32_head_sum ? launch_one<DT_FP8, 4, 0>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev)
                          : launch_one<DT_FP8, 4, 1>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev);
   }
   return rows_per_block == 4 ? launch_one<DT_BF16, 4>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev)
-                             : launch_one<DT_BF16, 1>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st);
+                             : launch_one<DT_BF16, 1>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev);
 }
 
 }  // namespace pivot
