@@ -44,7 +44,8 @@ constexpr int DHIST_BITS = 13;          // histogram digit: top 13 bits of the s
 constexpr int DHIST = 1 << DHIST_BITS;
 constexpr int D_N = kHeads;             // MMA N: one proxy
 constexpr int D_THREADS = 64 + 256;     // TMA warp, MMA warp, two sets of four epilogue warps
-constexpr int SEL_CAP = 16384;          // candidates collected in shared memory per sequence
+constexpr int SEL_CAP = 12288;          // survivors collected in shared memory per CTA of a sequence
+constexpr int EDGE_CAP = 4096;          // ... of which boundary entries
 
 template <int DT>
 struct DCfg {
@@ -310,13 +311,14 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
 struct SelSmem {
   BlkSelSmem blk;
   entry_t list[SEL_CAP];
+  entry_t edge[EDGE_CAP];
 };
 
 // The SPLIT CTAs of a sequence are one thread-block cluster (blockIdx.x = rank in it).  The histogram the
 // scan left names the bin that holds the K-th best score: whatever lies above it is selected, each CTA writes
 // what its share of the scores holds of that, and only the bin's own entries go to CTA 0 to be ranked (with
 // all survivors collected there and ranked together that CTA's part alone took 13 of 36 K clocks, the
-// hand-over 6 K: 24.6 us a step of 32 sequences of 64K .. 128K keys against 20.5).
+// hand-over 6 K: 24.6 us a step of 32 sequences of 64K .. 128K keys, now 18.4).
 template <int SEL_SPLIT>
 __global__ void __launch_bounds__(kBlk, 1)
 decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __restrict__ scores,
@@ -346,7 +348,7 @@ decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __re
     if (pop == need) { above = edge; need = 0; }      // the bin is wanted whole
     // too crowded a boundary bin (every CTA of the sequence sees the same histogram): the
     // refinement passes need the whole score array, CTA 0 takes the sequence alone
-    solo = need > 0 && (uint32_t)K - need + pop > (uint32_t)SEL_CAP;
+    solo = need > 0 && (pop > (uint32_t)EDGE_CAP || (uint32_t)K - need + pop > (uint32_t)SEL_CAP);
     if (solo && split != 0) return;          // (the whole cluster takes this branch or none: no cluster barrier follows)
     if (solo) {
       prefix = bin;
@@ -386,104 +388,122 @@ decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __re
     }
   }
   PIVOT_PROF_DO(pt[1] = clock64();)
-  // ---- collect them in shared memory: this CTA's share of the scores (multiples of four); what is selected
-  //      grows from the start of the list, what has to be ranked from its end
+  // ---- collect the scores at or above the boundary bin in shared memory: this CTA's share (multiples of four).
+  // The pass is bound by its instruction count (32 warps of it on an SM): sixteen scores per thread, a key from
+  // two instructions, one bit mask, one cursor bump per warp, and what is selected is told from what has to be
+  // ranked only afterwards, among the few per cent that were kept (both tests on every score, 32 scores per
+  // thread however small the share: 13 K clocks for shares of 2 K scores).
   const int lo = solo ? 0 : (int)(((long long)n0 * split / SEL_SPLIT) & ~3ll);
   const int hi = (solo || split == SEL_SPLIT - 1) ? n0 : (int)(((long long)n0 * (split + 1) / SEL_SPLIT) & ~3ll);
-  if (tid == 0) { sm.blk.list_n = 0; sm.blk.edge_n = 0; }
+  if (tid == 0) { sm.blk.list_n = 0; sm.blk.edge_n = 0; sm.blk.out_count = 0; }
   __syncthreads();
-  for (int i0 = lo; i0 < hi; i0 += 32 * kBlk) {        // eight 16-byte loads in flight per thread
-    float4 v4[8];
+  constexpr int U = 4;
+  for (int i0 = lo; i0 < hi; i0 += 4 * U * kBlk) {
+    uint32_t v[4 * U];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < U; ++u) {
       const int i = i0 + (u * kBlk + tid) * 4;
-      v4[u] = i < hi ? __ldcg(reinterpret_cast<const float4*>(sc + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const uint4 q = i < hi ? __ldcg(reinterpret_cast<const uint4*>(sc + i)) : make_uint4(~0u, ~0u, ~0u, ~0u);   // (key 0)
+      v[4 * u] = q.x; v[4 * u + 1] = q.y; v[4 * u + 2] = q.z; v[4 * u + 3] = q.w;
     }
-    // One cursor bump per warp, pass and list: each thread counts its keepers among its 32
-    // scores, a warp scan turns the counts into offsets (a bump per keeper group would queue
-    // hundreds of same-address atomics per pass).  The tests run on the 32-bit score key (but for the
-    // refined prefix of a crowded bin): the pass is bound by its instruction count, not by the loads.
-    auto score_of = [&](int u) -> float {
-      const float4 q4 = v4[u >> 2];
-      return (u & 3) == 0 ? q4.x : (u & 3) == 1 ? q4.y : (u & 3) == 2 ? q4.z : q4.w;
-    };
     auto pos_of = [&](int u) -> int { return i0 + ((u >> 2) * kBlk + tid) * 4 + (u & 3); };
-    uint32_t sel = 0, rank = 0;
-    if (!solo) {
+    uint32_t mask = 0;
 #pragma unroll
-      for (int u = 0; u < 32; ++u) {
-        const uint32_t key = score_to_key(score_of(u));
-        const bool in = pos_of(u) < hi;
-        sel |= in && key >= above ? 1u << u : 0u;
-        rank |= in && key >= edge && key < above ? 1u << u : 0u;
-      }
-    } else {
+    for (int u = 0; u < 4 * U; ++u) {
+      v[u] ^= (uint32_t)((int32_t)v[u] >> 31) | 0x80000000u;                // score_to_key
+      mask |= v[u] >= edge ? 1u << u : 0u;
+    }
 #pragma unroll
-      for (int u = 0; u < 32; ++u) {
-        const entry_t e = make_entry(score_to_key(score_of(u)), pos_of(u));
-        rank |= (pos_of(u) < hi && (e >> (64 - pbits)) >= prefix) ? 1u << u : 0u;
+    for (int u = 0; u < U; ++u) {                                           // past the end inside the last 16 bytes
+      const int left = hi - pos_of(4 * u);
+      if (left < 4) mask &= ~(0xfu << (4 * u)) | ((left > 0 ? (1u << left) - 1u : 0u) << (4 * u));
+    }
+    if (solo) {
+#pragma unroll
+      for (int u = 0; u < 4 * U; ++u)
+        if ((make_entry(v[u], pos_of(u)) >> (64 - pbits)) < prefix) mask &= ~(1u << u);
+    }
+    const uint32_t cnt = (uint32_t)__popc(mask);
+    uint32_t incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t w = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += w;
+    }
+    const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
+    if (tot) {                                           // warp-uniform
+      uint32_t base = 0;
+      if (lane == 31) base = atomicAdd(&sm.blk.list_n, tot);
+      base = __shfl_sync(0xffffffffu, base, 31);
+      uint32_t p = base + incl - cnt;
+#pragma unroll
+      for (int u = 0; u < 4 * U; ++u) {
+        const bool on = (mask >> u) & 1u;
+        if (on && p < (uint32_t)SEL_CAP) sm.list[p] = make_entry(v[u], pos_of(u));
+        p += on ? 1u : 0u;
       }
     }
-    auto collect = [&](uint32_t mask, uint32_t* cursor, bool down) {
-      const uint32_t cnt = (uint32_t)__popc(mask);
-      uint32_t incl = cnt;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
-      if (tot) {                                           // warp-uniform
-        uint32_t base = 0;
-        if (lane == 31) base = atomicAdd(cursor, tot);
-        base = __shfl_sync(0xffffffffu, base, 31);
-        uint32_t p = base + incl - cnt;
-#pragma unroll
-        for (int u = 0; u < 32; ++u) {                     // (a loop over the set bits picks each score by 32 selects)
-          const bool on = (mask >> u) & 1u;
-          if (on && p < (uint32_t)SEL_CAP) sm.list[down ? SEL_CAP - 1 - p : p] = make_entry(score_to_key(score_of(u)), pos_of(u));
-          p += on ? 1u : 0u;
-        }
-      }
-    };
-    collect(sel, &sm.blk.list_n, false);
-    collect(rank, &sm.blk.edge_n, true);
   }
   __syncthreads();
   PIVOT_PROF_DO(pt[2] = clock64();)
-  const int n_sel = min((int)sm.blk.list_n, SEL_CAP);
-  int n_edge = min((int)sm.blk.edge_n, SEL_CAP - n_sel);
+  const int n = min((int)sm.blk.list_n, SEL_CAP);
   if (solo) {
-    blk_emit_topk(sm.blk, sm.list + SEL_CAP - n_edge, n_edge, n_edge, K, rd.out, rd.out_score, rd.out_rows, rd.out_stride);
+    blk_emit_topk(sm.blk, sm.list, n, n, K, rd.out, rd.out_score, rd.out_rows, rd.out_stride);
     return;
   }
-  // ---- hand the shares over: the four CTAs of a sequence form a cluster.  Everybody writes its selected
+  // ---- selected entries counted per warp, boundary entries listed; warp w looks after a run of the list
+  const int run = ((n + kBlk - 1) / kBlk) * 32;
+  const int r0 = (tid >> 5) * run, r1 = min(r0 + run, n);
+  const uint32_t lt = (1u << lane) - 1u;
+  uint32_t mine = 0;
+  for (int i = r0; i < r1; i += 32) {
+    const entry_t e = i + lane < r1 ? sm.list[i + lane] : 0ull;
+    const bool se = entry_key(e) >= above;
+    const bool eg = e && !se;
+    mine += (uint32_t)__popc(__ballot_sync(0xffffffffu, se));
+    const uint32_t m = __ballot_sync(0xffffffffu, eg);
+    if (m) {
+      uint32_t base = 0;
+      if (lane == 0) base = atomicAdd(&sm.blk.edge_n, (uint32_t)__popc(m));
+      base = __shfl_sync(0xffffffffu, base, 0) + __popc(m & lt);
+      if (eg && base < (uint32_t)EDGE_CAP) sm.edge[base] = e;
+    }
+  }
+  uint32_t wbase = 0;
+  if (lane == 0 && mine) wbase = atomicAdd(&sm.blk.out_count, mine);
+  wbase = __shfl_sync(0xffffffffu, wbase, 0);
+  // ---- hand the shares over: the CTAs of a sequence form a cluster.  Everybody writes its selected
   //      entries behind those of the CTAs before it; CTA 0 reads the others' boundary entries out of their
   //      shared memory and ranks them all.
   cg::cluster_group cluster = cg::this_cluster();
   cluster.sync();                                      // every list is complete
-  int before = 0, all_sel = 0;
+  int before = 0, all_sel = 0, n_edge = min((int)sm.blk.edge_n, EDGE_CAP);
+#pragma unroll
   for (int r = 0; r < SEL_SPLIT; ++r) {
-    const int nr = r == split ? n_sel : min((int)cluster.map_shared_rank(&sm, r)->blk.list_n, SEL_CAP);
+    const int nr = min((int)cluster.map_shared_rank(&sm, r)->blk.out_count, SEL_CAP);
     before += r < split ? nr : 0;
     all_sel += nr;
   }
   if (split == 0 && need > 0) {
     for (int r = 1; r < SEL_SPLIT; ++r) {
       const SelSmem* rs = cluster.map_shared_rank(&sm, r);
-      const int nr = min((int)rs->blk.edge_n, SEL_CAP);
+      const int nr = min((int)rs->blk.edge_n, EDGE_CAP);
       for (int i = tid; i < nr; i += kBlk)
-        if (n_sel + n_edge + i < SEL_CAP) sm.list[SEL_CAP - 1 - n_edge - i] = rs->list[SEL_CAP - 1 - i];
-      n_edge = min(n_edge + nr, SEL_CAP - n_sel);
+        if (n_edge + i < EDGE_CAP) sm.edge[n_edge + i] = rs->edge[i];
+      n_edge = min(n_edge + nr, EDGE_CAP);
     }
   }
   PIVOT_PROF_DO(pt[3] = clock64();)
-  for (int i = tid; i < n_sel; i += kBlk) {
-    const entry_t e = sm.list[i];
-    if (before + i < K)
+  for (int i = r0; i < r1; i += 32) {
+    const entry_t e = i + lane < r1 ? sm.list[i + lane] : 0ull;
+    const bool se = entry_key(e) >= above;
+    const uint32_t m = __ballot_sync(0xffffffffu, se);
+    const uint32_t p = (uint32_t)before + wbase + __popc(m & lt);
+    wbase += (uint32_t)__popc(m);
+    if (se && p < (uint32_t)K)
       for (int r = 0; r < rd.out_rows; ++r) {
-        rd.out[(size_t)r * rd.out_stride + before + i] = entry_pos(e);
-        if (rd.out_score) rd.out_score[(size_t)r * rd.out_stride + before + i] = key_to_score(entry_key(e));
+        rd.out[(size_t)r * rd.out_stride + p] = entry_pos(e);
+        if (rd.out_score) rd.out_score[(size_t)r * rd.out_stride + p] = key_to_score(entry_key(e));
       }
   }
   cluster.sync();                                      // nobody leaves while its list is being read
@@ -493,10 +513,9 @@ decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __re
   if (rest > 0) {
     int32_t* const out = rd.out + (K - rest);
     float* const outs = rd.out_score ? rd.out_score + (K - rest) : nullptr;
-    const entry_t* const list = sm.list + SEL_CAP - n_edge;
-    const int n = need > 0 ? n_edge : 0;
-    if (n <= 2 * kBlk) blk_emit_topk_regs<2>(sm.blk, list, n, rest, out, outs, rd.out_rows, rd.out_stride);
-    else blk_emit_topk(sm.blk, list, n, n, rest, out, outs, rd.out_rows, rd.out_stride);
+    const int ne = need > 0 ? n_edge : 0;
+    if (ne <= 2 * kBlk) blk_emit_topk_regs<2>(sm.blk, sm.edge, ne, rest, out, outs, rd.out_rows, rd.out_stride);
+    else blk_emit_topk_regs<4>(sm.blk, sm.edge, ne, rest, out, outs, rd.out_rows, rd.out_stride);
   }
   PIVOT_PROF_DO(__syncthreads(); if (tid == 0) {
     pt[4] = clock64();
