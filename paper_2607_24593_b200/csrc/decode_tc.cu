@@ -251,7 +251,7 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
         cur_b = b;
         n_vis = prox[b].n_vis;
         tm.sync();
-        if (tt < kHeads) ct.w[set][tt] = 0.5f * prox[b].w[tt];      // proxy gate, halved (ReLU identity)
+        if (tt < kHeads) ct.w[set][tt] = prox[b].w[tt];      // proxy gate
         tm.sync();
       }
       const int buf = it & 1;                        // == set
@@ -271,25 +271,10 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&ct.tmem_empty[buf]);
-      float ap[4] = {0.f, 0.f, 0.f, 0.f}, an[4] = {0.f, 0.f, 0.f, 0.f};
-      const float4* wp = reinterpret_cast<const float4*>(&ct.w[set][0]);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const float4 wa = wp[j], wbv = wp[8 + j];
-        const float x0 = __uint_as_float(v0[4 * j]), x1 = __uint_as_float(v0[4 * j + 1]);
-        const float x2 = __uint_as_float(v0[4 * j + 2]), x3 = __uint_as_float(v0[4 * j + 3]);
-        const float y0 = __uint_as_float(v1[4 * j]), y1 = __uint_as_float(v1[4 * j + 1]);
-        const float y2 = __uint_as_float(v1[4 * j + 2]), y3 = __uint_as_float(v1[4 * j + 3]);
-        ap[0] = fmaf(fabsf(x0), wa.x, ap[0]); an[0] = fmaf(x0, wa.x, an[0]);
-        ap[1] = fmaf(fabsf(x1), wa.y, ap[1]); an[1] = fmaf(x1, wa.y, an[1]);
-        ap[2] = fmaf(fabsf(x2), wa.z, ap[2]); an[2] = fmaf(x2, wa.z, an[2]);
-        ap[3] = fmaf(fabsf(x3), wa.w, ap[3]); an[3] = fmaf(x3, wa.w, an[3]);
-        ap[0] = fmaf(fabsf(y0), wbv.x, ap[0]); an[0] = fmaf(y0, wbv.x, an[0]);
-        ap[1] = fmaf(fabsf(y1), wbv.y, ap[1]); an[1] = fmaf(y1, wbv.y, an[1]);
-        ap[2] = fmaf(fabsf(y2), wbv.z, ap[2]); an[2] = fmaf(y2, wbv.z, an[2]);
-        ap[3] = fmaf(fabsf(y3), wbv.w, ap[3]); an[3] = fmaf(y3, wbv.w, an[3]);
-      }
-      float sv = ((ap[0] + an[0]) + (ap[1] + an[1])) + ((ap[2] + an[2]) + (ap[3] + an[3]));
+      ptx::f32x2 acc[4] = {0ull, 0ull, 0ull, 0ull};
+      ptx::relu_dot32(v0, &ct.w[set][0], acc);
+      ptx::relu_dot32(v1, &ct.w[set][32], acc);
+      float sv = ptx::relu_dot_sum(acc);
       if (C::FP8) sv *= ksv;
       const int s_key = t * TILE_KEYS + key_in_tile;
       if (s_key < n_vis && PIVOT_BOUNDS(s_key < Lmax, status)) {

@@ -294,6 +294,44 @@ __device__ __forceinline__ void tc_mma_a_tmem_bf16(uint32_t d_tmem, uint32_t a_t
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// Two fp32 values in one 64-bit register pair and the packed arithmetic on them.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ float sum2(f32x2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return a + b;
+}
+// acc += w * max(x, 0) for 32 accumulator columns of a row; w: the row's gates in shared memory (16-byte aligned),
+// read as they are used (a broadcast), four independent chains.  A product of three register operands is
+// bound by the register file's read ports: as two scalar FMAs per value ((w/2) x + (w/2) |x|) it took 3.2
+// clocks per value, warp and scheduler, as a maximum and half a packed FMA 2.5.
+__device__ __forceinline__ void relu_dot32(const uint32_t (&x)[32], const float* w, f32x2 (&acc)[4]) {
+  const ulonglong2* wp = reinterpret_cast<const ulonglong2*>(w);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const ulonglong2 wv = wp[j];
+    acc[(2 * j) & 3] = fma2(pack2(fmaxf(__uint_as_float(x[4 * j]), 0.f), fmaxf(__uint_as_float(x[4 * j + 1]), 0.f)), wv.x,
+                            acc[(2 * j) & 3]);
+    acc[(2 * j + 1) & 3] = fma2(pack2(fmaxf(__uint_as_float(x[4 * j + 2]), 0.f), fmaxf(__uint_as_float(x[4 * j + 3]), 0.f)),
+                                wv.y, acc[(2 * j + 1) & 3]);
+  }
+}
+__device__ __forceinline__ float relu_dot_sum(const f32x2 (&acc)[4]) { return sum2(add2(add2(acc[0], acc[1]), add2(acc[2], acc[3]))); }
 __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }

@@ -485,7 +485,7 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* __re
           wv = gd.w[r * kHeads + jh];
           if (gd.qscale) wv = __fmul_rn(wv, gd.qscale[r * kHeads + jh]);
         }
-        ct.w[r][jh] = 0.5f * wv;       // halved: see the ReLU identity in the tile loop
+        ct.w[r][jh] = wv;
         tm.sync();
       }
       // One member row's result: a key never seen by the member (beyond its own position, or
@@ -612,26 +612,10 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* __re
           ptx::tmem_ld_32x32(taddr, v0);
           ptx::tmem_ld_32x32(taddr + 32, v1);
           ptx::tmem_wait_ld();
-          // w ReLU(x) = (w/2) x + (w/2) |x| (ct.w holds w/2): full-rate FMAs, eight chains
-          float ap[4] = {0.f, 0.f, 0.f, 0.f}, an[4] = {0.f, 0.f, 0.f, 0.f};
-          const float4* wp = reinterpret_cast<const float4*>(&ct.w[r][0]);
-#pragma unroll
-          for (int q4 = 0; q4 < 8; ++q4) {
-            const float4 wa = wp[q4], wb = wp[8 + q4];
-            const float x0 = __uint_as_float(v0[4 * q4]), x1 = __uint_as_float(v0[4 * q4 + 1]);
-            const float x2 = __uint_as_float(v0[4 * q4 + 2]), x3 = __uint_as_float(v0[4 * q4 + 3]);
-            const float y0 = __uint_as_float(v1[4 * q4]), y1 = __uint_as_float(v1[4 * q4 + 1]);
-            const float y2 = __uint_as_float(v1[4 * q4 + 2]), y3 = __uint_as_float(v1[4 * q4 + 3]);
-            ap[0] = fmaf(fabsf(x0), wa.x, ap[0]); an[0] = fmaf(x0, wa.x, an[0]);
-            ap[1] = fmaf(fabsf(x1), wa.y, ap[1]); an[1] = fmaf(x1, wa.y, an[1]);
-            ap[2] = fmaf(fabsf(x2), wa.z, ap[2]); an[2] = fmaf(x2, wa.z, an[2]);
-            ap[3] = fmaf(fabsf(x3), wa.w, ap[3]); an[3] = fmaf(x3, wa.w, an[3]);
-            ap[0] = fmaf(fabsf(y0), wb.x, ap[0]); an[0] = fmaf(y0, wb.x, an[0]);
-            ap[1] = fmaf(fabsf(y1), wb.y, ap[1]); an[1] = fmaf(y1, wb.y, an[1]);
-            ap[2] = fmaf(fabsf(y2), wb.z, ap[2]); an[2] = fmaf(y2, wb.z, an[2]);
-            ap[3] = fmaf(fabsf(y3), wb.w, ap[3]); an[3] = fmaf(y3, wb.w, an[3]);
-          }
-          score[rl] = ((ap[0] + an[0]) + (ap[1] + an[1])) + ((ap[2] + an[2]) + (ap[3] + an[3]));
+          ptx::f32x2 acc[4] = {0ull, 0ull, 0ull, 0ull};
+          ptx::relu_dot32(v0, &ct.w[r][0], acc);
+          ptx::relu_dot32(v1, &ct.w[r][32], acc);
+          score[rl] = ptx::relu_dot_sum(acc);
         }
         ptx::tc_fence_before();
         __syncwarp();

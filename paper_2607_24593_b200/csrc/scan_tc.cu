@@ -368,7 +368,7 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
             wv = rows[ri].w[j];
             if (rows[ri].qscale) wv = __fmul_rn(wv, rows[ri].qscale[j]);
           }
-          ct.w[r][j] = 0.5f * wv;       // halved: see the ReLU identity below
+          ct.w[r][j] = wv;
         }
       }
       int n_vis[C::ROWS_PER_TEAM];
@@ -468,27 +468,11 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
         ptx::tc_fence_after();
         // The accumulator comes over in 32-column chunks, two register sets in turn: while one
         // chunk goes through the FMAs the next is already on its way from TMEM.
-        // w ReLU(x) = (w/2) x + (w/2) |x|: two full-rate FMAs per element (|x| is a free operand
-        // modifier) instead of a half-rate max plus an FMA; ct.w holds w/2.  Eight independent
-        // accumulation chains per row keep the FMA pipe busy.
         float score[C::ROWS_PER_TEAM];
         constexpr int NCHUNK = 2 * C::ROWS_PER_TEAM;            // 32-column chunks of this warp
         const uint32_t tbase = tmem_base + ((uint32_t)(lq * 32) << 16) + buf * C::N + team * C::ROWS_PER_TEAM * kHeads;
         uint32_t va[32], vb[32];
-        float ap[4], an[4];
-        auto fma_chunk = [&](const uint32_t (&v)[32], const float* wrow) {
-          const float4* wp = reinterpret_cast<const float4*>(wrow);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float4 wv = wp[j];
-            const float x0 = __uint_as_float(v[4 * j]), x1 = __uint_as_float(v[4 * j + 1]);
-            const float x2 = __uint_as_float(v[4 * j + 2]), x3 = __uint_as_float(v[4 * j + 3]);
-            ap[0] = fmaf(fabsf(x0), wv.x, ap[0]); an[0] = fmaf(x0, wv.x, an[0]);
-            ap[1] = fmaf(fabsf(x1), wv.y, ap[1]); an[1] = fmaf(x1, wv.y, an[1]);
-            ap[2] = fmaf(fabsf(x2), wv.z, ap[2]); an[2] = fmaf(x2, wv.z, an[2]);
-            ap[3] = fmaf(fabsf(x3), wv.w, ap[3]); an[3] = fmaf(x3, wv.w, an[3]);
-          }
-        };
+        ptx::f32x2 acc[4];
         ptx::tmem_ld_32x32_async(tbase, va);
 #pragma unroll
         for (int c = 0; c < NCHUNK; ++c) {
@@ -498,14 +482,11 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
             if (c & 1) ptx::tmem_ld_32x32_async(tbase + (c + 1) * 32, va);
             else ptx::tmem_ld_32x32_async(tbase + (c + 1) * 32, vb);
           }
-          if ((c & 1) == 0) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { ap[i] = 0.f; an[i] = 0.f; }
-          }
+          if ((c & 1) == 0) acc[0] = acc[1] = acc[2] = acc[3] = 0ull;
           const float* wrow = &ct.w[team * C::ROWS_PER_TEAM + (c >> 1)][(c & 1) * 32];
-          if (c & 1) fma_chunk(vb, wrow);
-          else fma_chunk(va, wrow);
-          if (c & 1) score[c >> 1] = ((ap[0] + an[0]) + (ap[1] + an[1])) + ((ap[2] + an[2]) + (ap[3] + an[3]));
+          if (c & 1) ptx::relu_dot32(vb, wrow, acc);
+          else ptx::relu_dot32(va, wrow, acc);
+          if (c & 1) score[c >> 1] = ptx::relu_dot_sum(acc);
         }
         ptx::tc_fence_before();
         __syncwarp();
