@@ -129,6 +129,14 @@ __device__ __forceinline__ bool mbar_wait_poll(uint64_t* bar, uint32_t parity, v
   }
 }
 
+// Predicated stores: a branch around a store costs a warp its reconvergence.
+__device__ __forceinline__ void st_shared_if(uint32_t addr, uint64_t v, bool on) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.b64 [%0], %1;\n\t}" ::"r"(addr), "l"(v), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void st_shared_if(uint32_t addr, uint32_t v, bool on) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.b32 [%0], %1;\n\t}" ::"r"(addr), "r"(v), "r"((uint32_t)on) : "memory");
+}
+
 // ------------------------------------------------------------------ TMA
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* m) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");

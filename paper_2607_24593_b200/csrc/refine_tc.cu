@@ -371,16 +371,17 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* __re
           idx0[half] = idx1[half]; idx1[half] = idx2[half]; idx2[half] = idx3[half];
           row0[half] = row1[half]; row1[half] = row2[half];
         }
-        const uint32_t dst0 = ptx::smem_u32(kring + s * C::STAGE_BYTES);
+        // (row & 7 is sub or sub + 4 in turn: two swizzled offsets, everything else an immediate; the copy of
+        // a bf16 tile is bound by this loop's instruction count)
+        const uint32_t dst0 = ptx::smem_u32(kring + s * C::STAGE_BYTES) + (uint32_t)(wrow0 + sub) * 128u;
+        const uint32_t dsw[2] = {dst0 + (uint32_t)((chunk ^ sub) << 4), dst0 + (uint32_t)((chunk ^ (sub + 4)) << 4)};
+        const uint8_t* const kb = (const uint8_t*)gd.kbase + chunk * 16;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {                 // four rows per pass
-          const int rl = i * 4 + sub;                  // row inside this warp's 64
-          const int kr = __shfl_sync(0xffffffffu, krow[i >> 3], rl & 31);
-          const int row = wrow0 + rl;
-          const uint8_t* src = (const uint8_t*)gd.kbase + (long long)kr * krow_bytes + chunk * 16;
-          const uint32_t dst = dst0 + (uint32_t)row * 128u + (uint32_t)((chunk ^ (row & 7)) << 4);
+          const int kr = __shfl_sync(0xffffffffu, krow[i >> 3], (i & 7) * 4 + sub);
+          const uint8_t* src = kb + (long long)kr * krow_bytes;
 #pragma unroll
-          for (int h = 0; h < C::KHALVES; ++h) cp_async16(dst + h * C::HALF_TILE_BYTES, src + h * 128);
+          for (int h = 0; h < C::KHALVES; ++h) cp_async16(dsw[i & 1] + i * 512 + h * C::HALF_TILE_BYTES, src + h * 128);
         }
         cp_async_commit();
         if (it + 1 - pub > (uint32_t)C::LOOKAHEAD) {

@@ -85,14 +85,22 @@ __device__ __forceinline__ entry_t* row_segment(const ScanScratch& sc, int r, ui
   return sc.cand64 + (((size_t)blockIdx.x * NROWS + r) * 2 + (seq & 1u)) * sc.cap;
 }
 
-// A score warp leaves the survivors of its 32 keys of row r in the tile's queue: compacted by one
-// vote, count beside them.  `take` must already include the causal cut and the threshold test.
-template <int NROWS, int QD>
-__device__ __forceinline__ void push_survivors(SelectCtrl<NROWS, QD>& s, int qb, int r, int lq, int lane, bool take,
-                                               uint32_t key, int s_key) {
-  const uint32_t m = __ballot_sync(0xffffffffu, take);
-  if (take) s.q[qb][r][lq][__popc(m & ((1u << lane) - 1u))] = make_entry(key, s_key);
-  if (lane == 0) s.qn[qb][r][lq] = (uint32_t)__popc(m);
+// A score warp leaves the survivors of its 32 keys of rows r0 .. r0 + NR - 1 in the tile's queue: each row's
+// compacted by one vote, the counts beside them (lane i stores row r0 + i's).  `take` must already include the
+// causal cut and the threshold test.  No branches.
+template <int NR, int NROWS, int QD>
+__device__ __forceinline__ void push_survivors(SelectCtrl<NROWS, QD>& s, int qb, int r0, int lq, int lane, const bool (&take)[NR],
+                                               const uint32_t (&key)[NR], int s_key) {
+  const uint32_t lt = (1u << lane) - 1u;
+  const uint32_t q = ptx::smem_u32(&s.q[qb][r0][lq][0]);
+  uint32_t n = 0;
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    const uint32_t m = __ballot_sync(0xffffffffu, take[i]);
+    ptx::st_shared_if(q + i * (4 * 32 * 8) + __popc(m & lt) * 8, (uint64_t)make_entry(key[i], s_key), take[i]);
+    n = lane == i ? (uint32_t)__popc(m) : n;
+  }
+  ptx::st_shared_if(ptx::smem_u32(&s.qn[qb][r0][lq]) + (lane < NR ? lane : 0) * 16, n, lane < NR);
 }
 
 // Score key -> histogram bin: 256 bins per octave (8 mantissa bits), 2048 bins anchored two
@@ -186,10 +194,9 @@ __device__ __noinline__ void append_role(SelectCtrl<NROWS, QD>& s, int r, int la
       // at or below a valid threshold and can never reach a bin edge the threshold could still
       // move to, so the counts that matter stay exact.
       auto take = [&](entry_t x, bool on, int p) {
-        if (on) {
+        if (on && p < CAP) {                     // (CHK leaves room for every tile until the next check)
           atomicAdd(&rhist[select_bin(entry_key(x), base)], 1u);
-          if (p < CAP) seg[p] = x;
-          else s.abort_code = DEV_CAND_OVERFLOW;
+          seg[p] = x;
         }
       };
       if (t > 0 && total <= 32) {
@@ -228,7 +235,8 @@ __device__ __noinline__ void append_role(SelectCtrl<NROWS, QD>& s, int r, int la
           p += (int)nq[j];
         }
       }
-      cnt = min(cnt + (int)total, CAP);
+      cnt += (int)total;
+      if (cnt > CAP) { cnt = CAP; s.abort_code = DEV_CAND_OVERFLOW; }
     }
     // ---- end of the block: the histogram is exact for everything the segment still holds; read
     //      the boundary bin off it and hand the row to its finisher

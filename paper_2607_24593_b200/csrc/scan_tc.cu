@@ -444,11 +444,14 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
             const int qb = it % QD;
             (void)ptx::mbar_wait(&ct.s.sc_empty[qb], ((it / QD) & 1) ^ 1, abort_flag);
             const int s_key = t * TILE_KEYS + key_in_tile;
+            uint32_t key[NROWS];
+            bool take[NROWS];
 #pragma unroll
             for (int r = 0; r < NROWS; ++r) {
-              const uint32_t key = score_to_key((__uint_as_float(sv[r]) + __uint_as_float(sv[4 + r])) * ksv);
-              scan::push_survivors(ct.s, qb, r, lq, lane, s_key < nv4[r] && key > scan::row_threshold(ct.s, r, seq), key, s_key);
+              key[r] = score_to_key((__uint_as_float(sv[r]) + __uint_as_float(sv[4 + r])) * ksv);
+              take[r] = s_key < nv4[r] && key[r] > scan::row_threshold(ct.s, r, seq);
             }
+            scan::push_survivors<NROWS>(ct.s, qb, 0, lq, lane, take, key, s_key);
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&ct.s.sc_full[qb]);
           }
@@ -495,12 +498,14 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
         const int qb = it % QD;
         (void)ptx::mbar_wait(&ct.s.sc_empty[qb], ((it / QD) & 1) ^ 1, abort_flag);
         const int s_key = t * TILE_KEYS + key_in_tile;
+        uint32_t key[C::ROWS_PER_TEAM];
+        bool take[C::ROWS_PER_TEAM];
 #pragma unroll
         for (int rl = 0; rl < C::ROWS_PER_TEAM; ++rl) {
-          const int r = team * C::ROWS_PER_TEAM + rl;
-          const uint32_t key = score_to_key(C::FP8 ? score[rl] * ksv : score[rl]);
-          scan::push_survivors(ct.s, qb, r, lq, lane, s_key < n_vis[rl] && key > scan::row_threshold(ct.s, r, seq), key, s_key);
+          key[rl] = score_to_key(C::FP8 ? score[rl] * ksv : score[rl]);
+          take[rl] = s_key < n_vis[rl] && key[rl] > scan::row_threshold(ct.s, team * C::ROWS_PER_TEAM + rl, seq);
         }
+        scan::push_survivors<C::ROWS_PER_TEAM>(ct.s, qb, team * C::ROWS_PER_TEAM, lq, lane, take, key, s_key);
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&ct.s.sc_full[qb]);
       }
