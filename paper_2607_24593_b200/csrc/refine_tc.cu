@@ -54,8 +54,11 @@ struct RCfg {
   // the next group's queries load while this one is re-scored, except where 2 x 64 KB of bf16
   // queries would leave no room for the select warps' histograms
   static constexpr int QBUFS = (OVL && !FP8) ? 1 : 2;
-  static constexpr int STAGES = FP8 ? 6 : 2;
-  static constexpr int LOOKAHEAD = FP8 ? 4 : 1;   // gather tiles in flight per producer thread
+  static constexpr int STAGES = FP8 ? 6 : QBUFS == 1 ? 3 : 2;
+  // Gather tiles a producer thread has in flight beyond the one it publishes.  A tile is published once the next
+  // has been issued, and that needs a free stage: a deeper look-ahead holds finished tiles back (bf16, three
+  // stages: two ahead 2.42 ms, one ahead 1.85 at 32K; two stages 2.29).
+  static constexpr int LOOKAHEAD = 1;
   static constexpr int ROW_BYTES = FP8 ? 128 : 256;
   static constexpr uint32_t IDESC = ptx::make_idesc(FP8 ? 0u : 1u, TILE_KEYS, N);
   // FP8: the gate-weighted head sum of Eq. 8 runs on the tensor core, as in the shared scan (a
