@@ -8,6 +8,7 @@ kernels.  Importing this module fails loudly when the shared library has not bee
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 
 import torch
@@ -121,8 +122,8 @@ def _tensor(data: torch.Tensor, scale) -> pivot_tensor:
 
 
 def _stream(stream) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:                       # (the stream object costs more than a small call's launches leave room for)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -130,11 +131,18 @@ IMPL_TENSOR_CORE, IMPL_CUDA_CORE, IMPL_TENSOR_CORE_FP32_HEAD_SUM = 0, 1, 2
 
 
 def _opts(guard_len, pool, dbg_cand, dbg_scores, dbg_cand_scores, workspace, impl=0, rows=None, W=0, cand_in=None) -> pivot_opts:
-    p = lambda t: None if t is None else t.data_ptr()
     r0, r1 = (0, 0) if rows is None else rows
+    if dbg_cand is None and dbg_scores is None and dbg_cand_scores is None and workspace is None and cand_in is None:
+        return pivot_opts(-1 if guard_len is None else guard_len, pool, None, None, None, None, 0, impl, r0, r1, W, None)
+    p = lambda t: None if t is None else t.data_ptr()
     return pivot_opts(-1 if guard_len is None else guard_len, pool, p(dbg_cand), p(dbg_scores),
                       p(dbg_cand_scores), p(workspace), 0 if workspace is None else workspace.numel(), impl,
                       r0, r1, W, p(cand_in))
+
+
+@functools.lru_cache(maxsize=256)            # arithmetic on the sizes: a serving loop asks for the same ones every step
+def _workspace_bytes(device: int, *sizes: int) -> int:
+    return int((lib.pivot_workspace_bytes if len(sizes) == 4 else lib.pivot_decode_workspace_bytes)(*sizes))
 
 
 def pivot_workspace_bytes(rows: int, n_groups: int, c: int, k: int) -> int:
@@ -158,9 +166,9 @@ def pivot_decode_workspace_bytes(B: int, Lmax: int, g: int, c: int, k: int) -> i
 
 def ensure_workspace(rows: int, n_groups: int, c: int, k: int, device="cuda", need: int | None = None) -> torch.Tensor:
     """Allocates (or reuses) a registered workspace large enough for these sizes."""
-    need = pivot_workspace_bytes(rows, n_groups, c, k) if need is None else need
-    dev = torch.device(device)
+    dev = device if isinstance(device, torch.device) else torch.device(device)
     idx = dev.index if dev.index is not None else torch.cuda.current_device()
+    need = _workspace_bytes(idx, rows, n_groups, c, k) if need is None else need
     cur = _workspaces.get(idx)
     if cur is None or cur.numel() < need:
         with torch.cuda.device(idx):
@@ -239,7 +247,7 @@ def pivot_index_decode(q, w, kcache, pos0, B, Lmax, H_I, d, g, c, k, mode, out_i
     assert out_idx.numel() >= B * g * k
     assert cand_in is None or (cand_in.dtype == torch.int32 and cand_in.is_contiguous() and cand_in.numel() >= B * c)
     if workspace is None:
-        ensure_workspace(B * g, B, c, k, q.device, need=pivot_decode_workspace_bytes(B, Lmax, g, c, k))
+        ensure_workspace(B * g, B, c, k, q.device, need=_workspace_bytes(q.device.index, B, Lmax, g, c, k))
     o = _opts(guard_len, pool, dbg_cand, dbg_scores, dbg_cand_scores, workspace, impl, W=W, cand_in=cand_in)
     _check(lib.pivot_index_decode_ex(C.byref(tq), w.data_ptr(), C.byref(tk), pos0.data_ptr(), B, Lmax,
                                      H_I, d, g, c, k, mode, out_idx.data_ptr(), _stream(stream), C.byref(o)))
@@ -254,7 +262,7 @@ def pivot_index_decode_paged(q, w, kpages, block_table, pos0, B, max_pages, n_pa
     assert block_table.dtype == torch.int32 and block_table.is_contiguous() and block_table.numel() >= B * max_pages
     assert out_idx.numel() >= B * g * k
     if workspace is None:
-        ensure_workspace(B * g, B, c, k, q.device, need=pivot_decode_workspace_bytes(B, max_pages * 128, g, c, k))
+        ensure_workspace(B * g, B, c, k, q.device, need=_workspace_bytes(q.device.index, B, max_pages * 128, g, c, k))
     o = _opts(None, pool, dbg_cand, dbg_scores, dbg_cand_scores, workspace, impl, W=W)
     _check(lib.pivot_index_decode_paged(C.byref(tq), w.data_ptr(), C.byref(tk), block_table.data_ptr(),
                                         pos0.data_ptr(), B, max_pages, n_pages, H_I, d, g, c, k, mode,
@@ -269,7 +277,7 @@ def dense_index_decode(q, w, kcache, pos0, B, Lmax, H_I, d, g, k, out_idx, strea
     assert w.dtype == torch.float32 and out_idx.dtype == torch.int32 and pos0.dtype == torch.int32
     assert out_idx.numel() >= B * g * k
     if workspace is None:
-        ensure_workspace(B * g, B * g, k, k, q.device, need=pivot_decode_workspace_bytes(B * g, Lmax, 1, k, k))
+        ensure_workspace(B * g, B * g, k, k, q.device, need=_workspace_bytes(q.device.index, B * g, Lmax, 1, k, k))
     o = _opts(None, POOL_MEAN, None, dbg_scores, None, workspace, impl)
     _check(lib.dense_index_decode_ex(C.byref(tq), w.data_ptr(), C.byref(tk), pos0.data_ptr(), B, Lmax, H_I, d, g, k,
                                      out_idx.data_ptr(), _stream(stream), C.byref(o)))
