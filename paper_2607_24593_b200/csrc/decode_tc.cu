@@ -39,7 +39,7 @@ namespace {
 
 namespace cg = cooperative_groups;
 constexpr int TILE_KEYS = 128;
-constexpr int DKS_SLOTS = 14;
+constexpr int DKS_SLOTS = 16;           // key-scale ring (a power of two: the slot is a mask away)
 constexpr int DHIST_BITS = 13;          // histogram digit: top 13 bits of the score key (16 bins per octave)
 constexpr int DHIST = 1 << DHIST_BITS;
 constexpr int D_N = kHeads;             // MMA N: one proxy
@@ -76,10 +76,10 @@ constexpr size_t dsmem_bytes() {
 // Walks the global tile index space: sequence b owns tiles [prefix[b], prefix[b+1]).
 struct TileWalk {
   const int* prefix;
-  int B, b;
-  __device__ TileWalk(const int* p, int nb) : prefix(p), B(nb), b(0) {}
+  int B, b, end;                 // end: first tile past sequence b
+  __device__ TileWalk(const int* p, int nb) : prefix(p), B(nb), b(0), end(p[1]) {}
   __device__ __forceinline__ int seq_of(int g) {     // g non-decreasing between calls
-    while (b + 1 < B && g >= prefix[b + 1]) ++b;
+    while (b + 1 < B && g >= end) { ++b; end = prefix[b + 1]; }
     return b;
   }
 };
@@ -137,10 +137,13 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
       uint32_t it = 0, blk = 0;
       // keys are read once a step: they give way in L2 before the scores, which the select reads next
       const uint64_t once = ptx::l2_evict_first();
+      // this sequence's: what a tile costs this thread is on the stream's critical path (tile by tile it took as
+      // long as the tile's bytes), so nothing is looked up per tile that changes per sequence
+      const int32_t* pages = nullptr;
+      int first = 0, k_row0 = 0;
       PIVOT_PROF_DO(long long pwait = 0;)
       for (int g = g_lo; g < g_hi; ++g, ++it) {
         const int b = tw.seq_of(g);
-        const int t = g - tile_prefix[b];
         if (b != cur_b) {             // new sequence: its proxy becomes the MMA's B operand
           const int qb = blk & 1;
           if (!ptx::mbar_wait(&ct.q_empty[qb], ((blk >> 1) & 1) ^ 1, abort_flag, 64)) break;
@@ -150,12 +153,15 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
                              &ct.q_full[qb]);
           ++blk;
           cur_b = b;
+          pages = prox[b].pages;
+          k_row0 = prox[b].k_row0;
+          first = tile_prefix[b];
         }
         // Row of the tile inside the key tensor.  Paged cache: the sequence's block table names
         // the pool page (a page outside the pool reads as zero fill, like any out-of-range box).
-        const int32_t* pages = prox[b].pages;
+        const int t = g - first;
         (void)PIVOT_BOUNDS(t * TILE_KEYS < Lmax, status);              // checked build: the tile lies inside the sequence's rows
-        const int krow = pages ? __ldg(pages + t) * TILE_KEYS : prox[b].k_row0 + t * TILE_KEYS;
+        const int krow = pages ? __ldg(pages + t) * TILE_KEYS : k_row0 + t * TILE_KEYS;
         const int s = it % C::STAGES;
         PIVOT_PROF_DO(const long long pw0 = clock64();)
         if (!ptx::mbar_wait(&ct.empty[s], ((it / C::STAGES) & 1) ^ 1, abort_flag, 64)) break;
@@ -178,6 +184,7 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
       int cur_b = -1, qb = 0;
       uint32_t it = 0, blk = 0;
       bool ok = true;
+      const uint64_t k_desc = ptx::smem_desc_sw128(ptx::smem_u32(kring)), q_desc = ptx::smem_desc_sw128(ptx::smem_u32(qbuf));
       PIVOT_PROF_DO(long long pw[3] = {0, 0, 0}; const long long pstart = clock64();)
 #ifdef PIVOT_PROF
 #define PW(i, ...) { const long long t_ = clock64(); __VA_ARGS__; pw[i] += clock64() - t_; }
@@ -201,16 +208,14 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
         PW(2, ok = ptx::mbar_wait(&ct.full[s], (it / C::STAGES) & 1, abort_flag, 32))
         if (!ok) break;
         ptx::tc_fence_after();
-        const uint32_t k_addr = ptx::smem_u32(kring + s * C::STAGE_BYTES);
-        const uint32_t q_addr = ptx::smem_u32(qbuf + qb * C::QBUF_BYTES);
+        const uint64_t kd = k_desc + (uint32_t)((s * C::STAGE_BYTES) >> 4), qd = q_desc + (uint32_t)((qb * C::QBUF_BYTES) >> 4);
         const uint32_t d_tmem = tmem_base + buf * D_N;
 #pragma unroll
         for (int h = 0; h < C::KHALVES; ++h)
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks)
-            ptx::tc_mma<C::FP8>(d_tmem, ptx::smem_desc_sw128(k_addr + h * C::HALF_TILE_BYTES + ks * 32),
-                                ptx::smem_desc_sw128(q_addr + h * C::QHALF_BYTES + ks * 32), C::IDESC,
-                                (h | ks) ? 1u : 0u);
+            ptx::tc_mma<C::FP8>(d_tmem, kd + ((h * C::HALF_TILE_BYTES + ks * 32) >> 4), qd + ((h * C::QHALF_BYTES + ks * 32) >> 4),
+                                C::IDESC, (h | ks) ? 1u : 0u);
         ptx::tc_commit(&ct.empty[s]);
         ptx::tc_commit(&ct.tmem_full[buf]);
       }
@@ -233,7 +238,7 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     const int key_in_tile = lq * 32 + lane;
     const Team tm{tt, 128, 1 + set};
     TileWalk tw(tile_prefix, B);
-    int cur_b = -1, n_vis = 0;
+    int cur_b = -1, n_vis = 0, first = 0;
     auto flush_hist = [&](int b) {
       tm.sync();
       for (int i = tt; i < DHIST; i += 128) {
@@ -245,10 +250,10 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     for (int g = g_lo + set; g < g_hi; g += 2) {
       const uint32_t it = (uint32_t)(g - g_lo);
       const int b = tw.seq_of(g);
-      const int t = g - tile_prefix[b];
       if (b != cur_b) {
         if (cur_b >= 0) flush_hist(cur_b);
         cur_b = b;
+        first = tile_prefix[b];
         n_vis = prox[b].n_vis;
         tm.sync();
         if (tt < kHeads) ct.w[set][tt] = prox[b].w[tt];      // proxy gate
@@ -276,7 +281,7 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
       ptx::relu_dot32(v1, &ct.w[set][32], acc);
       float sv = ptx::relu_dot_sum(acc);
       if (C::FP8) sv *= ksv;
-      const int s_key = t * TILE_KEYS + key_in_tile;
+      const int s_key = (g - first) * TILE_KEYS + key_in_tile;
       if (s_key < n_vis && PIVOT_BOUNDS(s_key < Lmax, status)) {
         scores[(size_t)b * Lmax + s_key] = sv;
         atomicAdd(&ct.hist[set][score_to_key(sv) >> (32 - DHIST_BITS)], 1u);
