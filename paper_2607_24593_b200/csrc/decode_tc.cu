@@ -583,26 +583,9 @@ decode_prepare_kernel(DecodePlan p, RowDesc* rows, GroupDesc* plan_groups, uint3
   for (int i = tid; i < DHIST; i += blockDim.x) ghist[(size_t)b * DHIST + i] = 0u;
   __shared__ int seq_ok;
   __shared__ int wsum[32];
-  if (tid == 0) seq_ok = plan_decode_sequence(p, b, rows, plan_groups) ? 1 : 0;
-  if (b == 0) {                    // the step's status word and row counter start here (p.status is not set)
-    bool bad = false;
-    for (int bb = tid; bb < B; bb += blockDim.x) bad |= decode_bad_pos(p, p.pos0[bb / p.kv_share]);
-    const int any = __syncthreads_or(bad);
-    if (tid < 2) status[tid] = tid == 0 && any ? DEV_BAD_POS : 0;
-  }
-  // ---- tiles of the sequences before this one
-  int part = 0;
-  for (int bb = tid; bb < b; bb += blockDim.x) part += decode_live_tiles(p, bb);
-  part = __reduce_add_sync(0xffffffffu, part);
-  if (lane == 0) wsum[wid] = part;
-  __syncthreads();                                 // also: the descriptors thread 0 wrote are visible to the block
-  if (tid == 0) {
-    int before = 0;
-    for (int i = 0; i < 32; ++i) before += wsum[i];
-    tile_prefix[b] = before;
-    if (b == B - 1) tile_prefix[B] = before + decode_live_tiles(p, b);
-  }
-  if (!seq_ok) fill_decode_rows_empty(p, b, tid, blockDim.x);     // pos0 outside the cache: rows of -1
+  // the plan (the last warp's first thread: a chain of loads and descriptor stores) runs beside the proxy, which
+  // takes the first sixteen warps (e4m3) or a unit of every warp (bf16)
+  if (tid == 31 * 32) seq_ok = plan_decode_sequence(p, b, rows, plan_groups) ? 1 : 0;
   if (p.raw_q) {
     raw_query_gates(p, b, tid, blockDim.x);
   } else {
@@ -615,6 +598,25 @@ decode_prepare_kernel(DecodePlan p, RowDesc* rows, GroupDesc* plan_groups, uint3
         proxy_build_unit<DT_BF16>(p.q, p.qscale, p.w, p.proxy_q, p.proxy_w, b * g, g, b, u, pool, lane);
     }
   }
+  if (b == 0) {                    // the step's status word and row counter start here (p.status is not set)
+    bool bad = false;
+    for (int bb = tid; bb < B; bb += blockDim.x) bad |= decode_bad_pos(p, p.pos0[bb / p.kv_share]);
+    const int any = __syncthreads_or(bad);
+    if (tid < 2) status[tid] = tid == 0 && any ? DEV_BAD_POS : 0;
+  }
+  // ---- tiles of the sequences before this one
+  int part = 0;
+  for (int bb = tid; bb < b; bb += blockDim.x) part += decode_live_tiles(p, bb);
+  part = __reduce_add_sync(0xffffffffu, part);
+  if (lane == 0) wsum[wid] = part;
+  __syncthreads();                                 // also: the plan's descriptors are visible to the block
+  if (tid == 0) {
+    int before = 0;
+    for (int i = 0; i < 32; ++i) before += wsum[i];
+    tile_prefix[b] = before;
+    if (b == B - 1) tile_prefix[B] = before + decode_live_tiles(p, b);
+  }
+  if (!seq_ok) fill_decode_rows_empty(p, b, tid, blockDim.x);     // pos0 outside the cache: rows of -1
   if (mode != 1) return;
   // Refine: split every (sequence, member chunk) into candidate chunks so all SMs re-score,
   // each leaving packed entries; one entry list per query for the final top-k.
