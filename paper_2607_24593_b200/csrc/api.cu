@@ -208,6 +208,32 @@ int resolve_ws(const pivot_opts* o, size_t need, void** ws) {
   return PIVOT_OK;
 }
 
+// Parts that a chunk's scan is cut into.  Its row blocks are few and of nearly equal length (a chunk at the end of
+// a long prompt), so whole blocks leave SMs idle in the last round, or most SMs in the only one: 512 blocks on 148
+// SMs take four rounds where 3.46 would do, 64 blocks leave 84 SMs without any.  The cost of S parts, in tiles:
+// rounds of part blocks, each with its own start -- some sixteen tiles' time between two blocks, and K / 128 tiles
+// before a threshold has formed -- and the merge of the parts' selections, 2 SMs' worth of rows at a time (14 us a
+// round of 2 x 4096 entries).  fp8, c = 4096: 8192 rows at the end of 256K 5.9 ms in one part, 5.3 + 0.1 in two; 1024 rows
+// at the end of 128K 981 -> 610 us; 6000 rows at the end of 64K stay whole (1.64 ms; in three parts 2.07).
+// Calls whose blocks differ in length (a whole request) are balanced by the deal.
+int choose_split(int n_proxy, int first_pos, int last_pos, int K, int sms, size_t room, int slots) {
+  if (first_pos < last_pos / 2) return 1;
+  const int nb = (n_proxy + 3) / 4;
+  const double tiles = last_pos / 128.0;
+  int best = 1;
+  double least = 0.0;
+  for (int s = 1; s <= 8; ++s) {
+    if (s > 1) {
+      if (first_pos / s < 4 * K || s * K > kMaxMerge || nb * 4 * s > slots) break;
+      if (align_up((size_t)n_proxy * sizeof(MergeRow)) + 2 * align_up((size_t)n_proxy * s * K * 4) > room) break;
+    }
+    double cost = (double)((s * nb + sms - 1) / sms) * (tiles / s + 16.0 + K / 128.0);
+    if (s > 1) cost += (double)((n_proxy + 2 * sms - 1) / (2 * sms)) * (4.0 + 14.0 * s * K / 8192.0);
+    if (s == 1 || cost < 0.97 * least) { least = cost; best = s; }
+  }
+  return best;
+}
+
 // Requests cu[0] .. cu[n] of a packed batch (host array; one request: {0, L}), each indexed on its own.
 // All of them go through one prepare, one scan and one re-score launch.
 int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kcache, const int32_t* cu, int n, int g,
@@ -263,6 +289,23 @@ int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kcach
   p.cand_score = (o && o->dbg_cand_scores) ? o->dbg_cand_scores + (size_t)pg0 * c : nullptr;
   p.out = out_idx; p.out_score = o ? o->dbg_scores : nullptr;
 
+  if (p.n_req == 1 && p.req[0].n_dense == 0 && p.n_proxy > 0 && !(o && o->impl == 1)) {
+    // the part lists take candidate sets that this call has no groups for (a chunk's workspace is the request's)
+    const PrefillReq& q0 = p.req[0];
+    const int K = mode == PIVOT_REFINE ? c : k;
+    Carve cv((char*)ws.cand);
+    if (p.cand == ws.cand) cv.take<int32_t>((size_t)p.n_proxy * c);
+    const size_t have = (size_t)ws_groups * c * sizeof(int32_t);
+    p.split = choose_split(p.n_proxy, q0.first_group * g, (q0.first_group + p.n_proxy - 1) * g, K, sm_count(),
+                           have > cv.off ? have - cv.off : 0, ws_rows + ws_groups);
+    if (p.split > 1) {
+      p.merges = cv.take<MergeRow>(p.n_proxy);
+      p.part_pos = cv.take<int32_t>((size_t)p.n_proxy * p.split * K);
+      p.part_score = cv.take<float>((size_t)p.n_proxy * p.split * K);
+      p.n_slots = (p.n_slots + 3) / 4 * 4;
+    }
+  }
+
   int rc;
   mark(0, st);
   if ((rc = check_cuda(launch_prepare_prefill(p, ws.rows, ws.groups, st)))) return rc;
@@ -273,7 +316,10 @@ int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kcach
   } else {
     ScanOperands op{kcache->data, tokens, kcache->scale, q->data, tokens, ws.proxy_q, p.n_proxy, q->dtype};
     op.k_stride = p.k_stride;
-    if ((rc = check_cuda(launch_scan_tc(op, ws.rows, p.n_slots, 4, tc_scratch(ws), sm_count(), st, o && o->impl == 2, true))))
+    if ((rc = check_cuda(launch_scan_tc(op, ws.rows, p.n_slots * p.split, 4, tc_scratch(ws), sm_count(), st, o && o->impl == 2, true))))
+      return rc;
+    if (p.split > 1 &&
+        (rc = check_cuda(launch_merge_parts(p.merges, p.n_proxy, p.split * (mode == PIVOT_REFINE ? c : k), st))))
       return rc;
   }
   mark(3, st);

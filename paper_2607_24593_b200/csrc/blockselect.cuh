@@ -209,9 +209,9 @@ __device__ __forceinline__ entry_t blk_find_cut_regs(BlkSelSmem& sm, const entry
   return lo;
 }
 
-// blk_emit_topk for a list of at most U * 1024 entries, in list order, warp by warp.
-template <int U>
-__device__ __forceinline__ void blk_emit_topk_regs(BlkSelSmem& sm, const entry_t* list, int n, int K, int32_t* out,
+// blk_emit_topk for at most U * 1024 entries (entry i = list(i)), in list order, warp by warp.
+template <int U, typename List>
+__device__ __forceinline__ void blk_emit_topk_regs(BlkSelSmem& sm, List list, int n, int K, int32_t* out,
                                                    float* out_score, int copies, int stride) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   entry_t x[U];
@@ -219,7 +219,7 @@ __device__ __forceinline__ void blk_emit_topk_regs(BlkSelSmem& sm, const entry_t
 #pragma unroll
   for (int j = 0; j < U; ++j) {
     const int i = wid * (32 * U) + j * 32 + lane;
-    const entry_t e = i < n ? list[i] : kPadEntry;
+    const entry_t e = i < n ? list(i) : kPadEntry;
     x[j] = entry_pos(e) >= 0 ? e : kPadEntry;
   }
   const entry_t cut = n > K ? blk_find_cut_regs<U>(sm, x, K) : 1ull;

@@ -118,7 +118,8 @@ struct RowDesc {
   int out_stride;
   int q_map;            // which query tensor map holds q: 0 raw queries, 1 proxies
   int q_row;            // query row (units of H x d) inside that tensor
-  int k_row0;           // first row of this sequence's keys inside the key-cache tensor
+  int k_row0;           // first row of this sequence's keys inside the key-cache tensor (of this part's, if the prefix
+                        // is scanned in parts: n_vis and the selected positions count from it)
   // Paged key cache (decode): key tile t of this row is pool page pages[t]; nullptr = contiguous.
   const int32_t* pages = nullptr;
 };

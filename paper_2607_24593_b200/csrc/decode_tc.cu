@@ -504,8 +504,9 @@ decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __re
     int32_t* const out = rd.out + (K - rest);
     float* const outs = rd.out_score ? rd.out_score + (K - rest) : nullptr;
     const int ne = need > 0 ? n_edge : 0;
-    if (ne <= 2 * kBlk) blk_emit_topk_regs<2>(sm.blk, sm.edge, ne, rest, out, outs, rd.out_rows, rd.out_stride);
-    else blk_emit_topk_regs<4>(sm.blk, sm.edge, ne, rest, out, outs, rd.out_rows, rd.out_stride);
+    auto list = [&](int i) { return sm.edge[i]; };
+    if (ne <= 2 * kBlk) blk_emit_topk_regs<2>(sm.blk, list, ne, rest, out, outs, rd.out_rows, rd.out_stride);
+    else blk_emit_topk_regs<4>(sm.blk, list, ne, rest, out, outs, rd.out_rows, rd.out_stride);
   }
   PIVOT_PROF_DO(__syncthreads(); if (tid == 0) {
     pt[4] = clock64();
@@ -527,12 +528,33 @@ __global__ void __launch_bounds__(kBlk, PER_SM) entries_topk_kernel(const EntryL
   const EntryList el = lists[blockIdx.x];
   if (el.K <= 0) return;
   // by the entries a thread holds: the list is read once
-  const entry_t* list = (const entry_t*)el.list;
+  auto list = [&](int i) { return ((const entry_t*)el.list)[i]; };
   if (el.n <= 2 * kBlk) blk_emit_topk_regs<2>(sm, list, el.n, el.K, el.out, el.out_score, 1, el.K);
   else if (el.n <= 5 * kBlk) blk_emit_topk_regs<5>(sm, list, el.n, el.K, el.out, el.out_score, 1, el.K);
   else blk_emit_topk_regs<9>(sm, list, el.n, el.K, el.out, el.out_score, 1, el.K);
 }
 static_assert(8192 + kDecodeWinMax <= 9 * kBlk, "largest candidate budget plus window slots");
+
+// Top-K of a scan row whose prefix was scanned in parts, one block per row.  Bound by its chain of loads and
+// barriers: two blocks per SM where the registers allow it (2048 rows of 2 x 4096 entries: 104 us against 155).
+template <int U>
+__global__ void __launch_bounds__(kBlk, U <= 8 ? 2 : 1) merge_parts_kernel(const MergeRow* __restrict__ rows) {
+  __shared__ BlkSelSmem sm;
+  __shared__ int part0[8];               // first key of each part
+  ptx::grid_launch_dependents();
+  ptx::grid_dependency_wait();            // the scan's part lists
+  const MergeRow m = rows[blockIdx.x];
+  if ((int)threadIdx.x < m.parts) part0[threadIdx.x] = (int)((long long)m.tiles * threadIdx.x / m.parts) * TILE_KEYS;
+  __syncthreads();
+  auto list = [&](int i) {
+    const int32_t p = m.pos[i];
+    const float s = m.score[i];
+    int first = 0;                                     // (a few compares: a division per entry costs more than the rest)
+    for (int h = 1; h < m.parts; ++h) first = i >= h * m.K ? part0[h] : first;
+    return p < 0 ? kPadEntry : make_entry(score_to_key(s), first + p);
+  };
+  blk_emit_topk_regs<U>(sm, list, m.parts * m.K, m.K, m.out, m.out_score, m.out_rows, m.out_stride);
+}
 
 // Union of candidate lists -> packed entries -> exact top-K, one block.
 __global__ void __launch_bounds__(kBlk, 1)
@@ -729,6 +751,13 @@ size_t decode_fast_bytes(int B, int Lmax, int g, int c) {
   return up(B * Ls * 4) + up((size_t)B * DHIST * 4) + up((size_t)(B + 1) * 4) +
          up((size_t)B * mc * (ncc + 1) * sizeof(GroupDesc)) + up((size_t)B * g * sizeof(EntryList)) +
          up((size_t)B * kDecodeWinMax * 4) + up((size_t)B * g * (c + kDecodeWinMax) * 8);
+}
+
+cudaError_t launch_merge_parts(const MergeRow* rows, int n_rows, int n_max, cudaStream_t st) {
+  if (n_max > kMaxMerge) return cudaErrorInvalidValue;
+  ++launch_counter();
+  return launch_kernel(n_max <= 4 * kBlk ? merge_parts_kernel<4> : n_max <= 8 * kBlk ? merge_parts_kernel<8> : merge_parts_kernel<16>,
+                       dim3(n_rows), dim3(kBlk), 0, st, true, rows);
 }
 
 cudaError_t launch_merge_topk(const float* scores, const int32_t* idx, int n_seg, int seg_len, const int32_t* seg_offset,

@@ -71,6 +71,16 @@ struct PrefillReq {
 };
 constexpr int kMaxPlanReqs = 64;
 
+// One scan row whose prefix was scanned in parts: the top-K of every part, of which merge_parts takes the top-K.
+struct MergeRow {
+  const int32_t* pos;   // [parts, K] inside the part, which starts at key tile tiles * part / parts; -1: empty
+  const float* score;   // [parts, K]
+  int parts, tiles, K;
+  int32_t* out; float* out_score;
+  int out_rows, out_stride;
+};
+constexpr int kMaxMerge = 16384;      // entries (parts x K) merge_parts takes per row
+
 // Geometry of a prefill-shaped call (by value to the planner kernel).
 struct PrefillPlan {
   const void* q; const float* w; const float* qscale;   // raw per-query operands
@@ -87,6 +97,11 @@ struct PrefillPlan {
   int n_slots = 0;      // scan-row slots: the rows of all requests, each request padded to whole blocks of four if there are several
   int n_proxy = 0;      // proxies of all requests
   int n_req = 0;
+  // split > 1 (one request, no dense rows): every block of scan rows becomes `split` blocks over consecutive parts
+  // of the prefix, n_slots (a multiple of four) counts the rows before that
+  int split = 1;
+  int32_t* part_pos = nullptr; float* part_score = nullptr;     // [n_proxy, split, K]
+  MergeRow* merges = nullptr;                                   // [n_proxy]
   PrefillReq req[kMaxPlanReqs];
 };
 
@@ -154,6 +169,8 @@ cudaError_t launch_scan_tc(const ScanOperands& op, const RowDesc* rows, int n_ro
 cudaError_t launch_refine_tc(const void* q, int q_rows, int dtype, const GroupDesc* groups, int n_groups,
                              const ScanScratch& s, int sms, cudaStream_t st, bool fp32_head_sum = false,
                              bool chunked = false, int max_cand = 0, bool overlap_prev = false);
+
+cudaError_t launch_merge_parts(const MergeRow* rows, int n_rows, int n_max, cudaStream_t st);
 
 // Decode fast path: key-tile-split scan -> per-sequence select -> chunked re-score -> top-k.
 struct DecodeFast {

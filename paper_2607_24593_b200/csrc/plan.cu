@@ -161,11 +161,34 @@ prepare_prefill_kernel(const __grid_constant__ PrefillPlan p, RowDesc* rows, Gro
       r.out = nullptr; r.out_score = nullptr; r.out_rows = 0; r.out_stride = 0;
       r.q_map = 0; r.q_row = q.tok0;
     }
+    if (p.split > 1) {
+      // The block's key tiles in p.split equal runs, each a block of its own; what the parts select goes to the
+      // merge.  (The runs are the block's, so that its four rows keep sharing one key stream.)
+      const int last = row_pos(q, p.g, min(jb * 4 + 3, q.n_proxy - 1));
+      const int tiles = (max(p.W > 0 ? last - p.W + 1 : last + 1, 0) + 127) / 128;
+      const RowDesc whole = r;
+      const int pr = q.proxy0 + j;
+      for (int h = 0; h < p.split; ++h) {
+        const int lo = (int)((long long)tiles * h / p.split) * 128, hi = (int)((long long)tiles * (h + 1) / p.split) * 128;
+        r.k_row0 = whole.k_row0 + lo;
+        r.n_vis = min(max(whole.n_vis - lo, 0), hi - lo);
+        if (whole.K > 0) {
+          r.out = p.part_pos + ((size_t)pr * p.split + h) * whole.K;
+          r.out_score = p.part_score + ((size_t)pr * p.split + h) * whole.K;
+          r.out_rows = 1;
+        }
+        rows[(jb * p.split + h) * 4 + (j & 3)] = r;
+      }
+      if (whole.K > 0)
+        p.merges[pr] = MergeRow{p.part_pos + (size_t)pr * p.split * whole.K, p.part_score + (size_t)pr * p.split * whole.K,
+                                p.split, tiles, whole.K, whole.out, whole.out_score, whole.out_rows, whole.out_stride};
+    } else {         // (a split call has no rows without a choice)
     if (p.skip_trivial && r.K > 0 && r.n_vis <= r.K && !r.out_score) {
       fill[threadIdx.x] = FillRow{r.out, r.n_vis, r.K, r.out_rows, r.out_stride};
       r.K = 0;
     }
     rows[slot] = r;
+    }
   }
   __syncthreads();
   for (int s = warp; s < kPrepSlots; s += kPrepThreads / 32) {

@@ -924,3 +924,31 @@ def test_prefill_varlen_batches(pv, gu, g, mode, W, guard):
     if guard is None:                     # rows below the guardrail that see no more keys than they select
         for t in range(k):
             assert np.array_equal(one[cu[4] + t][k - t - 1:], np.arange(t + 1))
+
+
+@pytest.mark.parametrize("dtype,g,mode,W,rows,c,k", [
+    ("fp8", 4, 1, 0, (11904, 12288), 512, 256),       # 24 blocks: many parts
+    ("fp8", 8, 0, 0, (11000, 12289), 256, 128),       # ragged last group, Reuse copies
+    ("bf16", 4, 1, 4, (11200, 12289), 384, 200),      # window, odd budgets
+    ("fp8", 2, 1, 0, (10700, 12288), 640, 640),       # a round and a third of blocks, c = k
+])
+def test_chunk_scanned_in_parts(pv, gu, dtype, g, mode, W, rows, c, k):
+    """A chunk whose blocks leave the last round of SMs idle is scanned in parts of the prefix and merged: the
+    selection is the whole call's, row for row (the same scores enter the same order)."""
+    L = 12289
+    x = inputs.make_prefill(L, dtype=dtype, seed=91)
+    kw = dict(q_scale=x.qscale.cuda(), k_scale=x.kscale.cuda()) if dtype == "fp8" else {}
+    q, w, kk = x.q.cuda(), x.w.cuda(), x.k.cuda()
+    r1 = rows[1] if rows[1] % g == 0 else L
+    whole = torch.full((L, k), -7, dtype=torch.int32, device="cuda")
+    part = torch.full((L, k), -7, dtype=torch.int32, device="cuda")
+    pv.pivot_index_prefill(q, w, kk, L, 64, 128, g, c, k, mode, whole, W=W, **kw)
+    pv.lib.pivot_launch_count_reset()
+    pv.pivot_index_prefill(q, w, kk, L, 64, 128, g, c, k, mode, part, W=W, rows=(rows[0], r1), **kw)
+    launches = pv.lib.pivot_launch_count_reset()
+    torch.cuda.synchronize()
+    assert pv.pivot_device_status() == 0
+    assert launches == (4 if mode == 1 else 3), "the merge of the parts did not run"
+    a, b = whole[rows[0]:r1].cpu().numpy(), part[rows[0]:r1].cpu().numpy()
+    assert np.array_equal(_sorted_rows(a), _sorted_rows(b))
+    assert (part[:rows[0]] == -7).all() and (part[r1:] == -7).all()
