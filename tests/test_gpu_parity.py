@@ -952,3 +952,26 @@ def test_chunk_scanned_in_parts(pv, gu, dtype, g, mode, W, rows, c, k):
     a, b = whole[rows[0]:r1].cpu().numpy(), part[rows[0]:r1].cpu().numpy()
     assert np.array_equal(_sorted_rows(a), _sorted_rows(b))
     assert (part[:rows[0]] == -7).all() and (part[r1:] == -7).all()
+
+
+@pytest.mark.parametrize("B,dtype,mode", [(37, "fp8", 1), (38, "bf16", 1), (74, "fp8", 0), (80, "fp8", 1)])
+def test_decode_batch_sizes_select_alike(pv, gu, B, dtype, mode):
+    """The select's cluster size and the final top-k's blocks per SM follow the batch: a batch on either side of each
+    bound gives what its sequences give in calls of eight."""
+    g, c, k = 2, 384, 200
+    x = inputs.make_decode(B, g, 500, 2500, dtype=dtype, seed=17)
+    d = gu.to_cuda(x)
+    Lmax = x.k.shape[1]
+    cut = lambda t, a, b: None if t is None else t[a:b]
+    out = torch.full((B, g, k), -7, dtype=torch.int32, device="cuda")
+    pv.pivot_index_decode(d["q"], d["w"], d["k"], d["pos0"], B, Lmax, 64, 128, g, c, k, mode, out, q_scale=d["qscale"],
+                          k_scale=d["kscale"])
+    ref = torch.full((B, g, k), -7, dtype=torch.int32, device="cuda")
+    for a in range(0, B, 8):
+        b = min(a + 8, B)
+        pv.pivot_index_decode(d["q"][a:b], d["w"][a:b], d["k"][a:b], d["pos0"][a:b], b - a, Lmax, 64, 128, g, c, k, mode, ref[a:b],
+                              q_scale=cut(d["qscale"], a, b), k_scale=cut(d["kscale"], a, b))
+    torch.cuda.synchronize()
+    assert pv.pivot_device_status() == 0
+    same = _sorted_rows(out.view(-1, k).cpu().numpy()) == _sorted_rows(ref.view(-1, k).cpu().numpy())
+    assert same.all()
