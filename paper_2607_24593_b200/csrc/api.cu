@@ -216,15 +216,17 @@ int resolve_ws(const pivot_opts* o, size_t need, void** ws) {
 // round of 2 x 4096 entries).  fp8, c = 4096: 8192 rows at the end of 256K 5.9 ms in one part, 5.3 + 0.1 in two; 1024 rows
 // at the end of 128K 981 -> 610 us; 6000 rows at the end of 64K stay whole (1.64 ms; in three parts 2.07).
 // Calls whose blocks differ in length (a whole request) are balanced by the deal.
-int choose_split(int n_proxy, int first_pos, int last_pos, int K, int sms, size_t room, int slots) {
-  if (first_pos < last_pos / 2) return 1;
+// first_vis, last_vis: keys that the first and the last scan row see.  Every part of every block has a key tile of
+// its own (first_vis / 128 of them at least): a part without one would not be scanned and its list never written.
+int choose_split(int n_proxy, int first_vis, int last_vis, int K, int sms, size_t room, int slots) {
+  if (first_vis < last_vis / 2) return 1;
   const int nb = (n_proxy + 3) / 4;
-  const double tiles = last_pos / 128.0;
+  const double tiles = last_vis / 128.0;
   int best = 1;
   double least = 0.0;
   for (int s = 1; s <= 8; ++s) {
     if (s > 1) {
-      if (first_pos / s < 4 * K || s * K > kMaxMerge || nb * 4 * s > slots) break;
+      if (first_vis / s < 4 * K || first_vis / 128 < s || s * K > kMaxMerge || nb * 4 * s > slots) break;
       if (align_up((size_t)n_proxy * sizeof(MergeRow)) + 2 * align_up((size_t)n_proxy * s * K * 4) > room) break;
     }
     double cost = (double)((s * nb + sms - 1) / sms) * (tiles / s + 16.0 + K / 128.0);
@@ -296,8 +298,9 @@ int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kcach
     Carve cv((char*)ws.cand);
     if (p.cand == ws.cand) cv.take<int32_t>((size_t)p.n_proxy * c);
     const size_t have = (size_t)ws_groups * c * sizeof(int32_t);
-    p.split = choose_split(p.n_proxy, q0.first_group * g, (q0.first_group + p.n_proxy - 1) * g, K, sm_count(),
-                           have > cv.off ? have - cv.off : 0, ws_rows + ws_groups);
+    const int unseen = W > 0 ? W - 1 : -1;            // a row at t0 sees t0 - unseen keys
+    p.split = choose_split(p.n_proxy, q0.first_group * g - unseen, (q0.first_group + p.n_proxy - 1) * g - unseen, K,
+                           sm_count(), have > cv.off ? have - cv.off : 0, ws_rows + ws_groups);
     if (p.split > 1) {
       p.merges = cv.take<MergeRow>(p.n_proxy);
       p.part_pos = cv.take<int32_t>((size_t)p.n_proxy * p.split * K);

@@ -1,0 +1,51 @@
+"""GPU checks of the edges of the product path: parts of short prefixes, rows that only pad a block, NaN
+and infinite keys, crowded boundary bins, the status word of a packed batch."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_24593_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pv():
+    from paper_2607_24593_b200 import binding
+    return binding
+
+
+def _sorted(out):
+    return torch.sort(out.reshape(-1, out.shape[-1]), dim=1).values.cpu().numpy()
+
+
+def _operands(x):
+    kw = {} if x.qscale is None else dict(q_scale=x.qscale.cuda(), k_scale=x.kscale.cuda())
+    return x.q.cuda(), x.w.cuda(), x.k.cuda(), kw
+
+
+@pytest.mark.parametrize("dtype,g,mode,W,L,row0,c,k", [
+    ("fp8", 4, 1, 0, 880, 832, 24, 24),
+    ("bf16", 4, 1, 0, 880, 832, 24, 24),
+    ("fp8", 4, 0, 0, 900, 644, 256, 16),
+    ("fp8", 4, 0, 1004, 1500, 1024, 1024, 64),
+    ("bf16", 4, 1, 0, 1003, 960, 16, 16),
+    ("fp8", 2, 0, 0, 1100, 1000, 16, 8),
+    ("fp8", 1, 0, 0, 300, 290, 2, 1),
+    ("bf16", 16, 1, 8, 1201, 1104, 40, 9),
+])
+def test_chunk_of_a_short_prefix_and_a_small_budget(pv, dtype, g, mode, W, L, row0, c, k):
+    """Small budgets allow many parts of a prefix of few key tiles: every part has to have a tile (one that has
+    none is never scanned, and its list would be whatever the workspace held).  The workspace starts full of
+    words that read as positions with large scores."""
+    x = inputs.make_prefill(L, dtype=dtype, seed=L + k)
+    q, w, kk, kw = _operands(x)
+    ws = torch.full((pv.pivot_workspace_bytes(L, (L + g - 1) // g, c, k),), 0x44, dtype=torch.uint8, device="cuda")
+    whole = torch.full((L, k), -7, dtype=torch.int32, device="cuda")
+    part = torch.full((L, k), -7, dtype=torch.int32, device="cuda")
+    pv.pivot_index_prefill(q, w, kk, L, 64, 128, g, c, k, mode, whole, W=W, **kw)
+    pv.pivot_index_prefill(q, w, kk, L, 64, 128, g, c, k, mode, part, W=W, rows=(row0, L), workspace=ws, **kw)
+    torch.cuda.synchronize()
+    assert pv.pivot_device_status() == 0
+    assert np.array_equal(_sorted(whole[row0:]), _sorted(part[row0:]))
+    assert (part[:row0] == -7).all()
