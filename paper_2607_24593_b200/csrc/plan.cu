@@ -155,11 +155,15 @@ prepare_prefill_kernel(const __grid_constant__ PrefillPlan p, RowDesc* rows, Gro
         const int chunks = (p.g + kMembersPerDesc - 1) / kMembersPerDesc;
         put_group_chunks(groups + (size_t)pr * chunks, gd, p.g, p.dtype);
       }
-    } else {               // padding of the request's last block: never live, reads a row that exists
+    } else {
+      // Padding of the request's last block: never live.  Its queries are still multiplied (the head sum of FP8 runs
+      // over the block's four rows at once, with zero gates for this one, and zero times NaN is NaN), so they are
+      // those of the block's last live row: any other row's may not have been written yet, or not be numbers.
       r.q = p.q; r.w = p.w; r.qscale = p.qscale;
       r.n_vis = 0; r.K = 0;
       r.out = nullptr; r.out_score = nullptr; r.out_rows = 0; r.out_stride = 0;
-      r.q_map = 0; r.q_row = q.tok0;
+      r.q_map = q.n_proxy > 0 ? 1 : 0;
+      r.q_row = q.n_proxy > 0 ? q.proxy0 + q.n_proxy - 1 : q.tok0 + q.dense_begin + q.n_dense - 1;
     }
     if (p.split > 1) {
       // The block's key tiles in p.split equal runs, each a block of its own; what the parts select goes to the

@@ -49,3 +49,43 @@ def test_chunk_of_a_short_prefix_and_a_small_budget(pv, dtype, g, mode, W, L, ro
     assert pv.pivot_device_status() == 0
     assert np.array_equal(_sorted(whole[row0:]), _sorted(part[row0:]))
     assert (part[:row0] == -7).all()
+
+
+def _nan_rows(q, rows):
+    """e4m3 queries with NaN codes in the given rows."""
+    q = q.clone()
+    q.view(torch.uint8)[rows] = 0x7f
+    return q
+
+
+def test_chunk_does_not_read_queries_outside_its_rows(pv):
+    """A chunk's rows are all it indexes: the other rows of the query tensor may hold anything (they arrive
+    later, or were overwritten).  33 groups: the last block of scan rows is padded where the prefix is scanned in parts."""
+    L, g, c, k, row0 = 8192, 4, 256, 128, 8192 - 132
+    x = inputs.make_prefill(L, dtype="fp8", seed=3)
+    q, w, kk, kw = _operands(x)
+    a = torch.full((L, k), -7, dtype=torch.int32, device="cuda")
+    b = torch.full((L, k), -7, dtype=torch.int32, device="cuda")
+    pv.pivot_index_prefill(q, w, kk, L, 64, 128, g, c, k, pv.REFINE, a, rows=(row0, L), **kw)
+    pv.pivot_index_prefill(_nan_rows(q, slice(0, row0)), w, kk, L, 64, 128, g, c, k, pv.REFINE, b, rows=(row0, L), **kw)
+    torch.cuda.synchronize()
+    assert np.array_equal(_sorted(a), _sorted(b))
+
+
+def test_packed_request_is_not_touched_by_its_first_row_in_its_last_block(pv):
+    """Packed requests are padded to whole blocks of scan rows: what a padding row holds must not reach the live
+    rows of its block, so NaN queries in the first group change that group's selections only, as in separate calls."""
+    lens, g, c, k = [1004, 2003], 4, 256, 128
+    cu = [0, 1004, 3007]
+    x = inputs.make_prefill(cu[-1], dtype="fp8", seed=4)
+    q, w, kk, kw = _operands(x)
+    q = _nan_rows(q, slice(1004, 1008))
+    packed = torch.full((cu[-1], k), -7, dtype=torch.int32, device="cuda")
+    one = torch.full((cu[-1], k), -7, dtype=torch.int32, device="cuda")
+    pv.pivot_index_prefill_varlen(q, w, kk, cu, 64, 128, g, c, k, pv.REFINE, packed, **kw)
+    for a, b in zip(cu[:-1], cu[1:]):
+        pv.pivot_index_prefill(q[a:b], w[a:b], kk[a:b], b - a, 64, 128, g, c, k, pv.REFINE, one[a:b],
+                               q_scale=kw["q_scale"][a:b], k_scale=kw["k_scale"][a:b])
+    torch.cuda.synchronize()
+    assert lens == [b - a for a, b in zip(cu[:-1], cu[1:])]
+    assert np.array_equal(_sorted(packed), _sorted(one))
