@@ -66,7 +66,8 @@ __device__ __forceinline__ void prof_max(int* status, int slot, long long v) {
 #define PIVOT_PROF_DO(...)
 #endif
 
-// fp32 score -> uint32 key whose unsigned order equals the float order (-inf lowest).
+// fp32 score -> uint32 key whose unsigned order equals the float order (-inf lowest).  A NaN takes the key of -0
+// (the compiler sets the sign bit with a float negation, which returns the one NaN there is as it was).
 __device__ __forceinline__ uint32_t score_to_key(float s) {
   uint32_t b = __float_as_uint(s);
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);

@@ -281,6 +281,9 @@ decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
       ptx::relu_dot32(v1, &ct.w[set][32], acc);
       float sv = ptx::relu_dot_sum(acc);
       if (C::FP8) sv *= ksv;
+      // A NaN goes to the score array as the -0 that score_to_key takes it for: the select forms its keys from
+      // the bits, and both have to agree with the histogram.
+      sv = sv == sv ? sv : -0.f;
       const int s_key = (g - first) * TILE_KEYS + key_in_tile;
       if (s_key < n_vis && PIVOT_BOUNDS(s_key < Lmax, status)) {
         scores[(size_t)b * Lmax + s_key] = sv;

@@ -89,3 +89,26 @@ def test_packed_request_is_not_touched_by_its_first_row_in_its_last_block(pv):
     torch.cuda.synchronize()
     assert lens == [b - a for a, b in zip(cu[:-1], cu[1:])]
     assert np.array_equal(_sorted(packed), _sorted(one))
+
+
+NAN_AT, ZERO_AT = [5, 70, 130, 201], 250
+
+
+def _all_but_nan(n):
+    return np.array([p for p in range(n) if p not in NAN_AT])
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("B,n", [(2, 257), (3, 5000), (80, 700)])
+def test_nan_key_scales_rank_behind_every_number_in_decode(pv, mode, B, n):
+    """A NaN score counts in the scan's histogram as what the select takes it for: -0."""
+    g = 2
+    c = k = n - len(NAN_AT)
+    x = inputs.make_decode(B, g, n, n, dtype="fp8", seed=9)
+    x.kscale[:, NAN_AT] = float("nan")
+    q, w, kk, kw = _operands(x)
+    out = torch.full((B, g, k), -7, dtype=torch.int32, device="cuda")
+    pv.pivot_index_decode(q, w, kk, x.pos0.cuda(), B, kk.shape[1], 64, 128, g, c, k, mode, out, **kw)
+    torch.cuda.synchronize()
+    assert pv.pivot_device_status() == 0
+    assert (_sorted(out) == _all_but_nan(n)).all()
