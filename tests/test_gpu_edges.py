@@ -112,3 +112,49 @@ def test_nan_key_scales_rank_behind_every_number_in_decode(pv, mode, B, n):
     torch.cuda.synchronize()
     assert pv.pivot_device_status() == 0
     assert (_sorted(out) == _all_but_nan(n)).all()
+
+
+def _keys_without_a_score(x, nan_at, zero_at):
+    """NaN entries in the keys at nan_at (any leading dimensions, positions second to last), a key of zeros at zero_at."""
+    k = x.k.clone()
+    if k.dtype == torch.bfloat16:
+        k[..., nan_at, 17] = float("nan")
+        k[..., zero_at, :] = 0.0
+    else:
+        k.view(torch.uint8)[..., nan_at, 17] = 0x7f
+        k.view(torch.uint8)[..., zero_at, :] = 0
+    x.k = k
+    return x
+
+
+@pytest.mark.parametrize("dtype,impl", [("bf16", 0), ("fp8", 0), ("fp8", 2)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_nan_keys_rank_behind_every_number_in_prefill(pv, dtype, impl, mode):
+    """A NaN in a key makes its products, and so its score, NaN in every form of the head sum.  A NaN ranks as -0:
+    behind a later key whose score is exactly 0, which behind keys of equal score it would not."""
+    L, g, c = 401, 4, 257                        # the group at 256 sees exactly c keys, all of them candidates
+    k = c - len(NAN_AT)
+    x = _keys_without_a_score(inputs.make_prefill(L, dtype=dtype, seed=6), NAN_AT, ZERO_AT)
+    q, w, kk, kw = _operands(x)
+    out = torch.full((L, k), -7, dtype=torch.int32, device="cuda")
+    pv.pivot_index_prefill(q, w, kk, L, 64, 128, g, c, k, mode, out, impl=impl, **kw)
+    dense = torch.full((L, k), -7, dtype=torch.int32, device="cuda")
+    pv.dense_index(q, w, kk, L, 64, 128, k, dense, impl=impl, **kw)
+    torch.cuda.synchronize()
+    assert pv.pivot_device_status() == 0
+    assert (_sorted(out[256:260]) == _all_but_nan(c)).all()
+    assert (_sorted(dense[256:257]) == _all_but_nan(c)).all()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp8"])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_nan_keys_rank_behind_every_number_in_decode(pv, dtype, mode):
+    B, g, c = 3, 2, 257
+    k = c - len(NAN_AT)
+    x = _keys_without_a_score(inputs.make_decode(B, g, c, c, dtype=dtype, seed=7), NAN_AT, ZERO_AT)
+    q, w, kk, kw = _operands(x)
+    out = torch.full((B, g, k), -7, dtype=torch.int32, device="cuda")
+    pv.pivot_index_decode(q, w, kk, x.pos0.cuda(), B, kk.shape[1], 64, 128, g, c, k, mode, out, **kw)
+    torch.cuda.synchronize()
+    assert pv.pivot_device_status() == 0
+    assert (_sorted(out) == _all_but_nan(c)).all()
