@@ -87,8 +87,8 @@ struct TileWalk {
 template <int DT>
 __global__ void __launch_bounds__(D_THREADS, 1)
 decode_scan_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_q,
-                   const __grid_constant__ CUtensorMap tm_ks, const RowDesc* __restrict__ prox,
-                   const int* __restrict__ tile_prefix, int B, int Lmax, float* __restrict__ scores,
+                   const __grid_constant__ CUtensorMap tm_ks, const RowDesc* prox,
+                   const int* tile_prefix, int B, int Lmax, float* __restrict__ scores,
                    uint32_t* __restrict__ ghist, int* status) {
   using C = DCfg<DT>;
   extern __shared__ uint8_t smem_raw[];
@@ -314,8 +314,7 @@ struct SelSmem {
 // hand-over 6 K: 24.6 us a step of 32 sequences of 64K .. 128K keys, now 18.4).
 template <int SEL_SPLIT>
 __global__ void __launch_bounds__(kBlk, 1)
-decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __restrict__ scores,
-                     const uint32_t* __restrict__ ghist, int* status) {
+decode_select_kernel(const RowDesc* prox, int Ls, const float* scores, const uint32_t* ghist, int* status) {
   extern __shared__ uint8_t sel_raw[];
   SelSmem& sm = *reinterpret_cast<SelSmem*>(((uintptr_t)sel_raw + 15) & ~(uintptr_t)15);
   const int split = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
@@ -524,7 +523,7 @@ decode_select_kernel(const RowDesc* __restrict__ prox, int Ls, const float* __re
 // PER_SM: blocks that share an SM (two where one wave would not hold the queries otherwise: 192 queries took
 // two waves, 9 us; one block per SM has the registers to hold its list without spills, 5 us against 7.6).
 template <int PER_SM>
-__global__ void __launch_bounds__(kBlk, PER_SM) entries_topk_kernel(const EntryList* __restrict__ lists) {
+__global__ void __launch_bounds__(kBlk, PER_SM) entries_topk_kernel(const EntryList* lists) {
   __shared__ BlkSelSmem sm;
   ptx::grid_launch_dependents();
   ptx::grid_dependency_wait();            // the re-score's entries
@@ -541,7 +540,7 @@ static_assert(8192 + kDecodeWinMax <= 9 * kBlk, "largest candidate budget plus w
 // Top-K of a scan row whose prefix was scanned in parts, one block per row.  Bound by its chain of loads and
 // barriers: two blocks per SM where the registers allow it (2048 rows of 2 x 4096 entries: 104 us against 155).
 template <int U>
-__global__ void __launch_bounds__(kBlk, U <= 8 ? 2 : 1) merge_parts_kernel(const MergeRow* __restrict__ rows) {
+__global__ void __launch_bounds__(kBlk, U <= 8 ? 2 : 1) merge_parts_kernel(const MergeRow* rows) {
   __shared__ BlkSelSmem sm;
   __shared__ int part0[8];               // first key of each part
   ptx::grid_launch_dependents();
@@ -688,8 +687,7 @@ decode_prepare_kernel(DecodePlan p, RowDesc* rows, GroupDesc* plan_groups, uint3
 // pos0 - W + 1 .. pos0 + g - 1, becomes one more candidate chunk of the sequence; positions the
 // pool already holds (and positions before the start of the sequence) are left out as -1, and
 // the re-score kernel masks every slot to the members whose window covers it.
-__global__ void decode_window_kernel(const GroupDesc* __restrict__ groups, int mc, int g, int W,
-                                     int32_t* __restrict__ wcand) {
+__global__ void decode_window_kernel(const GroupDesc* groups, int mc, int g, int W, int32_t* wcand) {
   __shared__ int dup[kDecodeWinMax];
   const int b = blockIdx.x, tid = threadIdx.x;
   ptx::grid_launch_dependents();

@@ -35,7 +35,9 @@ __device__ __forceinline__ bool elect_one() {
 // the predecessor has completed and its writes are visible (a no-op in a kernel launched the
 // ordinary way), so everything before it must touch neither the predecessor's outputs nor anything
 // it still reads; grid_launch_dependents() lets the successor's blocks be scheduled as soon as
-// every block of this grid has called it or exited.
+// every block of this grid has called it or exited.  What the predecessor writes is read by plain or
+// L2 loads only: `const __restrict__` and __ldg promise data that is constant for the kernel's
+// whole life, and such loads may be moved across the wait.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -129,7 +129,7 @@ __device__ __forceinline__ int group_tiles(const GroupDesc& gd) {
 
 template <int DT, int EPI>
 __global__ void __launch_bounds__((RCfg<DT, EPI>::THREADS), 1)
-refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* __restrict__ groups, int n_groups,
+refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* groups, int n_groups,
                  int q_rows_total, ScanScratch sc) {
   using C = RCfg<DT, EPI>;
   extern __shared__ uint8_t smem_raw[];
@@ -340,7 +340,7 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* __re
       const int pos_limit = gd.pos_max;
       auto load_idx = [&](int tile, int half) -> int {
         const int sl = tile * TILE_KEYS + wrow0 + half * 32 + lane;
-        return (tile < ntiles && sl < gd.n_cand) ? __ldg(gd.cand + sl) : -1;
+        return (tile < ntiles && sl < gd.n_cand) ? gd.cand[sl] : -1;
       };
       // A candidate position beyond the group's last member (gd.pos_max) cannot come from the scan; it
       // can come from a caller-supplied candidate set.  Such a slot is dropped like a padding slot and

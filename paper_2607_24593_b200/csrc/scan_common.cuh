@@ -124,7 +124,7 @@ __device__ __forceinline__ uint32_t select_bin_lo(int bin, int base) {
 // the next block in the row's other segment.
 template <int NROWS, int QD>
 __device__ __noinline__ void append_role(SelectCtrl<NROWS, QD>& s, int r, int lane, const Team& tm,
-                                            const RowDesc* __restrict__ rows, int n_rows, int n_blocks,
+                                            const RowDesc* rows, int n_rows, int n_blocks,
                                             const ScanScratch& sc, volatile int* abort_flag) {
   SegSelSmem& sel = s.sel[r];
   const int CAP = sc.cap;                        // entries of this row's candidate segment
@@ -260,7 +260,7 @@ __device__ __noinline__ void append_role(SelectCtrl<NROWS, QD>& s, int r, int la
 // Reuse group.
 template <int NROWS, int QD>
 __device__ __noinline__ void finisher_role(SelectCtrl<NROWS, QD>& s, int r0, int nr, int lane,
-                                              const RowDesc* __restrict__ rows, int n_rows, int n_blocks,
+                                              const RowDesc* rows, int n_rows, int n_blocks,
                                               const ScanScratch& sc, volatile int* abort_flag) {
   BlockIter bi(n_blocks, gridDim.x, blockIdx.x);
   uint32_t seq = 0;

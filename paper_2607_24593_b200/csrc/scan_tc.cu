@@ -115,7 +115,7 @@ template <int DT, int NROWS, int EPI>
 __global__ void __launch_bounds__(Cfg<DT, NROWS, EPI>::THREADS, 1)
 scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_q0,
                       const __grid_constant__ CUtensorMap tm_q1, const __grid_constant__ CUtensorMap tm_ks,
-                      const RowDesc* __restrict__ rows, int n_rows, ScanScratch sc) {
+                      const RowDesc* rows, int n_rows, ScanScratch sc) {
   using C = Cfg<DT, NROWS, EPI>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);

@@ -390,7 +390,7 @@ struct KeyRowSrc {
   static constexpr bool kKeysApart = true;       // keys can be swept without their positions
   const uint32_t* keys;
   int nslots;
-  const int32_t* __restrict__ cand;
+  const int32_t* cand;          // (written by the kernel before this one: plain loads)
   int n_cand;
   __device__ __forceinline__ int slots() const { return nslots; }
   // U slots per lane from slot i0 on (key 0: empty)
@@ -401,7 +401,7 @@ struct KeyRowSrc {
 #pragma unroll
     for (int j = 0; j < U; ++j) {
       k[j] = i0 + j * 32 < nslots ? __ldcg(kp + j * 32) : 0u;
-      ps[j] = i0 + j * 32 + lane < n_cand ? __ldg(cp + j * 32) : -1;
+      ps[j] = i0 + j * 32 + lane < n_cand ? cp[j * 32] : -1;
     }
   }
   template <int U, typename F>
@@ -426,7 +426,7 @@ struct KeyRowSrc {
       for (int j = 0; j < U; ++j) {
         const int sl = s0 + j * 32 + lane;
         k[j] = sl < nslots ? __ldcg(keys + sl) : 0u;
-        ps[j] = (NEED_POS && sl < n_cand) ? __ldg(cand + sl) : -1;
+        ps[j] = (NEED_POS && sl < n_cand) ? cand[sl] : -1;
       }
 #pragma unroll
       for (int j = 0; j < U; ++j) f(k[j] ? make_entry(k[j], ps[j]) : 0ull);   // without positions: low word 0
@@ -627,7 +627,7 @@ __device__ __noinline__ int warp_topk_entries(SegSelSmem& sm, const Src src, ent
 }
 
 __device__ __forceinline__ int warp_row_topk(SegSelSmem& sm, const uint32_t* keys, int nslots,
-                                             const int32_t* __restrict__ cand, int n_cand, int32_t* out,
+                                             const int32_t* cand, int n_cand, int32_t* out,
                                              float* out_score, int K, int lane, uint32_t kmin, uint32_t kmax,
                                              uint32_t n_filled) {
   return warp_topk_entries(sm, KeyRowSrc{keys, nslots, cand, n_cand}, (entry_t)kmin << 32,
