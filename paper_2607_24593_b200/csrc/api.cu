@@ -237,10 +237,11 @@ int choose_split(int n_proxy, int first_vis, int last_vis, int K, int sms, size_
 }
 
 // Requests cu[0] .. cu[n] of a packed batch (host array; one request: {0, L}), each indexed on its own.
-// All of them go through one prepare, one scan and one re-score launch.
+// All of them go through one prepare, one scan and one re-score launch.  first: the call's first (or only) set of
+// launches -- it clears the status word; a later one leaves what the sets before it recorded.
 int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kcache, const int32_t* cu, int n, int g,
                 int c, int k, int mode, bool dense_only, int32_t* out_idx, cudaStream_t st, const pivot_opts* o, void* wsp,
-                int ws_rows, int ws_groups) {
+                int ws_rows, int ws_groups, bool first = true) {
   Workspace ws = carve_workspace(wsp, ws_rows, ws_groups, c, k);
   g_dev[cur_device()].last_status = ws.status;
   const int guard = (o && o->guard_len >= 0) ? o->guard_len : c;
@@ -260,7 +261,7 @@ int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kcach
   p.W = W;
   p.pool = o ? o->pool : 0;
   p.skip_trivial = !(o && o->impl == 1);      // (the cross-check kernels score every row)
-  p.status = ws.status;
+  p.status = first ? ws.status : nullptr;
   int pg0 = 0, live = 0;
   for (int i = 0; i < n; ++i) live += cu[i + 1] > cu[i];
   for (int i = 0; i < n; ++i) {
@@ -407,6 +408,7 @@ int pivot_index_prefill_varlen(const pivot_tensor* q, const float* w, const pivo
   const size_t krow = kcache->stride_row ? kcache->stride_row : (size_t)d * esz;
   const size_t ws_have = opts && opts->workspace ? opts->workspace_bytes : g_dev[cur_device()].ws_bytes;
   int32_t cu[kMaxPlanReqs + 1];
+  bool first = true;
   for (int i = 0; i < n_req;) {
     const int r0 = cu_seqlens[i];
     int n = 0, rows = 0, groups = 0;
@@ -430,8 +432,9 @@ int pivot_index_prefill_varlen(const pivot_tensor* q, const float* w, const pivo
     pivot_tensor tq{(const char*)q->data + (size_t)r0 * H_I * d * esz, q->scale ? q->scale + (size_t)r0 * H_I : nullptr, q->dtype, 0};
     pivot_tensor tk{(const char*)kcache->data + (size_t)r0 * krow, kcache->scale ? kcache->scale + r0 : nullptr, q->dtype, kcache->stride_row};
     rc = run_prefill(&tq, w + (size_t)r0 * H_I, &tk, cu, n, g, c, k, mode, false, out_idx + (size_t)r0 * k, (cudaStream_t)stream,
-                     opts, wsp, rows, groups);
+                     opts, wsp, rows, groups, first);
     if (rc) return rc;
+    first = false;
   }
   return PIVOT_OK;
 }

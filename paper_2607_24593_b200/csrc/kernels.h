@@ -93,7 +93,7 @@ struct PrefillPlan {
   int pool = 0;
   int W = 0;            // local window (Appendix B); 0 = off
   bool skip_trivial = true;   // rows that select all they see are written by the planner instead of scanned
-  int* status = nullptr;      // status word and row counter: cleared by the planner
+  int* status = nullptr;      // status word and row counter: cleared by the planner (nullptr: left as they are)
   int n_slots = 0;      // scan-row slots: the rows of all requests, each request padded to whole blocks of four if there are several
   int n_proxy = 0;      // proxies of all requests
   int n_req = 0;

@@ -158,3 +158,52 @@ def test_nan_keys_rank_behind_every_number_in_decode(pv, dtype, mode):
     torch.cuda.synchronize()
     assert pv.pivot_device_status() == 0
     assert (_sorted(out) == _all_but_nan(c)).all()
+
+
+def test_status_of_an_earlier_set_of_requests_survives(pv):
+    """A packed batch beyond one set of launches (more than 64 requests) is prepared in several: a condition that
+    the first set recorded is still there at the end of the call, and the next call starts clean.  The condition
+    is planted into a captured call between its two sets."""
+    cudart = pytest.importorskip("cuda.bindings.runtime")
+    lens, g, c, k = [64] * 70, 4, 32, 16
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(int)
+    x = inputs.make_prefill(int(cu[-1]), dtype="bf16", seed=12)
+    q, w, kk, kw = _operands(x)
+    out = torch.full((int(cu[-1]), k), -7, dtype=torch.int32, device="cuda")
+    ws = torch.empty(pv.pivot_workspace_bytes(int(cu[-1]) + 4 * 70, int(cu[-1]) // g, c, k), dtype=torch.uint8, device="cuda")
+    call = lambda: pv.pivot_index_prefill_varlen(q, w, kk, cu, 64, 128, g, c, k, pv.REFINE, out, workspace=ws, **kw)
+    pv.lib.pivot_launch_count_reset()
+    call()                                       # (function attributes are set before the capture)
+    per_set = pv.lib.pivot_launch_count_reset() // 2
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    raw = cudart.cudaGraph_t(graph.raw_cuda_graph())
+
+    def ok(r):
+        assert r[0] == cudart.cudaError_t.cudaSuccess, r[0]
+        return r[1:] if len(r) > 2 else (r[1] if len(r) == 2 else None)
+
+    n = ok(cudart.cudaGraphGetNodes(raw, 0))[1]
+    nodes = ok(cudart.cudaGraphGetNodes(raw, n))[0]
+    assert n == 2 * per_set == len(nodes)
+    edges = ok(cudart.cudaGraphGetEdges_v2(raw, 0))[-1]
+    src, dst = ok(cudart.cudaGraphGetEdges_v2(raw, edges))[:2]
+    after = {int(a): int(b) for a, b in zip(src, dst)}
+    order = [next(int(v) for v in nodes if int(v) not in after.values())]
+    while order[-1] in after:
+        order.append(after[order[-1]])
+    assert len(order) == n                       # a chain
+    by_id = {int(v): v for v in nodes}
+    end_first, begin_second = by_id[order[per_set - 1]], by_id[order[per_set]]
+    p = cudart.cudaMemsetParams()
+    p.dst, p.value, p.elementSize, p.width, p.height, p.pitch = ws.data_ptr(), pv.DEV_CAND_OVERFLOW, 4, 1, 1, 4
+    node = ok(cudart.cudaGraphAddMemsetNode(raw, [end_first], 1, p))
+    ok(cudart.cudaGraphAddDependencies(raw, [node], [begin_second], 1))
+    graph.instantiate()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert pv.pivot_device_status() == pv.DEV_CAND_OVERFLOW
+    call()
+    assert pv.pivot_device_status() == 0
