@@ -91,6 +91,7 @@ def _load():
 
 lib = _load()
 _workspaces: dict[int, torch.Tensor] = {}
+_no_room: dict[int, int] = {}                # per device: a batch's workspace that did not fit, until another one is registered
 
 
 def _check(rc: int):
@@ -153,11 +154,13 @@ def pivot_set_workspace(workspace: torch.Tensor | None):
     """Registers a uint8 CUDA tensor as the scratch of the short entry points (kept alive here)."""
     if workspace is None:
         _check(lib.pivot_set_workspace(None, 0))
-        _workspaces.pop(torch.cuda.current_device(), None)
+        for kept in (_workspaces, _no_room):
+            kept.pop(torch.cuda.current_device(), None)
         return
     assert workspace.dtype == torch.uint8 and workspace.is_cuda
     _check(lib.pivot_set_workspace(workspace.data_ptr(), workspace.numel()))
     _workspaces[workspace.device.index] = workspace
+    _no_room.pop(workspace.device.index, None)
 
 
 def pivot_decode_workspace_bytes(B: int, Lmax: int, g: int, c: int, k: int) -> int:
@@ -195,7 +198,11 @@ def pivot_index_prefill(q, w, kcache, L, H_I, d, g, c, k, mode, out_idx, stream=
 def pivot_index_prefill_varlen(q, w, kcache, cu_seqlens, H_I, d, g, c, k, mode, out_idx, stream=None, *,
                                q_scale=None, k_scale=None, guard_len=None, pool=POOL_MEAN, workspace=None, impl=0, W=0):
     """Several requests packed back to back; cu_seqlens is a host sequence [n_req + 1] starting at 0.
-    Positions in out_idx are relative to each row's own request."""
+    Positions in out_idx are relative to each row's own request.
+
+    Without `workspace` the registered one grows to hold the batch, up to 16384 groups of it (268 MB of candidates at
+    c = 4096, as much again for the proxies), so that its requests share their launches; where the GPU has no
+    room for that, to hold the longest request, which takes them one after the other."""
     cu = [int(v) for v in cu_seqlens]
     n_req = len(cu) - 1
     tq, tk = _tensor(q, q_scale), _tensor(kcache, k_scale)
@@ -203,11 +210,20 @@ def pivot_index_prefill_varlen(q, w, kcache, cu_seqlens, H_I, d, g, c, k, mode, 
     if workspace is None:
         # room for the longest request, and for the batch up to 16384 groups: what fits shares its launches
         Lmax = max(max((b - a for a, b in zip(cu[:-1], cu[1:])), default=1), 1)
-        rows, groups = Lmax + 4, (Lmax + g - 1) // g
+        rows, groups = Lmax, (Lmax + g - 1) // g
+        longest = (rows, groups)
         both = [(b - a + 4, (b - a + g - 1) // g) for a, b in zip(cu[:-1], cu[1:]) if b > a]
         rows = max(rows, min(sum(r for r, _ in both), 16384 * g + 4 * n_req))
         groups = max(groups, min(sum(n for _, n in both), 16384 + n_req))
-        ensure_workspace(rows, groups, c, k, q.device)
+        idx = q.device.index
+        need = _workspace_bytes(idx, rows, groups, c, k)
+        if need < _no_room.get(idx, need + 1):
+            try:
+                ensure_workspace(rows, groups, c, k, q.device, need=need)
+            except torch.OutOfMemoryError:
+                _no_room[idx] = need         # (asking again on every call would empty the allocator's cache each time)
+        if need >= _no_room.get(idx, need + 1):
+            ensure_workspace(*longest, c, k, q.device)
     o = _opts(guard_len, pool, None, None, None, workspace, impl, None, W)
     arr = (C.c_int32 * (n_req + 1))(*cu)
     _check(lib.pivot_index_prefill_varlen(C.byref(tq), w.data_ptr(), C.byref(tk), arr, n_req, H_I, d, g, c, k, mode,

@@ -207,3 +207,38 @@ def test_status_of_an_earlier_set_of_requests_survives(pv):
     assert pv.pivot_device_status() == pv.DEV_CAND_OVERFLOW
     call()
     assert pv.pivot_device_status() == 0
+
+
+def test_packed_batch_where_only_the_longest_request_fits(pv, monkeypatch):
+    """The binding's own workspace shares a batch's launches where there is memory for that; where there is not,
+    the call runs with room for its longest request, as it always could."""
+    lens, g, c, k = [400, 1600, 900, 1200], 4, 256, 128
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(int)
+    x = inputs.make_prefill(int(cu[-1]), dtype="fp8", seed=13)
+    q, w, kk, kw = _operands(x)
+    run = lambda: pv.pivot_index_prefill_varlen(q, w, kk, cu, 64, 128, g, c, k, pv.REFINE,
+                                                torch.full((int(cu[-1]), k), -7, dtype=torch.int32, device="cuda"), **kw)
+    want = _sorted(run())
+    longest = pv.pivot_workspace_bytes(max(lens), (max(lens) + g - 1) // g, c, k)
+    empty = torch.empty
+
+    refused = []
+
+    def small_gpu(*a, **kw_):
+        if kw_.get("dtype") == torch.uint8 and a and isinstance(a[0], int) and a[0] > longest:
+            refused.append(a[0])
+            raise torch.cuda.OutOfMemoryError("no room")
+        return empty(*a, **kw_)
+
+    keep = pv._workspaces.get(torch.cuda.current_device())
+    pv.pivot_set_workspace(None)
+    monkeypatch.setattr(torch, "empty", small_gpu)
+    try:
+        got = [_sorted(run()) for _ in range(4)]
+        assert pv._workspaces[torch.cuda.current_device()].numel() <= longest
+        assert len(refused) <= 2                 # not on every call
+    finally:
+        monkeypatch.undo()
+        pv.pivot_set_workspace(keep)
+    assert all(np.array_equal(v, want) for v in got)
+    assert np.array_equal(_sorted(run()), want)
