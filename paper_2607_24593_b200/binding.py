@@ -92,6 +92,7 @@ def _load():
 lib = _load()
 _workspaces: dict[int, torch.Tensor] = {}
 _no_room: dict[int, int] = {}                # per device: a batch's workspace that did not fit, until another one is registered
+_outgrown: dict[int, list] = {}              # per device: registered workspaces that held every request, but not a batch
 
 
 def _check(rc: int):
@@ -154,7 +155,7 @@ def pivot_set_workspace(workspace: torch.Tensor | None):
     """Registers a uint8 CUDA tensor as the scratch of the short entry points (kept alive here)."""
     if workspace is None:
         _check(lib.pivot_set_workspace(None, 0))
-        for kept in (_workspaces, _no_room):
+        for kept in (_workspaces, _no_room, _outgrown):
             kept.pop(torch.cuda.current_device(), None)
         return
     assert workspace.dtype == torch.uint8 and workspace.is_cuda
@@ -202,7 +203,10 @@ def pivot_index_prefill_varlen(q, w, kcache, cu_seqlens, H_I, d, g, c, k, mode, 
 
     Without `workspace` the registered one grows to hold the batch, up to 16384 groups of it (268 MB of candidates at
     c = 4096, as much again for the proxies), so that its requests share their launches; where the GPU has no
-    room for that, to hold the longest request, which takes them one after the other."""
+    room for that, to hold the longest request, which takes them one after the other.  A workspace that held
+    the longest request is not given back when a batch outgrows it (graphs captured with it and calls on other
+    streams go on using it) until pivot_set_workspace(None); growing by half at least keeps all of
+    these below twice the last one."""
     cu = [int(v) for v in cu_seqlens]
     n_req = len(cu) - 1
     tq, tk = _tensor(q, q_scale), _tensor(kcache, k_scale)
@@ -218,8 +222,13 @@ def pivot_index_prefill_varlen(q, w, kcache, cu_seqlens, H_I, d, g, c, k, mode, 
         idx = q.device.index
         need = _workspace_bytes(idx, rows, groups, c, k)
         if need < _no_room.get(idx, need + 1):
+            old = _workspaces.get(idx)
             try:
-                ensure_workspace(rows, groups, c, k, q.device, need=need)
+                if old is None or old.numel() < _workspace_bytes(idx, *longest, c, k):
+                    ensure_workspace(rows, groups, c, k, q.device, need=need)      # (has to be replaced as it is)
+                elif old.numel() < need:
+                    ensure_workspace(rows, groups, c, k, q.device, need=max(need, old.numel() * 3 // 2))
+                    _outgrown.setdefault(idx, []).append(old)
             except torch.OutOfMemoryError:
                 _no_room[idx] = need         # (asking again on every call would empty the allocator's cache each time)
         if need >= _no_room.get(idx, need + 1):

@@ -242,3 +242,39 @@ def test_packed_batch_where_only_the_longest_request_fits(pv, monkeypatch):
         pv.pivot_set_workspace(keep)
     assert all(np.array_equal(v, want) for v in got)
     assert np.array_equal(_sorted(run()), want)
+
+
+def test_workspace_that_a_batch_outgrows_stays_valid(pv):
+    """A graph captured with the registered workspace goes on using it after a packed batch made the binding
+    register a larger one: the memory is not handed to anyone else, and the graph's results stay right."""
+    dev = torch.cuda.current_device()
+    pv.pivot_set_workspace(None)
+    g, c, k, n = 2, 128, 64, 600
+    xd = inputs.make_decode(2, g, n, n, dtype="fp8", seed=14)
+    q, w, kk, kw = _operands(xd)
+    pos0, out = xd.pos0.cuda(), torch.full((2, g, k), -7, dtype=torch.int32, device="cuda")
+    xp = inputs.make_prefill(6000, dtype="fp8", seed=15)
+    pq, pw, pk, pkw = _operands(xp)
+    pv.ensure_workspace(2000, 500, 512, 256)                       # room for any one request
+    first = pv._workspaces[dev]
+    step = lambda: pv.pivot_index_decode(q, w, kk, pos0, 2, kk.shape[1], 64, 128, g, c, k, pv.REFINE, out, **kw)
+    step()
+    want = _sorted(out)
+    assert pv._workspaces[dev] is first
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        step()
+    at, size = first.data_ptr(), first.numel()
+    del first
+    pv.pivot_index_prefill_varlen(pq, pw, pk, [0, 2000, 4000, 6000], 64, 128, 4, 512, 256, pv.REFINE,
+                                  torch.full((6000, 256), -7, dtype=torch.int32, device="cuda"), **pkw)
+    assert pv._workspaces[dev].numel() > size
+    others = [torch.zeros(size, dtype=torch.uint8, device="cuda") for _ in range(3)]
+    assert all(o.data_ptr() + size <= at or o.data_ptr() >= at + size for o in others)
+    out.fill_(-7)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(_sorted(out), want)
+    assert not any(o.any() for o in others)
+    pv.pivot_set_workspace(None)
+    assert not pv._outgrown
