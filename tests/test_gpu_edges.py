@@ -278,3 +278,13 @@ def test_workspace_that_a_batch_outgrows_stays_valid(pv):
     assert not any(o.any() for o in others)
     pv.pivot_set_workspace(None)
     assert not pv._outgrown
+
+
+def test_current_stream_with_and_without_the_raw_handle(pv, monkeypatch):
+    """The stream of a call without a `stream` argument, also on a torch release that lacks the raw accessor."""
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        assert pv._stream(None) == side.cuda_stream
+        monkeypatch.setattr(pv, "_raw_stream", None)
+        assert pv._stream(None) == side.cuda_stream
+    assert pv._stream(None) == torch.cuda.current_stream().cuda_stream
