@@ -1,6 +1,7 @@
 // C ABI of the library (see include/pivot.h): argument checks, workspace carving, and the
 // launch sequence of Algorithm 1 -- proxy build (Eq. 4), planner, shared scan + streaming
 // select (Eq. 5-7), gather + re-score + top-k (Eq. 8-9).
+#include <math.h>
 #include <stdio.h>
 #include <string.h>
 
@@ -63,9 +64,10 @@ int cand_cap(int kmax) {
 #ifndef PIVOT_CAP_FACTOR
 #define PIVOT_CAP_FACTOR 8
 #endif
+constexpr int kMinSegment = 8192;
 int tc_cap(int kmax) {
   size_t cap = (size_t)PIVOT_CAP_FACTOR * kmax;     // a tight running threshold admits about K (1 + ln(n / K)) entries
-  if (cap < 8192) cap = 8192;
+  if (cap < kMinSegment) cap = kMinSegment;
   return (int)align_up(cap, 256);
 }
 
@@ -211,14 +213,27 @@ int resolve_ws(const pivot_opts* o, size_t need, void** ws) {
 // Parts that a chunk's scan is cut into.  Its row blocks are few and of nearly equal length (a chunk at the end of
 // a long prompt), so whole blocks leave SMs idle in the last round, or most SMs in the only one: 512 blocks on 148
 // SMs take four rounds where 3.46 would do, 64 blocks leave 84 SMs without any.  The cost of S parts, in tiles:
-// rounds of part blocks, each with its own start -- some sixteen tiles' time between two blocks, and K / 128 tiles
-// before a threshold has formed -- and the merge of the parts' selections, 2 SMs' worth of rows at a time (14 us a
-// round of 2 x 4096 entries).  fp8, c = 4096: 8192 rows at the end of 256K 5.9 ms in one part, 5.3 + 0.1 in two; 1024 rows
-// at the end of 128K 981 -> 610 us; 6000 rows at the end of 64K stay whole (1.64 ms; in three parts 2.07).
+//   - rounds of part blocks, each with its own start: some sixteen tiles' time between two blocks, and K / 128 tiles
+//     before a threshold has formed;
+//   - where a part's survivors fill its candidate segment, the sweep that thins it out, 64 entries in a tile's time.
+//     A part admits every key of the refresh interval before the first threshold and about K / n of the n-th interval
+//     (K (ln n + 0.58) in all, 3 % more for the thresholds' bins).  K = 2048, 8192 rows at the end of 128K, four
+//     rounds of whole blocks: 3.58 ms, with segments twice as large 3.07; at the end of 256K in two parts, which
+//     still fill them, 6.69, in three, which do not, 5.59.  Segments of the least size (budgets up to 1024) are
+//     thinned within two intervals in any part and the sweep is short: not charged;
+//   - the merge of the parts' selections, 2 SMs' worth of rows at a time (14 us a round of 2 x 4096 entries; lists
+//     of more than 8192 entries have an SM to themselves, but charging them for that chooses worse: 3072 rows at
+//     the end of 128K would take 1.54 ms in two parts, 1.50 in three).
+// fp8, c = 4096: 8192 rows at the end of 256K 5.9 ms in one part, 5.3 + 0.1 in two; 1024 rows at the end of 128K
+// 981 -> 610 us; 6000 rows at the end of 64K stay whole (1.64 ms; in three parts 2.07).  Over 464 chunks (512 ..
+// 12000 rows at the end of 16K .. 256K, both types, K 512 .. 4096) the choice is within 7 % of the best number of
+// parts, 0.3 % off it in the mean, and at most 4 % behind whole blocks; a bf16 tile takes 1.3 times as long
+// as an fp8 one, but a term for that changes no choice for the better.
 // Calls whose blocks differ in length (a whole request) are balanced by the deal.
-// first_vis, last_vis: keys that the first and the last scan row see.  Every part of every block has a key tile of
-// its own (first_vis / 128 of them at least): a part without one would not be scanned and its list never written.
-int choose_split(int n_proxy, int first_vis, int last_vis, int K, int sms, size_t room, int slots) {
+// first_vis, last_vis: keys that the first and the last scan row see; cap: entries of a row's candidate segment.  Every
+// part of every block has a key tile of its own (first_vis / 128 of them at least): a part without one would not be
+// scanned and its list never written.
+int choose_split(int n_proxy, int first_vis, int last_vis, int K, int cap, int sms, size_t room, int slots) {
   if (first_vis < last_vis / 2) return 1;
   const int nb = (n_proxy + 3) / 4;
   const double tiles = last_vis / 128.0;
@@ -229,7 +244,13 @@ int choose_split(int n_proxy, int first_vis, int last_vis, int K, int sms, size_
       if (first_vis / s < 4 * K || first_vis / 128 < s || s * K > kMaxMerge || nb * 4 * s > slots) break;
       if (align_up((size_t)n_proxy * sizeof(MergeRow)) + 2 * align_up((size_t)n_proxy * s * K * 4) > room) break;
     }
-    double cost = (double)((s * nb + sms - 1) / sms) * (tiles / s + 16.0 + K / 128.0);
+    double per_block = tiles / s + 16.0 + K / 128.0;
+    const double intervals = tiles / s / kThresholdRefreshTiles;
+    if (cap > kMinSegment && intervals > 1.0) {
+      const double admitted = 1.03 * (kThresholdRefreshTiles * 128.0 + K * (log(intervals) + 0.58));
+      if (admitted > cap - kThresholdRefreshTiles * 128) per_block += admitted / 64.0;
+    }
+    double cost = (double)((s * nb + sms - 1) / sms) * per_block;
     if (s > 1) cost += (double)((n_proxy + 2 * sms - 1) / (2 * sms)) * (4.0 + 14.0 * s * K / 8192.0);
     if (s == 1 || cost < 0.97 * least) { least = cost; best = s; }
   }
@@ -301,7 +322,7 @@ int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kcach
     const size_t have = (size_t)ws_groups * c * sizeof(int32_t);
     const int unseen = W > 0 ? W - 1 : -1;            // a row at t0 sees t0 - unseen keys
     p.split = choose_split(p.n_proxy, q0.first_group * g - unseen, (q0.first_group + p.n_proxy - 1) * g - unseen, K,
-                           sm_count(), have > cv.off ? have - cv.off : 0, ws_rows + ws_groups);
+                           ws.tc_cap, sm_count(), have > cv.off ? have - cv.off : 0, ws_rows + ws_groups);
     if (p.split > 1) {
       p.merges = cv.take<MergeRow>(p.n_proxy);
       p.part_pos = cv.take<int32_t>((size_t)p.n_proxy * p.split * K);

@@ -127,6 +127,11 @@ struct DecodePlan {
   bool raw_q = false;
 };
 
+#ifndef PIVOT_CHK
+#define PIVOT_CHK 32
+#endif
+constexpr int kThresholdRefreshTiles = PIVOT_CHK;   // the scan's append warps re-read their rows' thresholds off the histograms this often
+
 struct ScanScratch {
   uint32_t* cand_key;   // [n_cta][2][cap]   (CUDA-core kernels: separate key / index arrays)
   int32_t* cand_idx;    // [n_cta][2][cap]

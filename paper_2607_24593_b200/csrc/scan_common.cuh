@@ -13,10 +13,6 @@ namespace scan {
 
 constexpr int TILE_KEYS = 128;
 constexpr int KS_SLOTS = 8;       // key-scale ring: deeper than (key stages + accumulator buffers)
-#ifndef PIVOT_CHK
-#define PIVOT_CHK 32
-#endif
-constexpr int kThresholdRefreshTiles = PIVOT_CHK;   // the append warp re-reads its row's threshold off the histogram this often
 
 // Block sequence of one CTA: blocks sorted longest-first are dealt in snake order.
 struct BlockIter {

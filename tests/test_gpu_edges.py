@@ -288,3 +288,19 @@ def test_current_stream_with_and_without_the_raw_handle(pv, monkeypatch):
         monkeypatch.setattr(pv, "_raw_stream", None)
         assert pv._stream(None) == side.cuda_stream
     assert pv._stream(None) == torch.cuda.current_stream().cuda_stream
+
+
+@pytest.mark.parametrize("dtype,mode,c,k,row0", [("fp8", 0, 1280, 1280, 11264), ("bf16", 1, 1280, 700, 11904), ("fp8", 1, 2000, 1000, 12000)])
+def test_chunk_whose_parts_fill_their_segments(pv, dtype, mode, c, k, row0):
+    """Budgets whose candidate segments are thinned out on the way (more than 1024, a few refresh intervals of
+    keys): however the prefix is cut, the rows of a chunk are the whole call's."""
+    L, g = 12288, 4
+    x = inputs.make_prefill(L, dtype=dtype, seed=16)
+    q, w, kk, kw = _operands(x)
+    whole = torch.full((L, k), -7, dtype=torch.int32, device="cuda")
+    part = torch.full((L, k), -7, dtype=torch.int32, device="cuda")
+    pv.pivot_index_prefill(q, w, kk, L, 64, 128, g, c, k, mode, whole, **kw)
+    pv.pivot_index_prefill(q, w, kk, L, 64, 128, g, c, k, mode, part, rows=(row0, L), **kw)
+    torch.cuda.synchronize()
+    assert pv.pivot_device_status() == 0
+    assert np.array_equal(_sorted(whole[row0:]), _sorted(part[row0:]))
