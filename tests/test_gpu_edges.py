@@ -304,3 +304,39 @@ def test_chunk_whose_parts_fill_their_segments(pv, dtype, mode, c, k, row0):
     torch.cuda.synchronize()
     assert pv.pivot_device_status() == 0
     assert np.array_equal(_sorted(whole[row0:]), _sorted(part[row0:]))
+
+
+@pytest.mark.parametrize("B", [2, 40, 80])
+@pytest.mark.parametrize("n_tied", [4096, 4097, 9000, 11988, 11989, 12400])
+def test_decode_crowded_boundary_bin(pv, B, n_tied):
+    """The boundary bin holds n_tied equal scores (one key repeated) and c cuts it: on either side of the lists
+    that the select ranks in shared memory (4096 boundary entries; 12288 survivors, 300 of them above the bin), for every cluster size
+    (batches of up to 37, up to 74 and more).  The lowest positions of the tie win."""
+    g, c, k, n = 1, 1024, 512, 14000
+    x = inputs.make_decode(1, g, n, n, dtype="fp8", seed=21)
+    kk = x.k.clone()
+    raw = kk.view(torch.uint8)
+    scale = x.kscale.clone()
+    gen = torch.Generator().manual_seed(n_tied)
+    tied = torch.randperm(n, generator=gen)[:n_tied].sort().values
+    free = torch.ones(n, dtype=torch.bool)
+    free[tied] = False
+    above = torch.nonzero(free).view(-1)[:300]
+    raw[0, tied] = raw[0, 7].clone()
+    scale[0, :] = scale[0, :] * 1e-3
+    scale[0, tied] = 1.0
+    raw[0, above] = raw[0, 7].clone()
+    scale[0, above] = 4.0
+    rep = lambda t: t.cuda().view(torch.uint8).expand(B, *t.shape[1:]).contiguous().view(t.dtype) if t.element_size() == 1 \
+        else t.cuda().expand(B, *t.shape[1:]).contiguous()
+    pos0 = torch.full((B,), n - 1, dtype=torch.int32, device="cuda")
+    out = torch.full((B, g, k), -7, dtype=torch.int32, device="cuda")
+    cand = torch.full((B, c), -7, dtype=torch.int32, device="cuda")
+    pv.pivot_index_decode(rep(x.q), rep(x.w), rep(kk), pos0, B, kk.shape[1], 64, 128, g, c, k, pv.REFINE, out, dbg_cand=cand,
+                          q_scale=rep(x.qscale), k_scale=rep(scale))
+    torch.cuda.synchronize()
+    assert pv.pivot_device_status() == 0
+    want = np.sort(np.concatenate([above.numpy(), tied.numpy()[: c - len(above)]]))
+    assert (_sorted(cand) == want).all()
+    want = np.sort(np.concatenate([above.numpy(), tied.numpy()[: k - len(above)]]))
+    assert (_sorted(out) == want).all()
