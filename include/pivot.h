@@ -22,6 +22,7 @@
  *   - Index output rows are SETS in unspecified order, no duplicates, every entry <= t.  When
  *     fewer than k keys are visible (dense / guarded rows only) the valid entries come first
  *     and the remainder is -1.
+ *   - A score that is not a number (a NaN among the operands that form it) ranks as -0.
  *   - Supported shapes: H_I = 64 indexer heads, d = 128, 1 <= k <= c <= 8192 (Refine) or
  *     1 <= k <= 8192 (Reuse / dense).  Anything else returns PIVOT_ERR_UNSUPPORTED.
  *   - Return value: PIVOT_OK or a positive error code; argument errors are detected on the host
@@ -360,12 +361,14 @@ int pivot_debug_counters(pivot_stream_t stream, unsigned long long* out, int n);
 /*
  * Per-stage timing, off by default.  While enabled, every call records CUDA events on its own
  * stream around its stages; pivot_stage_times synchronises on the last call's final event and
- * returns elapsed milliseconds: ms[0] proxy build (Eq. 4), ms[1] planner, ms[2] shared scan +
- * streaming select (Eq. 5-7, and the dense rows), ms[3] gather + re-score + top-k (Eq. 8-9),
- * ms[4] the whole call.  n must be at least 5; with n >= 6, ms[5] is the key-streaming scan kernel
+ * returns elapsed milliseconds: ms[0] the prepare kernel of a prefill (proxies of Eq. 4, row and
+ * group descriptors, the rows that select all they see), ms[1] about zero (the planner where it is a
+ * kernel of its own: decode with impl = 1), ms[2] shared scan + streaming select (Eq. 5-7, and the
+ * dense rows) with the merge of a chunk that is scanned in parts, ms[3] gather + re-score + top-k
+ * (Eq. 8-9), ms[4] the whole call.  n must be at least 5; with n >= 6, ms[5] is the key-streaming scan kernel
  * of the last decode call (0 if the last call was not a decode call) and, with n >= 7, ms[6] its
- * per-sequence top-c select kernel (Eq. 6 / Eq. 7).  For decode calls ms[2] covers scan, select,
- * re-score and top-k together.  Not thread-safe.
+ * per-sequence top-c select kernel (Eq. 6 / Eq. 7).  For decode calls ms[2] covers prepare, scan,
+ * select, re-score and top-k together.  Not thread-safe.
  */
 int pivot_stage_timing(int enable);
 int pivot_stage_times(float* ms, int n);

@@ -423,7 +423,8 @@ def pivot_stage_timing(enable: bool):
 
 
 def pivot_stage_times() -> dict:
-    """Elapsed ms of the last call's stages (needs pivot_stage_timing(True) before the call)."""
+    """Elapsed ms of the last call's stages (needs pivot_stage_timing(True) before the call).  For a prefill
+    "proxy_build" is the whole prepare kernel (proxies, plan, rows without a choice) and "plan" about zero."""
     ms = (C.c_float * 7)()
     _check(lib.pivot_stage_times(ms, 7))
     return dict(zip(("proxy_build", "plan", "scan_select", "refine", "total", "decode_scan", "decode_select"),

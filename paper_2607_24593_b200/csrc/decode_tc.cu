@@ -12,11 +12,12 @@
 //                        8192-bin histogram of the scores' top 13 key bits per sequence.
 //   decode_select_kernel a cluster of up to four 1024-thread CTAs per sequence: the histogram gives the
 //                        bin holding the K-th best score; each CTA collects the survivors of its
-//                        quarter of the score array in its shared memory; after a cluster barrier
-//                        CTA 0 reads the other three lists through distributed shared memory and
-//                        takes the exact top-K (Eq. 6 / 7) of the union.  If the boundary bin
-//                        leaves too many candidates, one CTA alone refines it 12 bits at a time
-//                        with further passes over the scores.
+//                        share of the score array in its shared memory and writes those above the
+//                        bin straight out; after a cluster barrier CTA 0 reads the other CTAs'
+//                        entries of the bin itself through distributed shared memory, ranks them
+//                        and adds the best (Eq. 6 / 7).  If the boundary bin holds too many
+//                        entries, one CTA alone takes the sequence, refining the bin 12 bits at a
+//                        time with further passes over the scores where its list needs that.
 //   decode_window_kernel (only with a local window, Appendix B) the union of the step's per-query
 //                        windows as one more candidate chunk per sequence, minus the positions
 //                        the pool already holds.
@@ -55,7 +56,7 @@ struct DCfg {
   static constexpr int STAGE_BYTES = KHALVES * HALF_TILE_BYTES;
   static constexpr int QHALF_BYTES = kHeads * 128;
   static constexpr int QBUF_BYTES = KHALVES * QHALF_BYTES;
-    static constexpr int STAGES = FP8 ? 8 : 3;
+  static constexpr int STAGES = FP8 ? 8 : 3;
   static constexpr uint32_t IDESC = ptx::make_idesc(FP8 ? 0u : 1u, TILE_KEYS, D_N);
 };
 

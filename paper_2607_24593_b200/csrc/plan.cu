@@ -187,11 +187,11 @@ prepare_prefill_kernel(const __grid_constant__ PrefillPlan p, RowDesc* rows, Gro
         p.merges[pr] = MergeRow{p.part_pos + (size_t)pr * p.split * whole.K, p.part_score + (size_t)pr * p.split * whole.K,
                                 p.split, tiles, whole.K, whole.out, whole.out_score, whole.out_rows, whole.out_stride};
     } else {         // (a split call has no rows without a choice)
-    if (p.skip_trivial && r.K > 0 && r.n_vis <= r.K && !r.out_score) {
-      fill[threadIdx.x] = FillRow{r.out, r.n_vis, r.K, r.out_rows, r.out_stride};
-      r.K = 0;
-    }
-    rows[slot] = r;
+      if (p.skip_trivial && r.K > 0 && r.n_vis <= r.K && !r.out_score) {
+        fill[threadIdx.x] = FillRow{r.out, r.n_vis, r.K, r.out_rows, r.out_stride};
+        r.K = 0;
+      }
+      rows[slot] = r;
     }
   }
   __syncthreads();

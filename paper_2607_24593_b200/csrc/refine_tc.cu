@@ -7,8 +7,9 @@
 // 128-byte-swizzled K-major layout the tensor core reads (cp.async, 16 bytes at a time).  The
 // epilogue is the scan's: one key per thread, ReLU, gate-weighted head sum, key scale.  Scores
 // go to a per-CTA buffer, from which each member's exact top-k is selected and written out:
-// by select warps while the next group is re-scored (FP8 prefill), by the epilogue warps after
-// the group's last tile (bf16), or by a later kernel (the candidate chunks of a decode step).
+// by select warps while the next group is re-scored (prefill), by the epilogue warps after the
+// group's last tile (FP8 with fp32 head sums), or by a later kernel (the candidate chunks of a
+// decode step).
 //
 // Warps: 0 = query TMA, 1 = MMA issuer + TMEM owner, 2-3 = gather producers, 4-11 = epilogue,
 // 12-15 (EPI = 3) = select warps, one per member.
