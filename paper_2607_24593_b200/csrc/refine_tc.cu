@@ -230,6 +230,11 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* grou
       // MMA2: the head sum of tile it-1 follows the first MMA of tile it (see the shared scan)
       bool pend = false;
       uint32_t pend_it = 0, pend_blk = 0, w_blk = 0xffffffffu;
+      // (descriptors by constants and the key tile waited for first, as there: 1507 -> 1414 clocks per tile in groups
+      // of 32 tiles)
+      const uint64_t k_desc = ptx::smem_desc_sw128(ptx::smem_u32(kring)), q_desc = ptx::smem_desc_sw128(ptx::smem_u32(qbuf));
+      // (first slab of the gate matrix: its rows 8..15 lie 4096 bytes on)
+      const uint64_t w_desc = ptx::smem_desc_sw128(ptx::smem_u32(ct.wmat)) + ((uint64_t)((4096 - 1024) >> 4) << 32);
       // (a -DPIVOT_PROF build times this thread's waits: PW(slot, wait) adds the wait's clocks to pw[slot])
       PIVOT_PROF_DO(long long pw[6] = {0, 0, 0, 0, 0, 0}; const long long pstart = clock64();)
 #ifdef PIVOT_PROF
@@ -251,15 +256,12 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* grou
         PW(4, oka = ptx::mbar_wait_poll(&ct.a_ready[pb], (pend_it >> 1) & 1, abort_flag))
         if (!oka) return false;
         ptx::tc_fence_after();
-        const uint32_t w_addr = ptx::smem_u32(ct.wmat);
         const uint32_t a_tmem = tmem_base + pb * N;
 #pragma unroll
         for (int ks = 0; ks < 16; ++ks) {        // 16 bf16 of K per step: 8 TMEM columns, 32 bytes of W
-          const int slab = ks >> 2;
-          uint64_t d = ptx::smem_desc_sw128(w_addr + slab * 1024 + (ks & 3) * 32);
-          d &= ~((uint64_t)0x3FFF << 32);        // rows 8..15 of the slab: the shared zero block
-          d |= (uint64_t)(((4096 - slab * 1024) >> 4) & 0x3FFF) << 32;
-          ptx::tc_mma_a_tmem_bf16(a_tmem + 128, a_tmem + ks * 8, d, C::IDESC2, ks ? 1u : 0u);
+          // a slab further on, and that much less far from there to the zero block that serves as rows 8..15
+          constexpr uint64_t slab = (1024 >> 4) - ((uint64_t)(1024 >> 4) << 32);
+          ptx::tc_mma_a_tmem_bf16(a_tmem + 128, a_tmem + ks * 8, w_desc + (ks >> 2) * slab + (ks & 3) * 2, C::IDESC2, ks ? 1u : 0u);
         }
         ptx::tc_commit(&ct.s_ready[pb]);
         return true;
@@ -270,26 +272,24 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* grou
         const int qb = blk % C::QBUFS;
         PW(0, ok = ptx::mbar_wait(&ct.q_full[qb], (blk / C::QBUFS) & 1, abort_flag, 32))
         if (!ok) break;
-        const uint32_t q_addr = ptx::smem_u32(qbuf + qb * C::QBUF_BYTES);
+        const uint64_t qd = q_desc + (uint32_t)((qb * C::QBUF_BYTES) >> 4);
         for (int t = 0; t < ntiles; ++t, ++it) {
           const int s = it % C::STAGES;
           const uint32_t ph = (it / C::STAGES) & 1;
           const int buf = it & 1;
-          PW(1, ok = ptx::mbar_wait_poll(&ct.tmem_empty[buf], ((it >> 1) & 1) ^ 1, abort_flag))
-          if (!ok) break;
           PW(2, ok = ptx::mbar_wait_poll(&ct.full[s], ph, abort_flag))
           if (!ok) break;
+          const uint64_t kd = k_desc + (uint32_t)((s * C::STAGE_BYTES) >> 4);
+          PW(1, ok = ptx::mbar_wait_poll(&ct.tmem_empty[buf], ((it >> 1) & 1) ^ 1, abort_flag))
+          if (!ok) break;
           ptx::tc_fence_after();
-          const uint32_t k_addr = ptx::smem_u32(kring + s * C::STAGE_BYTES);
           const uint32_t d_tmem = tmem_base + buf * N;
 #pragma unroll
           for (int h = 0; h < C::KHALVES; ++h)
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-              const uint64_t a = ptx::smem_desc_sw128(k_addr + h * C::HALF_TILE_BYTES + ks * 32);
-              const uint64_t bq = ptx::smem_desc_sw128(q_addr + h * C::QHALF_BYTES + ks * 32);
-              ptx::tc_mma<C::FP8>(d_tmem, a, bq, C::IDESC, (h | ks) ? 1u : 0u);
-            }
+            for (int ks = 0; ks < 4; ++ks)
+              ptx::tc_mma<C::FP8>(d_tmem, kd + ((h * C::HALF_TILE_BYTES + ks * 32) >> 4), qd + ((h * C::QHALF_BYTES + ks * 32) >> 4),
+                                  C::IDESC, (h | ks) ? 1u : 0u);
           ptx::tc_commit(&ct.empty[s]);
           ptx::tc_commit(&ct.tmem_full[buf]);
           if constexpr (C::MMA2) {
