@@ -198,11 +198,13 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* grou
       const int qb = blk % C::QBUFS;
       if (!ptx::mbar_wait(&ct.q_empty[qb], ((blk / C::QBUFS) & 1) ^ 1, abort_flag, 128)) break;
       if (leader) {
-        ptx::mbar_arrive_expect_tx(&ct.q_full[qb], gd.m * C::KHALVES * C::QROW_HALF_BYTES);
-        for (int r = 0; r < gd.m; ++r)
+        ptx::mbar_arrive_expect_tx(&ct.q_full[qb], C::QBUF_BYTES);
+        // members missing from the group take its last one's queries: the second MMA's sums run over all
+        // members' columns, and stale bytes (possibly NaN patterns) must not reach it
+        for (int r = 0; r < NMEM; ++r)
           for (int h = 0; h < C::KHALVES; ++h)
             ptx::tma_load_2d(qbuf + qb * C::QBUF_BYTES + h * C::QHALF_BYTES + r * C::QROW_HALF_BYTES, &tm_q,
-                             h * 64, (gd.q_row + r) * kHeads, &ct.q_full[qb]);
+                             h * 64, (gd.q_row + min(r, gd.m - 1)) * kHeads, &ct.q_full[qb]);
       }
       if constexpr (C::MMA2) {
         float wv[NMEM * kHeads / 32];
@@ -544,10 +546,6 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* grou
               for (int i = 0; i < 16; ++i)
                 pk[i] = (c & 1) ? ptx::relu_pack_bf16x2(__uint_as_float(vb[2 * i]), __uint_as_float(vb[2 * i + 1]))
                                 : ptx::relu_pack_bf16x2(__uint_as_float(va[2 * i]), __uint_as_float(va[2 * i + 1]));
-              if ((c >> 1) >= gd.m) {                          // members missing from the group: zeros (warp-uniform)
-#pragma unroll
-                for (int i = 0; i < 16; ++i) pk[i] = 0u;
-              }
               ptx::tmem_st_32x16(xb + c * 16, pk);
             }
             ptx::tmem_wait_st();

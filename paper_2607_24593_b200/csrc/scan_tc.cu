@@ -194,12 +194,11 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
         const int qb = blk % C::QBUFS;
         ok = ptx::mbar_wait(&ct.q_empty[qb], ((blk / C::QBUFS) & 1) ^ 1, abort_flag, 64);
         if (!ok) break;
-        int present = 0;
-        for (int r = 0; r < NROWS; ++r) present += (b * NROWS + r < n_rows) ? 1 : 0;
-        ptx::mbar_arrive_expect_tx(&ct.q_full[qb], present * C::KHALVES * C::QROW_HALF_BYTES);
+        // rows missing from the last block take its last row's queries: the second MMA's sums run over all
+        // rows' columns, and stale bytes (possibly NaN patterns) must not reach it
+        ptx::mbar_arrive_expect_tx(&ct.q_full[qb], C::QBUF_BYTES);
         for (int r = 0; r < NROWS; ++r) {
-          const int ri = b * NROWS + r;
-          if (ri >= n_rows) continue;
+          const int ri = min(b * NROWS + r, n_rows - 1);
           const CUtensorMap* tm = rows[ri].q_map ? &tm_q1 : &tm_q0;
           const int y = rows[ri].q_row * kHeads;
           for (int h = 0; h < C::KHALVES; ++h)
@@ -386,10 +385,6 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
           // ---- ReLU warps: turn the fp32 accumulator into bf16 ReLU values in place.  Thread =
           // key (TMEM lane); 32 columns at a time come in, 16 packed columns go back to the start
           // of the buffer (writes trail the reads: column 16 c + 16 <= 32 c + 32).
-          // Rows missing from a partial block have no queries in shared memory: whatever the first
-          // MMA made of the stale bytes there (possibly NaN) must not reach the second one, whose
-          // sums run over all 256 columns -- those columns are written as zeros.
-          const int present = n_rows - b * NROWS;
           for (int t = 0; t < ntiles; ++t, ++it) {
             const int buf = it & 1;
             (void)ptx::mbar_wait(&ct.tmem_full[buf], (it >> 1) & 1, abort_flag);
@@ -410,10 +405,6 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
               for (int i = 0; i < 16; ++i)
                 pk[i] = (c & 1) ? ptx::relu_pack_bf16x2(__uint_as_float(vb[2 * i]), __uint_as_float(vb[2 * i + 1]))
                                 : ptx::relu_pack_bf16x2(__uint_as_float(va[2 * i]), __uint_as_float(va[2 * i + 1]));
-              if ((c >> 1) >= present) {                       // chunk c holds heads of row c / 2 (warp-uniform)
-#pragma unroll
-                for (int i = 0; i < 16; ++i) pk[i] = 0u;
-              }
               ptx::tmem_st_32x16(xb + c * 16, pk);
             }
             ptx::tmem_wait_st();
