@@ -295,6 +295,29 @@ __device__ __forceinline__ uint32_t relu_pack_bf16x2(float lo, float hi) {
   asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
   return r;
 }
+// One warp's share of the ReLU pass over a 128 x 256 fp32 accumulator: bf16 ReLU values in place, thread = key (TMEM
+// lane of the warp's quarter, which xb names).  32 columns at a time come in, 16 packed columns go back to the start of
+// the buffer (writes trail the reads: column 16 c + 16 <= 32 c + 32).
+__device__ __forceinline__ void relu_pack_in_place(uint32_t xb) {
+  uint32_t va[32], vb[32];
+  tmem_ld_32x32_async(xb, va);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    if (c & 1) tmem_wait_ld_regs(vb);
+    else tmem_wait_ld_regs(va);
+    if (c + 1 < 8) {
+      if (c & 1) tmem_ld_32x32_async(xb + (c + 1) * 32, va);
+      else tmem_ld_32x32_async(xb + (c + 1) * 32, vb);
+    }
+    uint32_t pk[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      pk[i] = (c & 1) ? relu_pack_bf16x2(__uint_as_float(vb[2 * i]), __uint_as_float(vb[2 * i + 1]))
+                      : relu_pack_bf16x2(__uint_as_float(va[2 * i]), __uint_as_float(va[2 * i + 1]));
+    tmem_st_32x16(xb + c * 16, pk);
+  }
+  tmem_wait_st();
+}
 // MMA with the A operand in tensor memory (bf16 pairs per column: even k in the low half).
 __device__ __forceinline__ void tc_mma_a_tmem_bf16(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                                    uint32_t accumulate) {

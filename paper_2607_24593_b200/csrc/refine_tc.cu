@@ -530,25 +530,7 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* grou
             const int buf = it & 1;
             (void)ptx::mbar_wait(&ct.tmem_full[buf], (it >> 1) & 1, abort_flag);
             ptx::tc_fence_after();
-            const uint32_t xb = tmem_base + ((uint32_t)(lq * 32) << 16) + buf * N;
-            uint32_t va[32], vb[32];
-            ptx::tmem_ld_32x32_async(xb, va);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              if (c & 1) ptx::tmem_wait_ld_regs(vb);
-              else ptx::tmem_wait_ld_regs(va);
-              if (c + 1 < 8) {
-                if (c & 1) ptx::tmem_ld_32x32_async(xb + (c + 1) * 32, va);
-                else ptx::tmem_ld_32x32_async(xb + (c + 1) * 32, vb);
-              }
-              uint32_t pk[16];
-#pragma unroll
-              for (int i = 0; i < 16; ++i)
-                pk[i] = (c & 1) ? ptx::relu_pack_bf16x2(__uint_as_float(vb[2 * i]), __uint_as_float(vb[2 * i + 1]))
-                                : ptx::relu_pack_bf16x2(__uint_as_float(va[2 * i]), __uint_as_float(va[2 * i + 1]));
-              ptx::tmem_st_32x16(xb + c * 16, pk);
-            }
-            ptx::tmem_wait_st();
+            ptx::relu_pack_in_place(tmem_base + ((uint32_t)(lq * 32) << 16) + buf * N);
             ptx::tc_fence_before();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&ct.a_ready[buf]);

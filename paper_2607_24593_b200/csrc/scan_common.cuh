@@ -27,28 +27,58 @@ struct BlockIter {
   }
 };
 
-// Key tiles a block of nrows_blk consecutive scan rows needs (its longest live row), and the
-// first key-tensor row of the block's sequence.
-__device__ __forceinline__ int block_tiles(const RowDesc* rows, int n_rows, int b, int nrows_blk, int* k_row0,
-                                           int* nv_max = nullptr) {
-  int mx = 0;
-  for (int r = 0; r < nrows_blk; ++r) {
-    const int ri = b * nrows_blk + r;
-    if (ri < n_rows) {
-      const int K = rows[ri].K;
-      const int nv = rows[ri].n_vis;
-      if (K > 0 && nv > mx) mx = nv;
-      if (r == 0) *k_row0 = rows[ri].k_row0;
-    }
+// What the roles of a CTA need to know about one of its row blocks.  The thread that loads the keys, several tiles ahead
+// of everybody else, looks it up and leaves it in a small ring in shared memory: a block's descriptors are chains of
+// global loads, and looked up by every role at the start of its block they left the tensor core idle for some three
+// tiles' time, a seventh of a block of a dozen tiles.  (The producer's whole warp fetching the gates as well, a block
+// ahead, starved the key ring: packed batch +4 %, dense 16K +14 %.)
+constexpr int kBlockSlots = 4;
+template <int NROWS>
+struct BlockInfo {
+  int b;                      // block index, -1: no more blocks
+  int ntiles, k_row0;         // key tiles (of its longest live row), first key-tensor row of its sequence
+  int n_vis[NROWS], K[NROWS]; // 0: no such row, or nothing to select
+  const float* w[NROWS];      // gates and their scales (K > 0)
+  const float* qscale[NROWS];
+};
+template <int NROWS>
+struct BlockRing {
+  BlockInfo<NROWS> info[kBlockSlots];
+  uint64_t full[kBlockSlots], empty[kBlockSlots];
+};
+
+// The consumers' side: block number n's info, nullptr at the end (or if the wait ran out).  Every consumer warp
+// arrives on empty[slot] once it needs it no more.  next_block: one thread; next_block_warp: a whole warp, whose
+// lanes agree on the outcome.
+template <int NROWS>
+__device__ __forceinline__ const BlockInfo<NROWS>* next_block(BlockRing<NROWS>& ring, uint32_t n, volatile int* abort_flag) {
+  const int slot = n % kBlockSlots;
+  const bool ok = ptx::mbar_wait(&ring.full[slot], (n / kBlockSlots) & 1, abort_flag, 32);
+  return ok && ring.info[slot].b >= 0 ? &ring.info[slot] : nullptr;
+}
+template <int NROWS>
+__device__ __forceinline__ const BlockInfo<NROWS>* next_block_warp(BlockRing<NROWS>& ring, uint32_t n, volatile int* abort_flag) {
+  const BlockInfo<NROWS>* const f = next_block(ring, n, abort_flag);
+  return __all_sync(0xffffffffu, f != nullptr) ? f : nullptr;
+}
+
+// One of a block's effective gates (fl32(w * qscale)), as the two loads that it takes: a row that selects nothing has
+// gates of 0, proxies no scale.
+struct GateLoad { float w, qscale; };
+template <int NROWS>
+__device__ __forceinline__ GateLoad load_gate(const BlockInfo<NROWS>& f, int r, int j) {
+  GateLoad g{0.f, 1.f};
+  if (f.K[r] > 0) {
+    g.w = f.w[r][j];
+    if (f.qscale[r]) g.qscale = f.qscale[r][j];
   }
-  if (nv_max) *nv_max = mx;
-  return (mx + TILE_KEYS - 1) / TILE_KEYS;
+  return g;
 }
 
 // Shared-memory state of the streaming select of a block of NROWS rows.
 template <int NROWS, int QD>
 struct SelectCtrl {
-  uint32_t rhist[NROWS][kSelBins];      // per row: histogram of every score appended so far
+  alignas(16) uint32_t rhist[NROWS][kSelBins];      // per row: histogram of every score appended so far
   uint64_t sc_full[QD], sc_empty[QD];   // survivor queues: score warps -> append warps
   alignas(16) unsigned long long q[QD][NROWS][4][32];   // [tile % QD][row][lane quarter]: packed entries
   alignas(16) uint32_t qn[QD][NROWS][4];                // their counts
@@ -58,6 +88,7 @@ struct SelectCtrl {
   // End of a block: what the row's finisher needs (the append warp moves on to the next block
   // and the row's other segment at once).  Two slots, used by alternate blocks like the segments.
   struct FinRow {
+    int b;                              // the block, -1: no more
     int cnt;                            // entries held in the row's segment
     int base;                           // the row histogram's anchor
     int bsel;                           // boundary bin of the exact histogram, -1 = everything is wanted
@@ -120,8 +151,7 @@ __device__ __forceinline__ uint32_t select_bin_lo(int bin, int base) {
 // the next block in the row's other segment.
 template <int NROWS, int QD>
 __device__ __noinline__ void append_role(SelectCtrl<NROWS, QD>& s, int r, int lane, const Team& tm,
-                                            const RowDesc* rows, int n_rows, int n_blocks,
-                                            const ScanScratch& sc, volatile int* abort_flag) {
+                                            BlockRing<NROWS>& ring, const ScanScratch& sc, volatile int* abort_flag) {
   SegSelSmem& sel = s.sel[r];
   const int CAP = sc.cap;                        // entries of this row's candidate segment
   uint32_t* const rhist = s.rhist[r];
@@ -130,25 +160,22 @@ __device__ __noinline__ void append_role(SelectCtrl<NROWS, QD>& s, int r, int la
   // only keys > t can still belong to the top K.
   auto hist_threshold = [&](int K, int base) -> uint32_t {
     uint32_t b, need_in, pop;
-    if (!warp_hist_boundary<2>(rhist, (uint32_t)K, lane, &b, &need_in, &pop)) return 0u;
+    if (!warp_hist_boundary(rhist, (uint32_t)K, lane, &b, &need_in, &pop)) return 0u;
     return b > 0 ? (((uint32_t)((int)b + base)) << 15) - 1u : 0u;
   };
   // The threshold is refreshed every CHK tiles; a tile adds at most TILE_KEYS entries, so a
   // segment checked then always has room until the next check.
   const int CHK = CAP / (2 * TILE_KEYS) < kThresholdRefreshTiles ? (CAP / (2 * TILE_KEYS) > 0 ? CAP / (2 * TILE_KEYS) : 1) : kThresholdRefreshTiles;
   const int headroom = TILE_KEYS * CHK;
-  BlockIter bi(n_blocks, gridDim.x, blockIdx.x);
   uint32_t it = 0, seq = 0;
-  for (int b = bi.next(); b >= 0; b = bi.next()) {
-    int k_row0 = 0;
-    const int ntiles = block_tiles(rows, n_rows, b, NROWS, &k_row0);
-    if (ntiles == 0) continue;
-    const int ri = b * NROWS + r;
-    const bool live = ri < n_rows && rows[ri].K > 0;
-    const int K = live ? rows[ri].K : 0;
+  while (const BlockInfo<NROWS>* const info = next_block_warp(ring, seq, abort_flag)) {
+    const int b = info->b, ntiles = info->ntiles, K = info->K[r];
+    __syncwarp();
+    if (lane == 0) ptx::mbar_arrive(&ring.empty[seq % kBlockSlots]);
     int cnt = 0, base = 0;
     uint32_t thr = 0;
-    for (int i = lane; i < kSelBins; i += 32) rhist[i] = 0;
+#pragma unroll 4
+    for (int i = lane; i < kSelBins / 4; i += 32) reinterpret_cast<uint4*>(rhist)[i] = make_uint4(0, 0, 0, 0);
     if (lane == 0) s.thr[r] = (unsigned long long)seq << 32;
     // this block's segment was the block's before last: its finisher must be through with it
     const int fb = seq & 1;
@@ -237,15 +264,21 @@ __device__ __noinline__ void append_role(SelectCtrl<NROWS, QD>& s, int r, int la
     // ---- end of the block: the histogram is exact for everything the segment still holds; read
     //      the boundary bin off it and hand the row to its finisher
     uint32_t bb = 0, need_b = 0, pop = 0;
-    const bool found = K > 0 && warp_hist_boundary<0>(rhist, (uint32_t)K, lane, &bb, &need_b, &pop);
+    const bool found = K > 0 && warp_hist_boundary(rhist, (uint32_t)K, lane, &bb, &need_b, &pop);
     if (lane == 0) {
       typename SelectCtrl<NROWS, QD>::FinRow& f = s.fin[r][fb];
-      f.cnt = cnt; f.base = base; f.bsel = found ? (int)bb : -1; f.need_b = need_b; f.pop = pop;
+      f.b = b; f.cnt = cnt; f.base = base; f.bsel = found ? (int)bb : -1; f.need_b = need_b; f.pop = pop;
     }
     __threadfence_block();
     __syncwarp();
     if (lane == 0) ptx::mbar_arrive(&s.fin_full[r][fb]);
     ++seq;
+  }
+  // no more blocks (or a wait ran out)
+  (void)ptx::mbar_wait(&s.fin_done[r][seq & 1], ((seq >> 1) & 1) ^ 1, abort_flag, 64);
+  if (lane == 0) {
+    s.fin[r][seq & 1].b = -1;
+    ptx::mbar_arrive(&s.fin_full[r][seq & 1]);
   }
 }
 
@@ -256,16 +289,14 @@ __device__ __noinline__ void append_role(SelectCtrl<NROWS, QD>& s, int r, int la
 // Reuse group.
 template <int NROWS, int QD>
 __device__ __noinline__ void finisher_role(SelectCtrl<NROWS, QD>& s, int r0, int nr, int lane,
-                                              const RowDesc* rows, int n_rows, int n_blocks,
-                                              const ScanScratch& sc, volatile int* abort_flag) {
-  BlockIter bi(n_blocks, gridDim.x, blockIdx.x);
-  uint32_t seq = 0;
-  for (int b = bi.next(); b >= 0; b = bi.next()) {
-    int k_row0 = 0;
-    if (block_tiles(rows, n_rows, b, NROWS, &k_row0) == 0) continue;
+                                              const RowDesc* rows, int n_rows, const ScanScratch& sc,
+                                              volatile int* abort_flag) {
+  for (uint32_t seq = 0;; ++seq) {
     const int fb = seq & 1;
     for (int r = r0; r < r0 + nr; ++r) {
-      if (!ptx::mbar_wait(&s.fin_full[r][fb], (seq >> 1) & 1, abort_flag, 64)) return;
+      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&s.fin_full[r][fb], (seq >> 1) & 1, abort_flag, 64))) return;
+      const int b = s.fin[r][fb].b;
+      if (b < 0) return;
       const int ri = b * NROWS + r;
       const int K = (ri < n_rows) ? rows[ri].K : 0;
       if (K > 0) {
@@ -301,7 +332,6 @@ __device__ __noinline__ void finisher_role(SelectCtrl<NROWS, QD>& s, int r0, int
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&s.fin_done[r][fb]);
     }
-    ++seq;
   }
 }
 

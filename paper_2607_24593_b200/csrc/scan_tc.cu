@@ -45,7 +45,6 @@ namespace {
 using scan::TILE_KEYS;
 using scan::KS_SLOTS;
 using scan::BlockIter;
-using scan::block_tiles;
 constexpr int MAX_STAGES = 8;
 constexpr int QDEPTH = 4;         // survivor-queue buffers between the score warps and the append warps
 
@@ -94,7 +93,8 @@ struct Ctrl {
   alignas(1024) uint8_t wmat[MMA2 ? 8192 : 16];
   uint64_t a_ready[2], s_ready[2], w_ready;      // MMA2 handshakes (see the kernel)
   alignas(128) float ks[KS_SLOTS][TILE_KEYS];   // key scales of the tiles in flight (TMA destination)
-  alignas(16) float w[4][kHeads];       // effective gates of the block's rows (read as float4)
+  scan::BlockRing<NROWS> ring;          // the CTA's next blocks
+  alignas(16) float w[MMA2 ? 1 : NROWS == 4 ? 8 : 4][MMA2 ? 4 : (NROWS == 4 ? 2 : 1) * kHeads];   // fp32 head sum: each score warp's gates (read as float4)
   uint64_t full[MAX_STAGES], empty[MAX_STAGES];
   uint64_t q_full[2], q_empty[2], tmem_full[2], tmem_empty[2];
   uint64_t ks_full[KS_SLOTS];
@@ -110,6 +110,107 @@ constexpr size_t smem_bytes() {
 }
 static_assert(smem_bytes<DT_FP8, 4, 1>() <= 232448 && smem_bytes<DT_FP8, 4, 0>() <= 232448 &&
               smem_bytes<DT_BF16, 4>() <= 232448, "shared memory budget");
+
+// The two kinds of score warps where the head sum runs on the tensor core, functions of their own so that
+// neither's registers are allocated around the other's (inlined, with the block ring: spills in both loops, 64K Reuse
+// 6.14 ms against 5.78, dense 16K 1650 us against 1467).  Every hand-over is an mbarrier: a wait that ran out may end any
+// warp's loop by itself.
+
+// ReLU warps: turn the fp32 accumulator into bf16 ReLU values in place.
+template <int NROWS>
+__device__ __noinline__ void relu_role(Ctrl<NROWS, true>& ct, uint32_t tmem_base, int lq, int lane) {
+  volatile int* abort_flag = &ct.abort;
+  uint32_t it = 0;
+  for (uint32_t seq = 0;; ++seq) {
+    const scan::BlockInfo<NROWS>* const info = scan::next_block_warp(ct.ring, seq, abort_flag);
+    if (!info) return;
+    const int ntiles = info->ntiles;
+    __syncwarp();
+    if (lane == 0) ptx::mbar_arrive(&ct.ring.empty[seq % scan::kBlockSlots]);
+    for (int t = 0; t < ntiles; ++t, ++it) {
+      const int buf = it & 1;
+      (void)ptx::mbar_wait(&ct.tmem_full[buf], (it >> 1) & 1, abort_flag);
+      ptx::tc_fence_after();
+      ptx::relu_pack_in_place(tmem_base + ((uint32_t)(lq * 32) << 16) + buf * (NROWS * kHeads));
+      ptx::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&ct.a_ready[buf]);
+    }
+  }
+}
+
+// Compact warps: read the four row scores of this thread's key, free the accumulator buffer, leave the survivors in
+// the row queues.  They also put every block's gates into the gate matrix.
+template <int NROWS>
+__device__ __noinline__ void compact_role(Ctrl<NROWS, true>& ct, uint32_t tmem_base, int lq, int wq, int lane) {
+  constexpr int QD = Ctrl<NROWS, true>::QD;
+  volatile int* abort_flag = &ct.abort;
+  const int key_in_tile = lq * 32 + lane;
+  uint32_t it = 0;
+  scan::GateLoad gate[2];                            // the next block's: heads lane and 32 + lane of row wq
+  const scan::BlockInfo<NROWS>* info = scan::next_block_warp(ct.ring, 0, abort_flag);
+  auto fetch_gates = [&]() {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) gate[u] = scan::load_gate(*info, wq, u * 32 + lane);
+  };
+  if (info) fetch_gates();
+  for (uint32_t seq = 0; info; ++seq) {
+    const int ntiles = info->ntiles;
+    int nv4[NROWS];
+#pragma unroll
+    for (int r = 0; r < NROWS; ++r) nv4[r] = info->n_vis[r];
+    // The block's gates: the four diagonal blocks of the gate matrix.  The last second MMA of the block before
+    // is through (this warp has read its scores); the first of this one waits for all four warps.
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int r = wq, j = u * 32 + lane;
+      const float wv = __fmul_rn(gate[u].w, gate[u].qscale);
+      // gate = hi + lo in bf16: matrix rows r and 4 + r (both inside slab r, the row's 64 columns)
+      const __nv_bfloat16 hi = __float2bfloat16_rn(wv);
+      const __nv_bfloat16 lo = __float2bfloat16_rn(wv - __bfloat162float(hi));
+      uint8_t* const p = ct.wmat + r * 2048 + (j & 7) * 2;
+      *reinterpret_cast<__nv_bfloat16*>(p + r * 128 + (((j >> 3) ^ (r & 7)) << 4)) = hi;
+      *reinterpret_cast<__nv_bfloat16*>(p + (4 + r) * 128 + (((j >> 3) ^ ((4 + r) & 7)) << 4)) = lo;
+    }
+    ptx::fence_proxy_async_smem();                   // generic-proxy writes -> tensor-core reads
+    __syncwarp();
+    if (lane == 0) { ptx::mbar_arrive(&ct.w_ready); ptx::mbar_arrive(&ct.ring.empty[seq % scan::kBlockSlots]); }
+    for (int t = 0, end = ntiles - 1; t < ntiles; end = ntiles) {
+      if (t == ntiles - 1) {       // the last tile is on its way: so are the next block's gates
+        info = scan::next_block_warp(ct.ring, seq + 1, abort_flag);
+        if (info) fetch_gates();
+        end = ntiles;
+      }
+      for (; t < end; ++t, ++it) {
+        const int buf = it & 1;
+        const int ksl = it % KS_SLOTS;
+        (void)ptx::mbar_wait(&ct.ks_full[ksl], (it / KS_SLOTS) & 1, abort_flag);
+        const float ksv = ct.ks[ksl][key_in_tile];
+        (void)ptx::mbar_wait(&ct.s_ready[buf], (it >> 1) & 1, abort_flag);
+        ptx::tc_fence_after();
+        uint32_t sv[8];          // columns r: sum with the gates' bf16 heads, 4 + r: with their remainders
+        ptx::tmem_ld_32x8(tmem_base + ((uint32_t)(lq * 32) << 16) + buf * (NROWS * kHeads) + 128, sv);
+        ptx::tmem_wait_ld();
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&ct.tmem_empty[buf]);
+        const int qb = it % QD;
+        (void)ptx::mbar_wait(&ct.s.sc_empty[qb], ((it / QD) & 1) ^ 1, abort_flag);
+        const int s_key = t * TILE_KEYS + key_in_tile;
+        uint32_t key[NROWS];
+        bool take[NROWS];
+#pragma unroll
+        for (int r = 0; r < NROWS; ++r) {
+          key[r] = score_to_key((__uint_as_float(sv[r]) + __uint_as_float(sv[4 + r])) * ksv);
+          take[r] = s_key < nv4[r] && key[r] > scan::row_threshold(ct.s, r, seq);
+        }
+        scan::push_survivors<NROWS>(ct.s, qb, 0, lq, lane, take, key, s_key);
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&ct.s.sc_full[qb]);
+      }
+    }
+  }
+}
 
 template <int DT, int NROWS, int EPI>
 __global__ void __launch_bounds__(Cfg<DT, NROWS, EPI>::THREADS, 1)
@@ -151,7 +252,11 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
       ptx::mbar_init(&ct.a_ready[i], 4);
       ptx::mbar_init(&ct.s_ready[i], 1);
     }
-    ptx::mbar_init(&ct.w_ready, 1);
+    ptx::mbar_init(&ct.w_ready, 4);
+    for (int i = 0; i < scan::kBlockSlots; ++i) {
+      ptx::mbar_init(&ct.ring.full[i], 1);
+      ptx::mbar_init(&ct.ring.empty[i], 1 + C::EPI_WARPS + C::SEL_WARPS);
+    }
     for (int i = 0; i < KS_SLOTS; ++i) ptx::mbar_init(&ct.ks_full[i], 1);
     for (int i = 0; i < QD; ++i) {
       ptx::mbar_init(&ct.s.sc_full[i], C::SC_FULL_ARRIVALS);
@@ -187,24 +292,50 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
       BlockIter bi(n_blocks, gridDim.x, blockIdx.x);
       uint32_t it = 0, blk = 0;
       bool ok = true;
-      for (int b = bi.next(); b >= 0 && ok; b = bi.next()) {
-        int k_row0 = 0;
-        const int ntiles = block_tiles(rows, n_rows, b, NROWS, &k_row0);
-        if (ntiles == 0) continue;
+      for (bool more = true; more && ok;) {
+        const int b = bi.next();
+        more = b >= 0;
+        // rows missing from the last block take its last row's queries (and no gates): the tensor core's head sum
+        // runs over the columns of all four rows, and stale bytes (possibly NaN patterns) must not reach it
+        int n_vis[NROWS], K[NROWS], q_row[NROWS], q_map[NROWS], k_row0 = 0, ntiles = 0;
+        const float *w[NROWS], *qscale[NROWS];
+        if (more) {
+          int mx = 0;
+#pragma unroll
+          for (int r = 0; r < NROWS; ++r) {
+            const RowDesc& rd = rows[min(b * NROWS + r, n_rows - 1)];
+            K[r] = b * NROWS + r < n_rows ? rd.K : 0;
+            n_vis[r] = rd.n_vis; q_row[r] = rd.q_row; q_map[r] = rd.q_map; w[r] = rd.w; qscale[r] = rd.qscale;
+            if (r == 0) k_row0 = rd.k_row0;
+          }
+#pragma unroll
+          for (int r = 0; r < NROWS; ++r) {
+            n_vis[r] = K[r] > 0 ? n_vis[r] : 0;
+            mx = n_vis[r] > mx ? n_vis[r] : mx;
+          }
+          ntiles = (mx + TILE_KEYS - 1) / TILE_KEYS;
+          if (ntiles == 0) continue;
+        }
+        const int slot = blk % scan::kBlockSlots;
+        ok = ptx::mbar_wait(&ct.ring.empty[slot], ((blk / scan::kBlockSlots) & 1) ^ 1, abort_flag, 64);
+        if (!ok) break;
+        scan::BlockInfo<NROWS>& f = ct.ring.info[slot];
+        f.b = b; f.ntiles = ntiles; f.k_row0 = k_row0;
+        if (more) {
+#pragma unroll
+          for (int r = 0; r < NROWS; ++r) { f.n_vis[r] = n_vis[r]; f.K[r] = K[r]; f.w[r] = w[r]; f.qscale[r] = qscale[r]; }
+        }
+        ptx::mbar_arrive(&ct.ring.full[slot]);
+        if (!more) break;
         const int qb = blk % C::QBUFS;
         ok = ptx::mbar_wait(&ct.q_empty[qb], ((blk / C::QBUFS) & 1) ^ 1, abort_flag, 64);
         if (!ok) break;
-        // rows missing from the last block take its last row's queries: the second MMA's sums run over all
-        // rows' columns, and stale bytes (possibly NaN patterns) must not reach it
         ptx::mbar_arrive_expect_tx(&ct.q_full[qb], C::QBUF_BYTES);
-        for (int r = 0; r < NROWS; ++r) {
-          const int ri = min(b * NROWS + r, n_rows - 1);
-          const CUtensorMap* tm = rows[ri].q_map ? &tm_q1 : &tm_q0;
-          const int y = rows[ri].q_row * kHeads;
+#pragma unroll
+        for (int r = 0; r < NROWS; ++r)
           for (int h = 0; h < C::KHALVES; ++h)
-            ptx::tma_load_2d(qbuf + qb * C::QBUF_BYTES + h * C::QHALF_BYTES + r * C::QROW_HALF_BYTES, tm,
-                             h * 64, y, &ct.q_full[qb]);
-        }
+            ptx::tma_load_2d(qbuf + qb * C::QBUF_BYTES + h * C::QHALF_BYTES + r * C::QROW_HALF_BYTES,
+                             q_map[r] ? &tm_q1 : &tm_q0, h * 64, q_row[r] * kHeads, &ct.q_full[qb]);
         for (int t = 0; t < ntiles; ++t, ++it) {
           const int s = it % C::STAGES;
           const uint32_t ph = (it / C::STAGES) & 1;
@@ -229,7 +360,6 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     if (ptx::elect_one()) {
-      BlockIter bi(n_blocks, gridDim.x, blockIdx.x);
       uint32_t it = 0, blk = 0;
       bool ok = true;
       // MMA2: the gate-weighted head sum of tile it-1, S[128 keys x 16] = ReLU(X)[128 x 256] . W^T,
@@ -270,10 +400,11 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
         ptx::tc_commit(&ct.s_ready[pb]);
         return true;
       };
-      for (int b = bi.next(); b >= 0 && ok; b = bi.next()) {
-        int k_row0 = 0;
-        const int ntiles = block_tiles(rows, n_rows, b, NROWS, &k_row0);
-        if (ntiles == 0) continue;
+      while (ok) {
+        const scan::BlockInfo<NROWS>* const info = scan::next_block(ct.ring, blk, abort_flag);
+        if (!info) break;
+        const int ntiles = info->ntiles;
+        ptx::mbar_arrive(&ct.ring.empty[blk % scan::kBlockSlots]);
         const int qb = blk % C::QBUFS;
         PW(0, ok = ptx::mbar_wait(&ct.q_full[qb], (blk / C::QBUFS) & 1, abort_flag, 32))
         if (!ok) break;
@@ -322,134 +453,28 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
     const int wq = ew & 3;
     const int lq = warp & 3;                       // TMEM lane quarter this warp may read
     const int key_in_tile = lq * 32 + lane;
-    const int tt = wq * 32 + lane;                 // rank inside the team (0..127)
-    const Team tm{tt, 128, 1 + team};
-    BlockIter bi(n_blocks, gridDim.x, blockIdx.x);
-    uint32_t it = 0, seq = 0xffffffffu;            // seq: this block's sequence number in the CTA
-    // A failed wait never changes this role's control flow (the team barriers below must stay
-    // matched); once the abort flag is up every later wait returns at once.
-    for (int b = bi.next(); b >= 0; b = bi.next()) {
-      int k_row0 = 0;
-      const int ntiles = block_tiles(rows, n_rows, b, NROWS, &k_row0);
-      if (ntiles == 0) continue;
-      ++seq;
-      // ---- effective gates of this team's rows
-      tm.sync();
-      if constexpr (C::MMA2) {
-        // team 1 (the compact warps) writes the four diagonal blocks of the gate matrix; the last
-        // second MMA of the previous block is through (its scores have been read)
-        if (team == 1) {
+    uint32_t it = 0, seq = 0;                      // seq: this block's sequence number in the CTA
+    if constexpr (C::MMA2) {
+      if (team == 0) relu_role(ct, tmem_base, lq, lane);
+      else compact_role(ct, tmem_base, lq, wq, lane);
+    } else {
+    // (every hand-over of this role is an mbarrier: a wait that ran out may end any warp's loop by itself)
+    // Each warp keeps a copy of its rows' gates in shared memory.
+    const scan::BlockInfo<NROWS>* info = scan::next_block_warp(ct.ring, 0, abort_flag);
+    while (info) {
+      const int ntiles = info->ntiles;
+      const int slot = seq % scan::kBlockSlots;
+      constexpr int GPT = C::ROWS_PER_TEAM * kHeads / 32;
+      scan::GateLoad gate[GPT];
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int i = tt + u * 128, r = i >> 6, j = i & 63;
-            const int ri = b * NROWS + r;
-            float wv = 0.f;
-            if (ri < n_rows && rows[ri].K > 0) {
-              wv = rows[ri].w[j];
-              if (rows[ri].qscale) wv = __fmul_rn(wv, rows[ri].qscale[j]);
-            }
-            // gate = hi + lo in bf16: matrix rows r and 4 + r (both inside slab r, the row's 64 columns)
-            const __nv_bfloat16 hi = __float2bfloat16_rn(wv);
-            const __nv_bfloat16 lo = __float2bfloat16_rn(wv - __bfloat162float(hi));
-            const uint32_t in_row = (j & 7) * 2;
-            *reinterpret_cast<__nv_bfloat16*>(ct.wmat + r * 2048 + r * 128 + (((j >> 3) ^ (r & 7)) << 4) + in_row) = hi;
-            *reinterpret_cast<__nv_bfloat16*>(ct.wmat + r * 2048 + (4 + r) * 128 + (((j >> 3) ^ ((4 + r) & 7)) << 4) + in_row) = lo;
-          }
-          ptx::fence_proxy_async_smem();         // generic-proxy writes -> tensor-core reads
-          tm.sync();
-          if (tt == 0) ptx::mbar_arrive(&ct.w_ready);
-        }
-      } else {
-        const int rl = tt >> 6, j = tt & 63;
-        if (rl < C::ROWS_PER_TEAM) {
-          const int r = team * C::ROWS_PER_TEAM + rl;
-          const int ri = b * NROWS + r;
-          float wv = 0.f;
-          if (ri < n_rows && rows[ri].K > 0) {
-            wv = rows[ri].w[j];
-            if (rows[ri].qscale) wv = __fmul_rn(wv, rows[ri].qscale[j]);
-          }
-          ct.w[r][j] = wv;
-        }
-      }
+      for (int u = 0; u < GPT; ++u) gate[u] = scan::load_gate(*info, team * C::ROWS_PER_TEAM + u / 2, (u & 1) * 32 + lane);
       int n_vis[C::ROWS_PER_TEAM];
 #pragma unroll
-      for (int rl = 0; rl < C::ROWS_PER_TEAM; ++rl) {
-        const int ri = b * NROWS + team * C::ROWS_PER_TEAM + rl;
-        const bool live = ri < n_rows && rows[ri].K > 0;
-        n_vis[rl] = live ? rows[ri].n_vis : 0;
-      }
-      tm.sync();
-      if constexpr (C::MMA2) {
-        if (team == 0) {
-          // ---- ReLU warps: turn the fp32 accumulator into bf16 ReLU values in place.  Thread =
-          // key (TMEM lane); 32 columns at a time come in, 16 packed columns go back to the start
-          // of the buffer (writes trail the reads: column 16 c + 16 <= 32 c + 32).
-          for (int t = 0; t < ntiles; ++t, ++it) {
-            const int buf = it & 1;
-            (void)ptx::mbar_wait(&ct.tmem_full[buf], (it >> 1) & 1, abort_flag);
-            ptx::tc_fence_after();
-            const uint32_t xb = tmem_base + ((uint32_t)(lq * 32) << 16) + buf * C::N;
-            uint32_t va[32], vb[32];
-            ptx::tmem_ld_32x32_async(xb, va);
+      for (int rl = 0; rl < C::ROWS_PER_TEAM; ++rl) n_vis[rl] = info->n_vis[team * C::ROWS_PER_TEAM + rl];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              if (c & 1) ptx::tmem_wait_ld_regs(vb);
-              else ptx::tmem_wait_ld_regs(va);
-              if (c + 1 < 8) {
-                if (c & 1) ptx::tmem_ld_32x32_async(xb + (c + 1) * 32, va);
-                else ptx::tmem_ld_32x32_async(xb + (c + 1) * 32, vb);
-              }
-              uint32_t pk[16];
-#pragma unroll
-              for (int i = 0; i < 16; ++i)
-                pk[i] = (c & 1) ? ptx::relu_pack_bf16x2(__uint_as_float(vb[2 * i]), __uint_as_float(vb[2 * i + 1]))
-                                : ptx::relu_pack_bf16x2(__uint_as_float(va[2 * i]), __uint_as_float(va[2 * i + 1]));
-              ptx::tmem_st_32x16(xb + c * 16, pk);
-            }
-            ptx::tmem_wait_st();
-            ptx::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&ct.a_ready[buf]);
-          }
-        } else {
-          // ---- compact warps: read the four row scores of this thread's key, free the
-          // accumulator buffer, leave the survivors in the row queues
-          int nv4[NROWS];
-#pragma unroll
-          for (int r = 0; r < NROWS; ++r) {
-            const int ri = b * NROWS + r;
-            nv4[r] = (ri < n_rows && rows[ri].K > 0) ? rows[ri].n_vis : 0;
-          }
-          for (int t = 0; t < ntiles; ++t, ++it) {
-            const int buf = it & 1;
-            const int ksl = it % KS_SLOTS;
-            (void)ptx::mbar_wait(&ct.ks_full[ksl], (it / KS_SLOTS) & 1, abort_flag);
-            const float ksv = ct.ks[ksl][key_in_tile];
-            (void)ptx::mbar_wait(&ct.s_ready[buf], (it >> 1) & 1, abort_flag);
-            ptx::tc_fence_after();
-            uint32_t sv[8];          // columns r: sum with the gates' bf16 heads, 4 + r: with their remainders
-            ptx::tmem_ld_32x8(tmem_base + ((uint32_t)(lq * 32) << 16) + buf * C::N + 128, sv);
-            ptx::tmem_wait_ld();
-            ptx::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&ct.tmem_empty[buf]);
-            const int qb = it % QD;
-            (void)ptx::mbar_wait(&ct.s.sc_empty[qb], ((it / QD) & 1) ^ 1, abort_flag);
-            const int s_key = t * TILE_KEYS + key_in_tile;
-            uint32_t key[NROWS];
-            bool take[NROWS];
-#pragma unroll
-            for (int r = 0; r < NROWS; ++r) {
-              key[r] = score_to_key((__uint_as_float(sv[r]) + __uint_as_float(sv[4 + r])) * ksv);
-              take[r] = s_key < nv4[r] && key[r] > scan::row_threshold(ct.s, r, seq);
-            }
-            scan::push_survivors<NROWS>(ct.s, qb, 0, lq, lane, take, key, s_key);
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&ct.s.sc_full[qb]);
-          }
-        }
-      } else
+      for (int u = 0; u < GPT; ++u) ct.w[ew][u * 32 + lane] = __fmul_rn(gate[u].w, gate[u].qscale);
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&ct.ring.empty[slot]);
       for (int t = 0; t < ntiles; ++t, ++it) {
         const int buf = it & 1;
         // Key scales come through shared memory (TMA): a global load issued by this warp would
@@ -479,7 +504,7 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
             else ptx::tmem_ld_32x32_async(tbase + (c + 1) * 32, vb);
           }
           if ((c & 1) == 0) acc[0] = acc[1] = acc[2] = acc[3] = 0ull;
-          const float* wrow = &ct.w[team * C::ROWS_PER_TEAM + (c >> 1)][(c & 1) * 32];
+          const float* wrow = &ct.w[ew][(c >> 1) * kHeads + (c & 1) * 32];
           if (c & 1) ptx::relu_dot32(vb, wrow, acc);
           else ptx::relu_dot32(va, wrow, acc);
           if (c & 1) score[c >> 1] = ptx::relu_dot_sum(acc);
@@ -502,17 +527,21 @@ scan_select_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&ct.s.sc_full[qb]);
       }
+      __syncwarp();                                // (nobody reads these gates any more)
+      ++seq;
+      info = scan::next_block_warp(ct.ring, seq, abort_flag);
       // (the rows' final exact select is the finisher warps' business: on to the next block)
+    }
     }
   } else if (warp < 2 + C::EPI_WARPS + C::SEL_WARPS) {
     // ------------------------------------------------------------------ append warps: one row each
     const int r = warp - 2 - C::EPI_WARPS;
-    scan::append_role(ct.s, r, lane, Team{lane, 32, 3 + r}, rows, n_rows, n_blocks, sc, abort_flag);
+    scan::append_role(ct.s, r, lane, Team{lane, 32, 3 + r}, ct.ring, sc, abort_flag);
   } else {
     // ------------------------------------------------------------------ finisher warps
     const int f = warp - 2 - C::EPI_WARPS - C::SEL_WARPS;
     constexpr int RPF = NROWS / C::FIN_WARPS;
-    scan::finisher_role(ct.s, f * RPF, RPF, lane, rows, n_rows, n_blocks, sc, abort_flag);
+    scan::finisher_role(ct.s, f * RPF, RPF, lane, rows, n_rows, sc, abort_flag);
   }
   // ------------------------------------------------------------------ teardown
   ptx::tc_fence_before();

@@ -143,9 +143,6 @@ __device__ __forceinline__ void hist_boundary(const Team& tm, SegSelSmem& sm, co
 // the histogram meanwhile; counts only grow, so a torn snapshot can only give a lower bin, which
 // is still a valid bound.  *need_in and *pop describe the boundary bin (entries still wanted
 // from it, and its population as read).
-// BATCHED issues all level-1 loads before the reductions (faster, 16 more live registers);
-// the serial form is for callers inside a register-bound loop.
-template <bool BATCHED = true>
 __device__ __forceinline__ bool warp_hist_boundary(const uint32_t* hist, uint32_t need, int lane, uint32_t* bin,
                                                    uint32_t* need_in, uint32_t* pop) {
   const uint4* h4 = reinterpret_cast<const uint4*>(hist);
@@ -154,31 +151,19 @@ __device__ __forceinline__ bool warp_hist_boundary(const uint32_t* hist, uint32_
   // level 1: chunks of 128 bins, lane holds four consecutive bins of each chunk.  All loads
   // first, then all reductions, so their latencies overlap.
   constexpr int NCH = kSelBins / 128;
-  if constexpr (BATCHED) {
-    uint32_t part[NCH];
+  uint32_t part[NCH];
 #pragma unroll
-    for (int j = 0; j < NCH; ++j) {
-      const uint4 v = h4[j * 32 + lane];
-      part[j] = (v.x + v.y) + (v.z + v.w);
-    }
+  for (int j = 0; j < NCH; ++j) {
+    const uint4 v = h4[j * 32 + lane];
+    part[j] = (v.x + v.y) + (v.z + v.w);
+  }
 #pragma unroll
-    for (int j = 0; j < NCH; ++j) part[j] = __reduce_add_sync(0xffffffffu, part[j]);
+  for (int j = 0; j < NCH; ++j) part[j] = __reduce_add_sync(0xffffffffu, part[j]);
 #pragma unroll
-    for (int j = NCH - 1; j >= 0; --j) {
-      if (jsel < 0) {
-        if (cum + part[j] >= need) jsel = j;
-        else cum += part[j];
-      }
-    }
-  } else {
-#pragma unroll
-    for (int j = NCH - 1; j >= 0; --j) {
-      const uint4 v = h4[j * 32 + lane];
-      const uint32_t c = __reduce_add_sync(0xffffffffu, (v.x + v.y) + (v.z + v.w));
-      if (jsel < 0) {
-        if (cum + c >= need) jsel = j;
-        else cum += c;
-      }
+  for (int j = NCH - 1; j >= 0; --j) {
+    if (jsel < 0) {
+      if (cum + part[j] >= need) jsel = j;
+      else cum += part[j];
     }
   }
   if (jsel < 0) { *bin = 0; *need_in = 0; *pop = 0; return false; }
