@@ -216,11 +216,10 @@ int resolve_ws(const pivot_opts* o, size_t need, void** ws) {
 //   - rounds of part blocks, each with its own start: some sixteen tiles' time between two blocks, and K / 128 tiles
 //     before a threshold has formed;
 //   - where a part's survivors fill its candidate segment, the sweep that thins it out, 64 entries in a tile's time.
-//     A part admits every key of the refresh interval before the first threshold and about K / n of the n-th interval
-//     (K (ln n + 0.58) in all, 3 % more for the thresholds' bins).  K = 2048, 8192 rows at the end of 128K, four
-//     rounds of whole blocks: 3.58 ms, with segments twice as large 3.07; at the end of 256K in two parts, which
-//     still fill them, 6.69, in three, which do not, 5.59.  Segments of the least size (budgets up to 1024) are
-//     thinned within two intervals in any part and the sweep is short: not charged;
+//     A part of n keys admits K (1 + ln(n / K)) of them, a ninth more for the refresh intervals and the thresholds'
+//     bins, so this takes more than half a million keys.  (While a part refreshed its thresholds every 32 tiles only
+//     and kept room for as many, budgets of 1.2 K to 3 K paid the sweep at 64K or 128K keys already.)  Segments of
+//     the least size (budgets up to 1024) are thinned late and the sweep is short: not charged;
 //   - the merge of the parts' selections, 2 SMs' worth of rows at a time (14 us a round of 2 x 4096 entries; lists
 //     of more than 8192 entries have an SM to themselves, but charging them for that chooses worse: 3072 rows at
 //     the end of 128K would take 1.54 ms in two parts, 1.50 in three).
@@ -245,10 +244,10 @@ int choose_split(int n_proxy, int first_vis, int last_vis, int K, int cap, int s
       if (align_up((size_t)n_proxy * sizeof(MergeRow)) + 2 * align_up((size_t)n_proxy * s * K * 4) > room) break;
     }
     double per_block = tiles / s + 16.0 + K / 128.0;
-    const double intervals = tiles / s / kThresholdRefreshTiles;
-    if (cap > kMinSegment && intervals > 1.0) {
-      const double admitted = 1.03 * (kThresholdRefreshTiles * 128.0 + K * (log(intervals) + 0.58));
-      if (admitted > cap - kThresholdRefreshTiles * 128) per_block += admitted / 64.0;
+    const double part = tiles / s * 128.0;
+    if (cap > kMinSegment && part > K) {
+      const double admitted = 1.11 * K * (1.0 + log(part / K));
+      if (admitted > cap - kLeastRoomTiles * 128) per_block += admitted / 64.0;
     }
     double cost = (double)((s * nb + sms - 1) / sms) * per_block;
     if (s > 1) cost += (double)((n_proxy + 2 * sms - 1) / (2 * sms)) * (4.0 + 14.0 * s * K / 8192.0);

@@ -144,6 +144,17 @@ __device__ __forceinline__ uint32_t select_bin_lo(int bin, int base) {
   return bin >= kSelBins || bin + base > 0x1ffff ? 0xffffffffu : (uint32_t)(bin + base) << 15;
 }
 
+// The append warps' rare steps, out of their loop: a row's segment without what lies at or below a threshold (returns
+// what is left), and its K best alone (returns the key of the last; more than K entries).
+static __device__ __noinline__ int drop_below(entry_t* seg, int cnt, int lane, uint32_t thr) {
+  return seg_filter_inplace(seg, cnt, lane, [thr](entry_t x) { return entry_key(x) > thr; });
+}
+static __device__ __noinline__ uint32_t compact_to_best(const Team& tm, SegSelSmem& sel, entry_t* seg, int cnt, int K) {
+  entry_t cut;
+  (void)seg_compact<false>(tm, sel, Seg{seg, cnt}, K, &cut);
+  return entry_key(cut);
+}
+
 // The append warp of row r (one warp, all blocks of this CTA): counts the survivors of every tile
 // in the row histogram, moves them to the row's segment in the L2-resident scratch and keeps the
 // row's threshold fresh -- alone, without barriers.  At the end of a block it reads the boundary
@@ -163,8 +174,9 @@ __device__ __noinline__ void append_role(SelectCtrl<NROWS, QD>& s, int r, int la
     if (!warp_hist_boundary(rhist, (uint32_t)K, lane, &b, &need_in, &pop)) return 0u;
     return b > 0 ? (((uint32_t)((int)b + base)) << 15) - 1u : 0u;
   };
-  // The threshold is refreshed every CHK tiles; a tile adds at most TILE_KEYS entries, so a
-  // segment checked then always has room until the next check.
+  // The threshold is refreshed every CHK tiles, more often while it still moves fast (the K-th best of t tiles lets
+  // K / (128 t) of the next one through).  A tile adds at most TILE_KEYS entries, so a segment that has room for the
+  // tiles until the next refresh never overflows.
   const int CHK = CAP / (2 * TILE_KEYS) < kThresholdRefreshTiles ? (CAP / (2 * TILE_KEYS) > 0 ? CAP / (2 * TILE_KEYS) : 1) : kThresholdRefreshTiles;
   const int headroom = TILE_KEYS * CHK;
   uint32_t it = 0, seq = 0;
@@ -183,31 +195,41 @@ __device__ __noinline__ void append_role(SelectCtrl<NROWS, QD>& s, int r, int la
     entry_t* const seg = row_segment<NROWS>(sc, r, seq);
     bool sel_mine = seq == 0;                    // the finisher of the previous block may still use `sel`
     __syncwarp();
-    int due = CHK;                               // tiles until the next refresh
+    // tiles until the next refresh; the first when the segment holds a quarter more than K
+    int due = (K + K / 4 + TILE_KEYS - 1) / TILE_KEYS;
+    due = due < kRefreshMin ? kRefreshMin : due;
+    due = due < CAP / (2 * TILE_KEYS) ? due : CHK;
     for (int t = 0; t < ntiles; ++t, ++it) {
       if (due-- == 0) {
-        due = CHK - 1;
-        if (K > 0) {
+        int next = t / 2 < kRefreshMin ? kRefreshMin : t / 2;
+        next = next < CHK ? next : CHK;
+        const int left = ntiles - t;
+        if (left <= kRefreshLast && cnt + TILE_KEYS * left <= CAP) {
+          next = left;                             // too few tiles left to gain by it
+        } else if (K > 0) {
           const uint32_t th = hist_threshold(K, base);
           thr = th > thr ? th : thr;
-          if (cnt + headroom > CAP) {
+          if (cnt + TILE_KEYS * (next < kLeastRoomTiles ? next : kLeastRoomTiles) > CAP) {
             // Nearly full: drop what fell below the threshold; if that is not enough (ties, adversarial
             // order) compact exactly to the K best.  What goes lies below every bin the final boundary can
             // be in, so the histogram stays exact for what the selection looks at.
             const uint32_t tcur = thr;
-            cnt = seg_filter_inplace(seg, cnt, lane, [tcur](entry_t x) { return entry_key(x) > tcur; });
+            cnt = drop_below(seg, cnt, lane, tcur);
             if (cnt + headroom > CAP && cnt > K) {
               if (!sel_mine) {                     // (rare path: waiting here costs nothing that matters)
                 (void)ptx::mbar_wait(&s.fin_done[r][fb ^ 1], ((seq - 1) >> 1) & 1, abort_flag, 64);
                 sel_mine = true;
               }
-              entry_t cut;
-              cnt = seg_compact<false>(tm, sel, Seg{seg, cnt}, K, &cut);
-              thr = entry_key(cut) > thr ? entry_key(cut) : thr;
+              const uint32_t cut = compact_to_best(tm, sel, seg, cnt, K);
+              cnt = K;
+              thr = cut > thr ? cut : thr;
             }
           }
+          const int room = (CAP - cnt) / TILE_KEYS;
+          next = next < room ? next : room;
           if (lane == 0) s.thr[r] = ((unsigned long long)seq << 32) | thr;
         }
+        due = next - 1;
       }
       const int sb = it % QD;
       (void)ptx::mbar_wait(&s.sc_full[sb], (it / QD) & 1, abort_flag);

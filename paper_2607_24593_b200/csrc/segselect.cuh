@@ -19,6 +19,7 @@
 // (CACHED = true, loops unrolled) and re-read them from memory otherwise (rolled loops).
 #pragma once
 #include "common.cuh"
+#include "ptx.cuh"
 #include "select.cuh"
 
 namespace pivot {
@@ -143,55 +144,47 @@ __device__ __forceinline__ void hist_boundary(const Team& tm, SegSelSmem& sm, co
 // the histogram meanwhile; counts only grow, so a torn snapshot can only give a lower bin, which
 // is still a valid bound.  *need_in and *pop describe the boundary bin (entries still wanted
 // from it, and its population as read).
+// Some 110 instructions; the chunk sums by warp reductions that this replaced took 170 and, one warp beside fifteen others,
+// 3 K clocks (now 2 K), which blocks of a dozen tiles pay at their end.  (As a function of its own it made the append
+// warps' loop, whose registers then have to survive the call, 3 .. 9 % slower on long requests.)
 __device__ __forceinline__ bool warp_hist_boundary(const uint32_t* hist, uint32_t need, int lane, uint32_t* bin,
                                                    uint32_t* need_in, uint32_t* pop) {
-  const uint4* h4 = reinterpret_cast<const uint4*>(hist);
-  uint32_t cum = 0;
-  int jsel = -1;
-  // level 1: chunks of 128 bins, lane holds four consecutive bins of each chunk.  All loads
-  // first, then all reductions, so their latencies overlap.
-  constexpr int NCH = kSelBins / 128;
-  uint32_t part[NCH];
+  const uint32_t h = ptx::smem_u32(hist);
+  __syncwarp();                      // this warp's own counts
+  // level 1: each lane adds up 64 neighbouring bins, 16 bytes at a time in an order that spreads a quarter warp's lanes
+  // over all banks; suffix sums over the lanes say whose bins the boundary lies in.
+  constexpr int PER = kSelBins / 32;
+  uint32_t s = 0;
 #pragma unroll
-  for (int j = 0; j < NCH; ++j) {
-    const uint4 v = h4[j * 32 + lane];
-    part[j] = (v.x + v.y) + (v.z + v.w);
+  for (int i = 0; i < PER / 4; ++i) {
+    const uint4 v = ptx::ld_shared_v4(h + (uint32_t)lane * (PER * 4) + (uint32_t)((i ^ (lane & (PER / 4 - 1))) << 4));
+    s += (v.x + v.y) + (v.z + v.w);
   }
-#pragma unroll
-  for (int j = 0; j < NCH; ++j) part[j] = __reduce_add_sync(0xffffffffu, part[j]);
-#pragma unroll
-  for (int j = NCH - 1; j >= 0; --j) {
-    if (jsel < 0) {
-      if (cum + part[j] >= need) jsel = j;
-      else cum += part[j];
-    }
-  }
-  if (jsel < 0) { *bin = 0; *need_in = 0; *pop = 0; return false; }
-  // level 2: inside the chunk, suffix sums over the lanes
-  const uint4 v = h4[jsel * 32 + lane];
-  const uint32_t s = (v.x + v.y) + (v.z + v.w);
   uint32_t incl = s;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const uint32_t t = __shfl_down_sync(0xffffffffu, incl, o);
     if (lane + o < 32) incl += t;
   }
-  const uint32_t above = cum + incl - s;              // entries in bins above this lane's four
-  const bool here = above < need && need <= above + s;
-  uint32_t b = 0, ni = 0, pp = 0;
-  if (here) {
-    uint32_t c = above;
-    if (c + v.w >= need) { b = 3; ni = need - c; pp = v.w; }
-    else if ((c += v.w) + v.z >= need) { b = 2; ni = need - c; pp = v.z; }
-    else if ((c += v.z) + v.y >= need) { b = 1; ni = need - c; pp = v.y; }
-    else { c += v.y; b = 0; ni = need - c; pp = v.x; }
-    b += (uint32_t)(jsel * 128 + lane * 4);
+  const uint32_t m1 = __ballot_sync(0xffffffffu, incl >= need);      // suffix sums fall with the lane: a run from lane 0 up
+  if (m1 == 0) { *bin = 0; *need_in = 0; *pop = 0; return false; }
+  const int l1 = 31 - __clz(m1);
+  const uint32_t cum = __shfl_sync(0xffffffffu, incl - s, l1);       // entries in the bins above that lane's
+  // level 2: two bins per lane of those 64 (read again: other warps may have added to them, never taken away)
+  const uint2 v = ptx::ld_shared_v2(h + (uint32_t)(l1 * PER + lane * 2) * 4);
+  const uint32_t s2 = v.x + v.y;
+  uint32_t incl2 = s2;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_down_sync(0xffffffffu, incl2, o);
+    if (lane + o < 32) incl2 += t;
   }
-  const uint32_t m = __ballot_sync(0xffffffffu, here);
-  const int src = __ffs(m) - 1;                        // exactly one lane
-  *bin = __shfl_sync(0xffffffffu, b, src);
-  *need_in = __shfl_sync(0xffffffffu, ni, src);
-  *pop = __shfl_sync(0xffffffffu, pp, src);
+  const uint32_t above = cum + incl2 - s2;                           // entries in bins above this lane's two
+  const int l2 = 31 - __clz(__ballot_sync(0xffffffffu, cum + incl2 >= need));
+  const bool hi = above + v.y >= need;
+  *bin = __shfl_sync(0xffffffffu, (uint32_t)(l1 * PER + lane * 2) + (hi ? 1u : 0u), l2);
+  *need_in = __shfl_sync(0xffffffffu, need - (hi ? above : above + v.y), l2);
+  *pop = __shfl_sync(0xffffffffu, hi ? v.y : v.x, l2);
   return true;
 }
 

@@ -340,3 +340,29 @@ def test_decode_crowded_boundary_bin(pv, B, n_tied):
     assert (_sorted(cand) == want).all()
     want = np.sort(np.concatenate([above.numpy(), tied.numpy()[: k - len(above)]]))
     assert (_sorted(out) == want).all()
+
+
+@pytest.mark.parametrize("impl", [0, 2])
+@pytest.mark.parametrize("L,K,slope", [
+    (513, 1, 2.0 ** -10), (1409, 1024, 2.0 ** -10), (1537, 100, 2.0 ** -10), (2100, 777, -2.0 ** -16),
+    (12000, 512, 2.0 ** -12), (12000, 1024, 2.0 ** -8), (16500, 1300, 2.0 ** -13), (9999, 64, -2.0 ** -18),
+])
+def test_scores_that_rise_or_fall_along_the_prefix(pv, L, K, slope, impl):
+    """One key under scales that rise (every key beats all before it: no threshold drops anything, segments of 8192
+    entries fill up and are thinned, by the threshold or, where the scores outgrow the histogram, to the K best) or fall
+    with its position (nothing is appended after the first K).  Row t selects its last or its first K keys; on
+    either side of the first thresholds (5/4 K keys, four tiles) and of a block's last refresh."""
+    x = inputs.make_prefill(L, dtype="fp8", seed=3)
+    raw = x.k.clone().view(torch.uint8)
+    raw[:] = raw[5].clone()
+    scale = 1.0 + slope * torch.arange(L, dtype=torch.float32)
+    q, w, _, kw = _operands(x)
+    kw["k_scale"] = scale.cuda()
+    out = torch.full((L, K), -7, dtype=torch.int32, device="cuda")
+    pv.dense_index(q, w, raw.view(x.k.dtype).cuda(), L, 64, 128, K, out, impl=impl, **kw)
+    torch.cuda.synchronize()
+    assert pv.pivot_device_status() == 0
+    t = torch.arange(L, device="cuda", dtype=torch.int32).view(-1, 1)
+    j = torch.arange(K, device="cuda", dtype=torch.int32).view(1, -1)
+    want = torch.where(t - K + 1 + j >= 0, t - K + 1 + j, -1) if slope > 0 else torch.where(j <= t, j, -1).sort(dim=1).values
+    assert torch.equal(out.sort(dim=1).values, want)
