@@ -112,16 +112,8 @@ static_assert(rsmem_bytes<DT_FP8, 0>() <= 232448 && rsmem_bytes<DT_FP8, 2>() <= 
               rsmem_bytes<DT_FP8, 3>() <= 232448 && rsmem_bytes<DT_BF16, 3>() <= 232448 &&
               rsmem_bytes<DT_BF16>() <= 232448, "shared memory budget");
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int NPEND>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(NPEND) : "memory");
 }
 
 __device__ __forceinline__ int group_tiles(const GroupDesc& gd) {
@@ -387,16 +379,16 @@ refine_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const GroupDesc* grou
           const int kr = __shfl_sync(0xffffffffu, krow[i >> 3], (i & 7) * 4 + sub);
           const uint8_t* src = kb + (long long)kr * krow_bytes;
 #pragma unroll
-          for (int h = 0; h < C::KHALVES; ++h) cp_async16(dsw[i & 1] + i * 512 + h * C::HALF_TILE_BYTES, src + h * 128);
+          for (int h = 0; h < C::KHALVES; ++h) ptx::cp_async16(dsw[i & 1] + i * 512 + h * C::HALF_TILE_BYTES, src + h * 128);
         }
-        cp_async_commit();
+        ptx::cp_async_commit();
         if (it + 1 - pub > (uint32_t)C::LOOKAHEAD) {
-          cp_async_wait<C::LOOKAHEAD>();
+          ptx::cp_async_wait<C::LOOKAHEAD>();
           publish(pub++);
         }
       }
     }
-    cp_async_wait<0>();
+    ptx::cp_async_wait<0>();
     while (pub < it) publish(pub++);
   } else if (C::OVL && warp >= 2 + GATHER_WARPS + EPI_WARPS) {
     // ------------------------------------------------------------------ select warps (EPI = 3)

@@ -320,14 +320,16 @@ __device__ __noinline__ void finisher_role(SelectCtrl<NROWS, QD>& s, int r0, int
       const int b = s.fin[r][fb].b;
       if (b < 0) return;
       const int ri = b * NROWS + r;
-      const int K = (ri < n_rows) ? rows[ri].K : 0;
+      const typename SelectCtrl<NROWS, QD>::FinRow f = s.fin[r][fb];
+      const StagedSeg staged(s.sel[r], row_segment<NROWS>(sc, r, seq), f.cnt);
+      staged.start(lane);
+      const RowDesc rd = rows[ri < n_rows ? ri : n_rows - 1];
+      const int K = ri < n_rows ? rd.K : 0;
       if (K > 0) {
-        const RowDesc rd = rows[ri];
-        const typename SelectCtrl<NROWS, QD>::FinRow f = s.fin[r][fb];
         const int rbase = f.base;
         auto bin_lo = [rbase](int bin) { return select_bin_lo(bin, rbase); };
-        const int n_valid = warp_seg_topk_binned(s.sel[r], row_segment<NROWS>(sc, r, seq), f.cnt, bin_lo, f.bsel,
-                                                 f.need_b, f.pop, rd.out, rd.out_score, K, lane);
+        const int n_valid = warp_seg_topk_binned(s.sel[r], staged, bin_lo, f.bsel, f.need_b, f.pop, rd.out, rd.out_score, K,
+                                                 lane);
         for (int i = n_valid + lane; i < K; i += 32) {
           rd.out[i] = -1;
           if (rd.out_score) rd.out_score[i] = -INFINITY;

@@ -27,8 +27,8 @@ namespace pivot {
 
 constexpr int kSelBins = 2048;
 constexpr int kSelSmall = 256;
-// Entries per lane in flight in the emitting sweep.  Measured, 30001-token fp8 scan: 4 1.95 ms, 8 1.47, 10 1.40, 12 1.37,
-// 14 1.44, 16 1.39 -- fewer leave the loads exposed, more cost the other warps instruction fetches.
+// Entries per lane in flight in the emitting sweep (measured when the scan's finishers used it too, 30001 tokens fp8: 4 1.95 ms, 8
+// 1.47, 10 1.40, 12 1.37, 14 1.44, 16 1.39 -- fewer leave the loads exposed, more cost the other warps instruction fetches).
 constexpr int kEmitBatch = 12;
 constexpr int kSelEpt = 64;      // register-cached entries per lane
 
@@ -501,6 +501,95 @@ __device__ __forceinline__ int warp_emit_keys(SegSelSmem& sm, const Src& src, ui
   return (int)(base < (uint32_t)K ? base : (uint32_t)K);
 }
 
+// A scan row's segment on its way through shared memory, for the one sweep its finisher makes: four chunks of 256 entries in
+// flight (the first before the finisher has read its row's descriptor), each lane reading pairs.  A finisher (one warp for two
+// rows) is what short blocks wait for, and loads straight into registers left an L2 round trip per twelve entries of a
+// lane exposed: 230 -> 186 clocks per 32 entries, 5003 tokens 168 -> 163 us, dense 16K 1511 -> 1488, dense 5001 tokens
+// 184 -> 181, 8K tokens 415 -> 401.
+struct StagedSeg {
+  static constexpr int kChunk = 256;                               // entries: eight per lane
+  static constexpr int kSlots = kSelBins * 4 / (kChunk * 8);       // the histogram's 8 KB, which only ties need
+  const entry_t* seg;
+  int cnt;
+  uint32_t buf;
+  __device__ __forceinline__ StagedSeg(SegSelSmem& sm, const entry_t* e, int n) : seg(e), cnt(n), buf(ptx::smem_u32(sm.hist)) {}
+  // Whole chunks are read: a segment's size is a multiple of kChunk, and what lies behind its entries is masked later.
+  __device__ __forceinline__ void fetch(int c, int lane) const {
+    if (c * kChunk < cnt) {
+#pragma unroll
+      for (int u = 0; u < kChunk / 64; ++u)
+        ptx::cp_async16(buf + (uint32_t)(((c % kSlots) * kChunk + u * 64 + lane * 2) * 8), seg + c * kChunk + u * 64 + lane * 2);
+    }
+    ptx::cp_async_commit();
+  }
+  __device__ __forceinline__ void start(int lane) const {
+#pragma unroll
+    for (int c = 0; c < kSlots; ++c) fetch(c, lane);
+  }
+  __device__ __forceinline__ void drain() const {
+    ptx::cp_async_wait<0>();
+    __syncwarp();
+  }
+};
+
+// The sweep of warp_emit_keys over a started StagedSeg.
+__device__ __forceinline__ int warp_emit_staged(SegSelSmem& sm, const StagedSeg& src, uint32_t khi, uint32_t n_keys,
+                                                uint32_t* n_list, int32_t* __restrict__ out, int K, int lane) {
+  constexpr int CH = StagedSeg::kChunk;
+  const uint32_t lt = (1u << lane) - 1u;
+  const uint32_t klo = khi - n_keys + 1u;
+  uint32_t base = 0, ln = 0;
+  for (int c = 0; c * CH < src.cnt; ++c) {
+    ptx::cp_async_wait<StagedSeg::kSlots - 1>();
+    __syncwarp();
+    const uint32_t buf = src.buf + (uint32_t)((c % StagedSeg::kSlots) * CH * 8);
+    if (src.cnt - c * CH < CH) {                         // the last chunk: what lies behind the entries is empty
+      for (int i = src.cnt - c * CH + lane; i < CH; i += 32) ptx::st_shared_if(buf + (uint32_t)i * 8, (uint64_t)0, true);
+      __syncwarp();
+    }
+    uint32_t k[CH / 32], np[CH / 32];                    // keys and ~positions: a lane has neighbouring pairs
+#pragma unroll
+    for (int u = 0; u < CH / 64; ++u) {
+      const uint4 v = ptx::ld_shared_v4(buf + (uint32_t)((u * 64 + lane * 2) * 8));
+      np[2 * u] = v.x; k[2 * u] = v.y; np[2 * u + 1] = v.z; k[2 * u + 1] = v.w;
+    }
+    __syncwarp();
+    src.fetch(c + StagedSeg::kSlots, lane);
+    uint32_t edge = 0;                                   // a handful per row
+#pragma unroll
+    for (int u = 0; u < CH / 64; ++u) {
+      const bool e0 = k[2 * u] > khi, e1 = k[2 * u + 1] > khi;
+      const uint32_t m0 = __ballot_sync(0xffffffffu, e0), m1 = __ballot_sync(0xffffffffu, e1);
+      const uint32_t p0 = base + __popc(m0 & lt) + __popc(m1 & lt);
+      const uint32_t p1 = p0 + (e0 ? 1u : 0u);
+      if (e0 && p0 < (uint32_t)K) out[p0] = (int32_t)~np[2 * u];
+      if (e1 && p1 < (uint32_t)K) out[p1] = (int32_t)~np[2 * u + 1];
+      base += __popc(m0) + __popc(m1);
+      edge |= k[2 * u] - klo < n_keys ? 1u << (2 * u) : 0u;
+      edge |= k[2 * u + 1] - klo < n_keys ? 2u << (2 * u) : 0u;
+    }
+    if (__any_sync(0xffffffffu, edge != 0)) {
+      const uint32_t ec = (uint32_t)__popc(edge);
+      uint32_t ei = ec;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, ei, o);
+        if (lane >= o) ei += v;
+      }
+      uint32_t q = ln + ei - ec;
+#pragma unroll
+      for (int j = 0; j < CH / 32; ++j) {
+        const bool e = (edge >> j) & 1u;
+        if (e && q < (uint32_t)kSelSmall) sm.list[q] = ((entry_t)k[j] << 32) | np[j];
+        q += e ? 1u : 0u;
+      }
+      ln += __shfl_sync(0xffffffffu, ei, 31);
+    }
+  }
+  *n_list = ln < (uint32_t)kSelSmall ? ln : (uint32_t)kSelSmall;
+  return (int)(base < (uint32_t)K ? base : (uint32_t)K);
+}
+
 // The need_b best of the ln listed entries follow the `base` entries already written (entries are distinct: a
 // rank is a slot).  Returns the row's length.
 __device__ __forceinline__ int warp_emit_list(const SegSelSmem& sm, uint32_t ln, uint32_t need_b, uint32_t base, int32_t* out,
@@ -616,11 +705,11 @@ __device__ __forceinline__ int warp_row_topk(SegSelSmem& sm, const uint32_t* key
 // bin_lo(b) .. bin_lo(b + 1) - 1: bsel = the boundary bin (need_b of its pop entries are wanted), -1 = everything is wanted.
 // One sweep, unless the boundary bin is too crowded to rank (ties): then the general way.
 template <typename BinFn>
-__device__ __noinline__ int warp_seg_topk_binned(SegSelSmem& sm, const entry_t* seg, int cnt, BinFn bin_lo, int bsel,
-                                                 uint32_t need_b, uint32_t pop, int32_t* out, float* out_score, int K,
-                                                 int lane) {
-  const SegSrc src{seg, cnt};
+__device__ __noinline__ int warp_seg_topk_binned(SegSelSmem& sm, const StagedSeg staged, BinFn bin_lo, int bsel, uint32_t need_b,
+                                                 uint32_t pop, int32_t* out, float* out_score, int K, int lane) {
+  const SegSrc src{staged.seg, staged.cnt};
   if (bsel >= 0 && pop != need_b && pop > (uint32_t)kSelSmall) {
+    staged.drain();
     entry_t mn = ~0ull, mx = 0ull;
     uint32_t nv = 0;
     src.template sweep<16, true>(lane, [&](entry_t e) {
@@ -644,9 +733,10 @@ __device__ __noinline__ int warp_seg_topk_binned(SegSelSmem& sm, const entry_t* 
   const uint32_t n_keys = bsel < 0 || whole ? 0u : above - bin_lo(bsel);      // keys of the boundary bin
   if (!out_score) {
     uint32_t ln = 0;
-    const int base = warp_emit_keys<kEmitBatch>(sm, src, khi, n_keys, &ln, out, K, lane);
+    const int base = warp_emit_staged(sm, staged, khi, n_keys, &ln, out, K, lane);
     return warp_emit_list(sm, ln, need_b, (uint32_t)base, out, out_score, K, lane);
   }
+  staged.drain();
   const entry_t ebhi = ((entry_t)khi << 32) | 0xffffffffull;
   return warp_emit_above(sm, src, n_keys == 0u ? ~0ull : (entry_t)(above - n_keys) << 32, ebhi, need_b, out, out_score, K, lane);
 }
