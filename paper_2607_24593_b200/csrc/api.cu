@@ -284,6 +284,7 @@ int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kcach
   p.status = first ? ws.status : nullptr;
   int pg0 = 0, live = 0;
   for (int i = 0; i < n; ++i) live += cu[i + 1] > cu[i];
+  long long scan_rows = 0, scan_keys = 0;               // what the scan's rows see in all
   for (int i = 0; i < n; ++i) {
     const int L = cu[i + 1] - cu[i];
     if (L == 0) continue;
@@ -304,6 +305,8 @@ int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kcach
     pg0 = g_begin > first_group ? g_begin : first_group;   // first proxy group of this call
     const int n_proxy = g_end > pg0 ? g_end - pg0 : 0;
     const int rows = dense1 - dense0 + n_proxy;
+    scan_rows += rows;
+    scan_keys += (long long)(dense1 - dense0) * (dense0 + dense1) / 2 + (long long)n_proxy * (pg0 + g_end) / 2 * g;
     p.req[p.n_req++] = PrefillReq{cu[i], L, dense0, dense1 - dense0, pg0, n_proxy, p.n_slots, p.n_proxy};
     p.n_slots += live > 1 ? (rows + 3) / 4 * 4 : rows;
     p.n_proxy += n_proxy;
@@ -340,7 +343,8 @@ int run_prefill(const pivot_tensor* q, const float* w, const pivot_tensor* kcach
   } else {
     ScanOperands op{kcache->data, tokens, kcache->scale, q->data, tokens, ws.proxy_q, p.n_proxy, q->dtype};
     op.k_stride = p.k_stride;
-    if ((rc = check_cuda(launch_scan_tc(op, ws.rows, p.n_slots * p.split, 4, tc_scratch(ws), sm_count(), st, o && o->impl == 2, true))))
+    if ((rc = check_cuda(launch_scan_tc(op, ws.rows, p.n_slots * p.split, 4, tc_scratch(ws), sm_count(), st, o && o->impl == 2, true,
+                                        scan_keys / (scan_rows > 0 ? scan_rows : 1) / p.split))))
       return rc;
     if (p.split > 1 &&
         (rc = check_cuda(launch_merge_parts(p.merges, p.n_proxy, p.split * (mode == PIVOT_REFINE ? c : k), st))))

@@ -173,10 +173,12 @@ struct ScanOperands {
 };
 // rows_per_block consecutive scan rows share one key stream (4 in prefill, 1 in decode).
 // fp32_head_sum: keep the gate-weighted head sum in fp32 FMAs even where the tensor-core form
-// (FP8, four rows per block) is available.
+// (FP8, four rows per block) is available.  mean_keys: keys that a scan row sees on average; up to
+// kShortBlockKeys (48 tiles: four finisher warps win up to 61 tiles a block and lose from 72 on) every row has a finisher of its own.
+constexpr long long kShortBlockKeys = 6144;
 cudaError_t launch_scan_tc(const ScanOperands& op, const RowDesc* rows, int n_rows, int rows_per_block,
                            const ScanScratch& s, int sms, cudaStream_t st, bool fp32_head_sum = false,
-                           bool overlap_prev = false);
+                           bool overlap_prev = false, long long mean_keys = 1ll << 40);
 
 cudaError_t launch_refine_tc(const void* q, int q_rows, int dtype, const GroupDesc* groups, int n_groups,
                              const ScanScratch& s, int sms, cudaStream_t st, bool fp32_head_sum = false,

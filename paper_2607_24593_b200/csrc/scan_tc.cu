@@ -48,8 +48,8 @@ using scan::BlockIter;
 constexpr int MAX_STAGES = 8;
 constexpr int QDEPTH = 4;         // survivor-queue buffers between the score warps and the append warps
 
-// EPI: 1 = the gate-weighted head sum runs on the tensor core where the configuration allows it
-// (FP8, four rows); 0 = fp32 FMA epilogue everywhere.
+// EPI: 1, 2 = the gate-weighted head sum runs on the tensor core where the configuration allows it
+// (FP8, four rows), with two or four finisher warps; 0 = fp32 FMA epilogue everywhere.
 template <int DT, int NROWS, int EPI = 1>
 struct Cfg {
   static constexpr bool FP8 = DT == DT_FP8;
@@ -69,12 +69,16 @@ struct Cfg {
   static constexpr int ROWS_PER_TEAM = NROWS == 4 ? 2 : 1;
   static constexpr int TEAMS = EPI_WARPS / 4;
   static constexpr int SEL_WARPS = NROWS;                     // append warps, one per row
-  static constexpr int FIN_WARPS = NROWS == 4 ? 2 : 1;        // finisher warps, one per two rows
+  // Finisher warps: one per two rows, or one per row (EPI 2) where short blocks wait for them.  The two more leave every
+  // thread 96 instead of 128 registers (a few spills around the roles' loops), which long blocks pay for.  us, two -> four: packed
+  // batch (12 tiles a block) 465 -> 420, 5003 tokens (17) 163.6 -> 153, dense 5001 (22) 175 -> 165, 8K (32) 400 -> 372, 16K
+  // K = 512 (61) 457 -> 453; dense 16K (72) 1522 -> 1531, dense 32K (130) 5271 -> 5540, 64K (243) 5738 -> 5990.
+  static constexpr int FIN_WARPS = FP8 && NROWS == 4 && EPI == 2 ? 4 : NROWS == 4 ? 2 : 1;
   static constexpr int THREADS = 64 + (EPI_WARPS + SEL_WARPS + FIN_WARPS) * 32;
   static constexpr int TMEM_COLS = 2 * N < 32 ? 32 : 2 * N;
   // FP8, four rows: the gate-weighted head sum itself runs on the tensor core (see the kernel
   // header).  Other configurations keep the fp32 FMA epilogue.
-  static constexpr bool MMA2 = FP8 && NROWS == 4 && EPI == 1;
+  static constexpr bool MMA2 = FP8 && NROWS == 4 && EPI >= 1;
   static constexpr int QD = MMA2 ? 2 : QDEPTH;                 // survivor-queue depth
   static constexpr int TMEM_EMPTY_ARRIVALS = MMA2 ? 4 : EPI_WARPS;
   static constexpr int SC_FULL_ARRIVALS = MMA2 ? 4 : EPI_WARPS;
@@ -109,7 +113,7 @@ constexpr size_t smem_bytes() {
   return 1024 + C::QBUFS * C::QBUF_BYTES + C::STAGES * C::STAGE_BYTES + sizeof(Ctrl<NROWS, C::MMA2>);
 }
 static_assert(smem_bytes<DT_FP8, 4, 1>() <= 232448 && smem_bytes<DT_FP8, 4, 0>() <= 232448 &&
-              smem_bytes<DT_BF16, 4>() <= 232448, "shared memory budget");
+              smem_bytes<DT_FP8, 4, 2>() <= 232448 && smem_bytes<DT_BF16, 4>() <= 232448, "shared memory budget");
 
 // The two kinds of score warps where the head sum runs on the tensor core, functions of their own so that
 // neither's registers are allocated around the other's (inlined, with the block ring: spills in both loops, 64K Reuse
@@ -617,7 +621,7 @@ bool make_scale_map(CUtensorMap* m, const float* base, long long n, int box) {
 
 
 cudaError_t launch_scan_tc(const ScanOperands& op, const RowDesc* rows, int n_rows, int rows_per_block,
-                           const ScanScratch& s, int sms, cudaStream_t st, bool fp32_head_sum, bool overlap_prev) {
+                           const ScanScratch& s, int sms, cudaStream_t st, bool fp32_head_sum, bool overlap_prev, long long mean_keys) {
   if (n_rows <= 0) return cudaSuccess;
   CUtensorMap mk, mq0, mq1, mks;
   memset(&mks, 0, sizeof(mks));
@@ -629,6 +633,7 @@ cudaError_t launch_scan_tc(const ScanOperands& op, const RowDesc* rows, int n_ro
   if (op.dtype == DT_FP8) {
     if (rows_per_block != 4) return launch_one<DT_FP8, 1>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev);
     return fp32_head_sum ? launch_one<DT_FP8, 4, 0>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev)
+           : mean_keys <= kShortBlockKeys ? launch_one<DT_FP8, 4, 2>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev)
                          : launch_one<DT_FP8, 4, 1>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev);
   }
   return rows_per_block == 4 ? launch_one<DT_BF16, 4>(mk, mq0, mq1, mks, rows, n_rows, s, sms, st, overlap_prev)

@@ -85,6 +85,6 @@ extern "C" int dense_index_static(const pivot_tensor* q, const float* w, const p
     const size_t row = (size_t)kDim * (kcache->dtype == PIVOT_FP8_E4M3 ? 1 : 2);
     op.k_stride = kcache->stride_row == 0 || kcache->stride_row == row ? 0 : (int)kcache->stride_row;
   }
-  if (int rc = record_cuda(launch_scan_tc(op, rows, L, 4, sc, kStaticCtas, st))) return rc;
+  if (int rc = record_cuda(launch_scan_tc(op, rows, L, 4, sc, kStaticCtas, st, false, false, L / 2))) return rc;
   return record_cuda(cudaGetLastError());
 }

@@ -366,3 +366,24 @@ def test_scores_that_rise_or_fall_along_the_prefix(pv, L, K, slope, impl):
     j = torch.arange(K, device="cuda", dtype=torch.int32).view(1, -1)
     want = torch.where(t - K + 1 + j >= 0, t - K + 1 + j, -1) if slope > 0 else torch.where(j <= t, j, -1).sort(dim=1).values
     assert torch.equal(out.sort(dim=1).values, want)
+
+
+@pytest.mark.parametrize("mode", ["dense", 0, 1])
+def test_rows_select_the_same_whatever_the_finishers(pv, mode):
+    """Requests on either side of the mean prefix (6144 keys) up to which each row has a finisher warp of its own: the
+    rows that both have select the same keys."""
+    L, g, c, k = 15000, 4, 1024, 500
+    x = inputs.make_prefill(L, dtype="fp8", seed=27)
+    q, w, kk, kw = _operands(x)
+    outs = []
+    for n in (11001, L):
+        out = torch.full((n, k), -7, dtype=torch.int32, device="cuda")
+        part = dict(q_scale=kw["q_scale"][:n], k_scale=kw["k_scale"][:n])
+        if mode == "dense":
+            pv.dense_index(q[:n], w[:n], kk[:n], n, 64, 128, k, out, **part)
+        else:
+            pv.pivot_index_prefill(q[:n], w[:n], kk[:n], n, 64, 128, g, c, k, mode, out, **part)
+        torch.cuda.synchronize()
+        assert pv.pivot_device_status() == 0
+        outs.append(_sorted(out[:11000]))
+    assert np.array_equal(*outs)
