@@ -387,3 +387,27 @@ def test_rows_select_the_same_whatever_the_finishers(pv, mode):
         assert pv.pivot_device_status() == 0
         outs.append(_sorted(out[:11000]))
     assert np.array_equal(*outs)
+
+
+@pytest.mark.parametrize("dtype,impl", [("bf16", 0), ("fp8", 2)])
+@pytest.mark.parametrize("g,L", [(4, 4001), (6, 4003), (2, 3001), (9, 4000)])
+def test_members_missing_from_a_group_lend_nothing(pv, dtype, impl, g, L):
+    """fp32 head sums take no queries for members that a group (or its last chunk) does not have: what the groups before
+    it left in their place -- here NaN -- reaches no other member's selection."""
+    c, k = 512, 256
+    x = inputs.make_prefill(L, dtype=dtype, seed=31)
+    q, w, kk, kw = _operands(x)
+    first = torch.arange(L, device="cuda") % g == 0
+    bad = q.clone()
+    if dtype == "bf16":
+        bad[~first] = float("nan")
+    else:
+        bad.view(torch.uint8)[~first] = 0x7f
+    outs = []
+    for queries in (q, bad):
+        out = torch.full((L, k), -7, dtype=torch.int32, device="cuda")
+        pv.pivot_index_prefill(queries, w, kk, L, 64, 128, g, c, k, pv.REFINE, out, impl=impl, pool=pv.POOL_FIRST, **kw)
+        torch.cuda.synchronize()
+        assert pv.pivot_device_status() == 0
+        outs.append(_sorted(out[first]))
+    assert np.array_equal(*outs)
