@@ -535,8 +535,10 @@ struct StagedSeg {
 // The sweep of warp_emit_keys over a started StagedSeg.  The boundary's entries take their places in the list from a counter: in
 // short rows every chunk has one, and the prefix sum over the lanes that this replaced cost as much as half the chunk (12
 // packed requests 464 -> 453 us, dense 16K 1523 -> 1490, dense 5001 tokens 181 -> 175).
+template <bool SCORES>
 __device__ __forceinline__ int warp_emit_staged(SegSelSmem& sm, const StagedSeg& src, uint32_t khi, uint32_t n_keys,
-                                                uint32_t* n_list, int32_t* __restrict__ out, int K, int lane) {
+                                                uint32_t* n_list, int32_t* __restrict__ out, float* __restrict__ out_score, int K,
+                                                int lane) {
   constexpr int CH = StagedSeg::kChunk;
   const uint32_t lt = (1u << lane) - 1u;
   const uint32_t klo = khi - n_keys + 1u;
@@ -565,8 +567,14 @@ __device__ __forceinline__ int warp_emit_staged(SegSelSmem& sm, const StagedSeg&
       const uint32_t m0 = __ballot_sync(0xffffffffu, e0), m1 = __ballot_sync(0xffffffffu, e1);
       const uint32_t p0 = base + __popc(m0 & lt) + __popc(m1 & lt);
       const uint32_t p1 = p0 + (e0 ? 1u : 0u);
-      if (e0 && p0 < (uint32_t)K) out[p0] = (int32_t)~np[2 * u];
-      if (e1 && p1 < (uint32_t)K) out[p1] = (int32_t)~np[2 * u + 1];
+      if (e0 && p0 < (uint32_t)K) {
+        out[p0] = (int32_t)~np[2 * u];
+        if constexpr (SCORES) out_score[p0] = key_to_score(k[2 * u]);
+      }
+      if (e1 && p1 < (uint32_t)K) {
+        out[p1] = (int32_t)~np[2 * u + 1];
+        if constexpr (SCORES) out_score[p1] = key_to_score(k[2 * u + 1]);
+      }
       base += __popc(m0) + __popc(m1);
       edge |= k[2 * u] - klo < n_keys ? 1u << (2 * u) : 0u;
       edge |= k[2 * u + 1] - klo < n_keys ? 2u << (2 * u) : 0u;
@@ -728,14 +736,17 @@ __device__ __noinline__ int warp_seg_topk_binned(SegSelSmem& sm, const StagedSeg
   const uint32_t above = bsel < 0 ? 1u : bin_lo(whole ? bsel : bsel + 1);      // smallest key above the boundary (0 = empty slot)
   const uint32_t khi = above - 1u;
   const uint32_t n_keys = bsel < 0 || whole ? 0u : above - bin_lo(bsel);      // keys of the boundary bin
+  // Rows that return scores too (a part of a split prefix among them) have a sweep of their own.  us, against two sweeps of 64-bit
+  // compares from L2 after the copies: dense 16K 2359 -> 1564, 5003 tokens 213 -> 177, 8192 rows at the end of 256K in two parts
+  // 6101 -> 5788, 1024 rows at the end of 64K 296 -> 284.  (Both in a function of their own: plain rows 5 .. 8 % slower; one sweep
+  // with a test per entry: 3 .. 9 %.)
+  uint32_t ln = 0;
   if (!out_score) {
-    uint32_t ln = 0;
-    const int base = warp_emit_staged(sm, staged, khi, n_keys, &ln, out, K, lane);
-    return warp_emit_list(sm, ln, need_b, (uint32_t)base, out, out_score, K, lane);
+    const int base = warp_emit_staged<false>(sm, staged, khi, n_keys, &ln, out, nullptr, K, lane);
+    return warp_emit_list(sm, ln, need_b, (uint32_t)base, out, nullptr, K, lane);
   }
-  staged.drain();
-  const entry_t ebhi = ((entry_t)khi << 32) | 0xffffffffull;
-  return warp_emit_above(sm, src, n_keys == 0u ? ~0ull : (entry_t)(above - n_keys) << 32, ebhi, need_b, out, out_score, K, lane);
+  const int base = warp_emit_staged<true>(sm, staged, khi, n_keys, &ln, out, out_score, K, lane);
+  return warp_emit_list(sm, ln, need_b, (uint32_t)base, out, out_score, K, lane);
 }
 
 }  // namespace pivot

@@ -411,3 +411,40 @@ def test_members_missing_from_a_group_lend_nothing(pv, dtype, impl, g, L):
         assert pv.pivot_device_status() == 0
         outs.append(_sorted(out[first]))
     assert np.array_equal(*outs)
+
+
+@pytest.mark.parametrize("dtype,impl", [("fp8", 0), ("fp8", 2), ("bf16", 0)])
+@pytest.mark.parametrize("K,form", [(1, ""), (255, ""), (257, ""), (700, "rising"), (300, "tied"), (1300, "")])
+def test_rows_that_return_scores_select_the_same(pv, dtype, impl, K, form):
+    """Rows with their scores against the same rows without, and every score against the one that the row's key has when all
+    keys are wanted.  Rows hold 1 .. 2300 entries: on either side of the sweep's chunks of 256; rising scores append
+    every key, tied ones leave a boundary too crowded to rank."""
+    L = 2300
+    x = inputs.make_prefill(L, dtype=dtype, seed=41)
+    q, w, kk, kw = _operands(x)
+    if form == "rising":
+        b = kk.view(torch.uint8) if dtype == "fp8" else kk
+        b[:] = b[5].clone()
+        if dtype == "fp8":
+            kw["k_scale"] = (1.0 + 2.0 ** -10 * torch.arange(L, dtype=torch.float32)).cuda()
+        else:                                   # (bf16 keys have no scale: 16 magnitudes, rising)
+            kk = (kk.float() * 2.0 ** (torch.arange(L, device="cuda") * 16 // L - 8).view(-1, 1)).to(kk.dtype)
+    if form == "tied":
+        w = torch.zeros_like(w)
+
+    def index(k, scored):
+        out = torch.full((L, k), -7, dtype=torch.int32, device="cuda")
+        sc = torch.full((L, k), float("nan"), device="cuda") if scored else None
+        pv.dense_index(q, w, kk, L, 64, 128, k, out, dbg_scores=sc, impl=impl, **kw)
+        torch.cuda.synchronize()
+        assert pv.pivot_device_status() == 0
+        return out, sc
+
+    every, score = index(L, True)
+    table = torch.full((L, L + 1), float("-inf"), device="cuda")         # column 0: the -1 of short rows
+    table.scatter_(1, every.long() + 1, score)
+    table[:, 0] = float("-inf")
+    plain, _ = index(K, False)
+    out, sc = index(K, True)
+    assert np.array_equal(_sorted(plain), _sorted(out))
+    assert torch.equal(sc, table.gather(1, out.long() + 1))
