@@ -1,5 +1,8 @@
 """GPU checks of the edges of the product path: parts of short prefixes, rows that only pad a block, NaN
 and infinite keys, crowded boundary bins, the status word of a packed batch."""
+import os
+import re
+
 import numpy as np
 import pytest
 import torch
@@ -346,12 +349,14 @@ def test_decode_crowded_boundary_bin(pv, B, n_tied):
 @pytest.mark.parametrize("L,K,slope", [
     (513, 1, 2.0 ** -10), (1409, 1024, 2.0 ** -10), (1537, 100, 2.0 ** -10), (2100, 777, -2.0 ** -16),
     (12000, 512, 2.0 ** -12), (12000, 1024, 2.0 ** -8), (16500, 1300, 2.0 ** -13), (9999, 64, -2.0 ** -18),
+    (20000, 700, -2.0 ** -16), (20001, 900, 2.0 ** -10), (24000, 64, 2.0 ** -13),
 ])
 def test_scores_that_rise_or_fall_along_the_prefix(pv, L, K, slope, impl):
     """One key under scales that rise (every key beats all before it: no threshold drops anything, segments of 8192
     entries fill up and are thinned, by the threshold or, where the scores outgrow the histogram, to the K best) or fall
     with its position (nothing is appended after the first K).  Row t selects its last or its first K keys; on
-    either side of the first thresholds (5/4 K keys, four tiles) and of a block's last refresh."""
+    either side of the first thresholds (5/4 K keys, four tiles), of a block's last refresh, and of the mean prefix up to
+    which each row has a finisher warp of its own (6144 keys: dense requests of 12288)."""
     x = inputs.make_prefill(L, dtype="fp8", seed=3)
     raw = x.k.clone().view(torch.uint8)
     raw[:] = raw[5].clone()
@@ -368,25 +373,36 @@ def test_scores_that_rise_or_fall_along_the_prefix(pv, L, K, slope, impl):
     assert torch.equal(out.sort(dim=1).values, want)
 
 
+@pytest.mark.parametrize("scored", [False, True])
 @pytest.mark.parametrize("mode", ["dense", 0, 1])
-def test_rows_select_the_same_whatever_the_finishers(pv, mode):
-    """Requests on either side of the mean prefix (6144 keys) up to which each row has a finisher warp of its own: the
-    rows that both have select the same keys."""
-    L, g, c, k = 15000, 4, 1024, 500
+def test_rows_select_the_same_whatever_the_finishers(pv, mode, scored):
+    """Requests on either side of the mean prefix up to which each row has a finisher warp of its own: the rows that both
+    have select the same keys, with the same scores."""
+    sizes, g, c, k = (9001, 24000), 4, 1024, 500
+    header = open(os.path.join(os.path.dirname(pv.__file__), "csrc", "kernels.h")).read()
+    bound = int(re.search(r"kShortBlockKeys = (\d+);", header).group(1))
+    L = sizes[-1]
     x = inputs.make_prefill(L, dtype="fp8", seed=27)
     q, w, kk, kw = _operands(x)
     outs = []
-    for n in (11001, L):
+    for n in sizes:
+        rows = list(range(n)) if mode == "dense" else list(range(c)) + list(range(c, n, g))
+        mean = sum(t + 1 for t in rows) / len(rows)
+        assert mean < bound * 3 / 4 if n == sizes[0] else mean > bound * 4 / 3
         out = torch.full((n, k), -7, dtype=torch.int32, device="cuda")
-        part = dict(q_scale=kw["q_scale"][:n], k_scale=kw["k_scale"][:n])
+        sc = torch.full((n, k), float("nan"), device="cuda") if scored else None
+        part = dict(q_scale=kw["q_scale"][:n], k_scale=kw["k_scale"][:n], dbg_scores=sc)
         if mode == "dense":
             pv.dense_index(q[:n], w[:n], kk[:n], n, 64, 128, k, out, **part)
         else:
             pv.pivot_index_prefill(q[:n], w[:n], kk[:n], n, 64, 128, g, c, k, mode, out, **part)
         torch.cuda.synchronize()
         assert pv.pivot_device_status() == 0
-        outs.append(_sorted(out[:11000]))
-    assert np.array_equal(*outs)
+        # (the last group of the shorter request has one member: its proxy is another)
+        ids, at = out[:sizes[0] - 1].sort(dim=1)
+        outs.append((ids, sc[:sizes[0] - 1].gather(1, at) if scored else None))
+    assert torch.equal(outs[0][0], outs[1][0])
+    assert not scored or torch.equal(outs[0][1], outs[1][1])
 
 
 @pytest.mark.parametrize("dtype,impl", [("bf16", 0), ("fp8", 2)])
