@@ -217,17 +217,19 @@ int resolve_ws(const pivot_opts* o, size_t need, void** ws) {
 //     before a threshold has formed;
 //   - where a part's survivors fill its candidate segment, the sweep that thins it out, 64 entries in a tile's time.
 //     A part of n keys admits K (1 + ln(n / K)) of them, a ninth more for the refresh intervals and the thresholds'
-//     bins, so this takes more than half a million keys.  (While a part refreshed its thresholds every 32 tiles only
-//     and kept room for as many, budgets of 1.2 K to 3 K paid the sweep at 64K or 128K keys already.)  Segments of
-//     the least size (budgets up to 1024) are thinned late and the sweep is short: not charged;
+//     bins: a segment of 8 K entries fills up at 257 thousand keys for K = 1025, 418 for 1536, 648 for 2048, 1.6 million
+//     for 4096.  (While a part refreshed its thresholds every 32 tiles only and kept room for as many, budgets of 1.2 K
+//     to 3 K paid the sweep at 64K or 128K keys already.)  Segments of the least size (budgets up to 1024) are thinned
+//     late and the sweep is short: not charged;
 //   - the merge of the parts' selections, 2 SMs' worth of rows at a time (14 us a round of 2 x 4096 entries; lists
 //     of more than 8192 entries have an SM to themselves, but charging them for that chooses worse: 3072 rows at
-//     the end of 128K would take 1.54 ms in two parts, 1.50 in three).
-// fp8, c = 4096: 8192 rows at the end of 256K 5.9 ms in one part, 5.3 + 0.1 in two; 1024 rows at the end of 128K
-// 981 -> 610 us; 6000 rows at the end of 64K stay whole (1.64 ms; in three parts 2.07).  Over 464 chunks (512 ..
-// 12000 rows at the end of 16K .. 256K, both types, K 512 .. 4096) the choice is within 7 % of the best number of
-// parts, 0.3 % off it in the mean, and at most 4 % behind whole blocks; a bf16 tile takes 1.3 times as long
-// as an fp8 one, but a term for that changes no choice for the better.
+//     the end of 128K would take 1.22 ms in two parts, 1.18 in three).
+// Scan and merge, fp8, K = 4096: 8192 rows at the end of 256K 6.08 ms in one part, 5.56 in two; 1024 rows at the end of
+// 128K 753 -> 478 us; 6000 rows at the end of 64K stay whole (1.13 ms; in two parts 1.28).  Over 694 chunks (512 .. 12000
+// rows at the end of 16K .. 256K, both types, K 512 .. 4096) the choice is 0.5 % behind the best number of parts in the
+// mean, within 7 % in 99 of 100, at most 14 % (1536 rows at the end of 16K: 124 us whole, 109 in three parts) and at
+// most 4 % behind whole blocks.  (The charge for thinning as it was for a refresh every 32 tiles: 1.4 % in the mean, 24 % at
+// most.)  A bf16 tile takes 1.3 times as long as an fp8 one, but a term for that changes no choice for the better.
 // Calls whose blocks differ in length (a whole request) are balanced by the deal.
 // first_vis, last_vis: keys that the first and the last scan row see; cap: entries of a row's candidate segment.  Every
 // part of every block has a key tile of its own (first_vis / 128 of them at least): a part without one would not be

@@ -133,10 +133,10 @@ struct DecodePlan {
 constexpr int kThresholdRefreshTiles = PIVOT_CHK;   // the scan's append warps re-read their rows' thresholds off the histograms this often
 // ... sooner while a threshold still moves fast: first when a row has seen 5/4 K keys, then after half as many tiles as it has
 // seen, kRefreshMin at least; not with kRefreshLast or fewer tiles left of its block (a refresh takes some two tiles' time:
-// without this 12 packed requests took 488 us instead of 473); and as soon as the segment's room asks for it, which is thinned
-// out only when that is less than kLeastRoomTiles.  Against a refresh every 32 tiles, with room kept for as many, us:
-// 16K tokens, K = 512 482 -> 427; dense 5001 tokens, K = 512 202 -> 184; dense 32001, K = 1024 6060 -> 5330.  After a quarter
-// as many tiles instead of half: 432, 190, 5390.
+// without this 12 packed requests took 3 % longer); and as soon as the segment's room asks for it, which is thinned
+// out only when that is less than kLeastRoomTiles.  Against a refresh every 32 tiles, with room kept for as many (and the boundary
+// read of that time), us, medians of calls timed in turn: 16K tokens, K = 512 480 -> 425 (runs of one side within 2 %); dense 5001
+// tokens, K = 512 193.6 -> 175.7 (0.2 %); dense 32001, K = 1024 5816 -> 5228 (3.5 %).  After a quarter as many tiles instead of half: 1 .. 3 % slower.
 constexpr int kRefreshMin = 4, kRefreshLast = 12, kLeastRoomTiles = 8;
 
 struct ScanScratch {

@@ -19,7 +19,8 @@
 // barriers.  Splitting the epilogue this way puts more warps on every scheduler within the
 // register file (the score warps carry no select state) and takes the histogram atomics, the
 // global stores and the threshold refresh off the warps that feed the tensor core.  At the end
-// of a block the append warp hands its row's segment to a FINISHER warp (one per two rows), which
+// of a block the append warp hands its row's segment to a FINISHER warp (one per two rows, one per row
+// in FP8 launches of short blocks), which
 // takes the final exact select while the other warps are already scanning the next block (a row
 // has two segments, used by alternate blocks).  Row blocks are dealt to CTAs longest-first in
 // snake order.

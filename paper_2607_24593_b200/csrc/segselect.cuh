@@ -502,10 +502,10 @@ __device__ __forceinline__ int warp_emit_keys(SegSelSmem& sm, const Src& src, ui
 }
 
 // A scan row's segment on its way through shared memory, for the one sweep its finisher makes: four chunks of 256 entries in
-// flight (the first before the finisher has read its row's descriptor), each lane reading pairs.  A finisher (one warp for two
-// rows) is what short blocks wait for, and loads straight into registers left an L2 round trip per twelve entries of a
-// lane exposed: 230 -> 186 clocks per 32 entries, 5003 tokens 168 -> 163 us, dense 16K 1511 -> 1488, dense 5001 tokens
-// 184 -> 181, 8K tokens 415 -> 401.
+// flight (the first before the finisher has read its row's descriptor), each lane reading pairs.  The finishers (a warp for two
+// rows, or for one in launches of short blocks) are what short blocks wait for, and loads straight into registers left an
+// L2 round trip per twelve entries of a lane exposed: 230 -> 186 clocks per 32 entries.  us, medians of calls timed in turn: 5003
+// tokens 164.3 -> 159.3, dense 5001 tokens 175.7 -> 171.8 (runs of one side within 0.2 %), 8K 420 -> 402 (1 %), 30001 tokens 2717 -> 2610 (2 %).
 struct StagedSeg {
   static constexpr int kChunk = 256;                               // entries: eight per lane
   static constexpr int kSlots = kSelBins * 4 / (kChunk * 8);       // the histogram's 8 KB, which only ties need
@@ -533,8 +533,8 @@ struct StagedSeg {
 };
 
 // The sweep of warp_emit_keys over a started StagedSeg.  The boundary's entries take their places in the list from a counter: in
-// short rows every chunk has one, and the prefix sum over the lanes that this replaced cost as much as half the chunk (12
-// packed requests 464 -> 453 us, dense 16K 1523 -> 1490, dense 5001 tokens 181 -> 175).
+// short rows every chunk has one, and the prefix sum over the lanes that this replaced cost as much as half the chunk (medians of
+// calls timed in turn: 12 packed requests 457.5 -> 446.1 us, dense 5001 tokens 171.8 -> 166.8, runs of one side within 0.3 %).
 template <bool SCORES>
 __device__ __forceinline__ int warp_emit_staged(SegSelSmem& sm, const StagedSeg& src, uint32_t khi, uint32_t n_keys,
                                                 uint32_t* n_list, int32_t* __restrict__ out, float* __restrict__ out_score, int K,
