@@ -174,7 +174,14 @@ struct ScanOperands {
 // rows_per_block consecutive scan rows share one key stream (4 in prefill, 1 in decode).
 // fp32_head_sum: keep the gate-weighted head sum in fp32 FMAs even where the tensor-core form
 // (FP8, four rows per block) is available.  mean_keys: keys that a scan row sees on average; up to
-// kShortBlockKeys (48 tiles: four finisher warps win up to 61 tiles a block and lose from 72 on) every row has a finisher of its own.
+// kShortBlockKeys (48 tiles) every row has a finisher of its own.  us, two -> four finisher warps, medians of calls timed in turn (runs
+// of one side within 0.3 % below 20 tiles, 2 % below 35, 3 .. 5 % above), by the mean: 12 tiles, 12 packed requests 431 -> 407, dense
+// K = 256 73.1 -> 66.4, K = 1024 72.6 -> 64.6; 20 tiles, 5003 tokens 157 -> 149, 7K 316 -> 299, dense K = 512 159.8 -> 156.5; 23 tiles,
+// 8K 394 -> 378, dense K = 256 and 1024 no change, K = 2048 220 -> 209; 31 .. 43 tiles, requests with dense rows and proxies 12K
+// c = 4096 722 -> 699, c = 1024 423 -> 409, c = 8192 850 -> 849, 16K 1095 -> 1075; but dense requests, whose blocks are all
+// alike, 35 tiles 444 -> 458 (K = 256), 470 -> 480 (1024), 462 -> 468 (2048), 420 -> 421 (4096), 47 tiles 2 .. 5 % slower for
+// the same four budgets; 55 tiles and more, 16K K = 512 412 -> 416, dense 2 .. 5 % slower for every budget.  (When the bound was chosen the dense
+// requests of 35 .. 47 tiles gained 0 .. 6 % from it, more for larger budgets: two finishers have become faster since.)
 constexpr long long kShortBlockKeys = 6144;
 cudaError_t launch_scan_tc(const ScanOperands& op, const RowDesc* rows, int n_rows, int rows_per_block,
                            const ScanScratch& s, int sms, cudaStream_t st, bool fp32_head_sum = false,

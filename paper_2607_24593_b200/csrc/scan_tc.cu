@@ -71,9 +71,9 @@ struct Cfg {
   static constexpr int TEAMS = EPI_WARPS / 4;
   static constexpr int SEL_WARPS = NROWS;                     // append warps, one per row
   // Finisher warps: one per two rows, or one per row (EPI 2) where short blocks wait for them.  The two more leave every
-  // thread 96 instead of 128 registers (a few spills around the roles' loops), which long blocks pay for.  us, two -> four: packed
-  // batch (12 tiles a block) 465 -> 420, 5003 tokens (17) 163.6 -> 153, dense 5001 (22) 175 -> 165, 8K (32) 400 -> 372, 16K
-  // K = 512 (61) 457 -> 453; dense 16K (72) 1522 -> 1531, dense 32K (130) 5271 -> 5540, 64K (243) 5738 -> 5990.
+  // thread 96 instead of 128 registers (a few spills around the roles' loops), which long blocks pay for: 64K Reuse 5802 -> 6046 us
+  // (medians of calls timed in turn, runs of one side within 1 %), dense 32001 tokens 5272 -> 5528 (2 %).
+  // The rule that chooses, with both sides measured: kShortBlockKeys.
   static constexpr int FIN_WARPS = FP8 && NROWS == 4 && EPI == 2 ? 4 : NROWS == 4 ? 2 : 1;
   static constexpr int THREADS = 64 + (EPI_WARPS + SEL_WARPS + FIN_WARPS) * 32;
   static constexpr int TMEM_COLS = 2 * N < 32 ? 32 : 2 * N;
